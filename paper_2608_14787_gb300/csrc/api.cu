@@ -747,15 +747,13 @@ sdd_status_t sdd_permutation_diagnostic(const float *q, const int32_t *L, int B,
         cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(int64_t) * (n_rep + 1), reinterpret_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? SDD_OK : cuda_fail(e, "memset");
     }
-    unsigned char *base = static_cast<unsigned char *>(workspace);
-    float *pq = reinterpret_cast<float *>(base);   // the permuted scores, [n_rep][gamma][B]
-    unsigned long long *acc = reinterpret_cast<unsigned long long *>(
-        base + align256(static_cast<size_t>(n_rep) * gamma * B * sizeof(float)));
-    const cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
-    cudaError_t e = launch_perm_diag(q, L, B, gamma, signal, eta_loc, log_eta_c, n_rep, seed, pq, acc, st);
-    if (e != cudaSuccess) return cuda_fail(e, "permutation diagnostic launch");
-    e = cudaMemcpyAsync(sums, acc, sizeof(int64_t) * (n_rep + 1), cudaMemcpyDeviceToDevice, st);
-    return e == cudaSuccess ? SDD_OK : cuda_fail(e, "copy");
+    // the workspace holds the permutations ([n_rep][gamma][B] 16-bit indices:
+    // half of it)
+    const cudaError_t e = launch_perm_diag(q, L, B, gamma, signal, eta_loc, log_eta_c, n_rep, seed,
+                                           static_cast<uint16_t *>(workspace),
+                                           reinterpret_cast<unsigned long long *>(sums),
+                                           reinterpret_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? SDD_OK : cuda_fail(e, "permutation diagnostic launch");
 }
 
 sdd_status_t sdd_position_metrics(const float *q, const int32_t *L, int B, int gamma, int conditional, double *bce,

@@ -14,53 +14,60 @@
 // perm_build_kernel  -- one CTA per (repetition, position): Fisher-Yates over
 //                       the valid blocks in shared memory (order-preserving
 //                       compaction by ballots; Philox partners drawn in
-//                       parallel, the swaps in order by one thread; 64
-//                       threads, so that 32 CTAs interleave on an SM); it
-//                       writes the permuted scores of its position.
-// perm_prefix_kernel -- one warp per (repetition, block): the gates of Eq. 3 on
-//                       the permuted scores (the schedule's own arithmetic),
+//                       parallel; the swaps resolved in parallel up to
+//                       kPermPar blocks, in order by one thread above); it
+//                       writes, for every block, the block whose score it takes.
+// perm_prefix_kernel -- one thread per (repetition, block): the gates of Eq. 3
+//                       on the permuted scores (the schedule's own arithmetic),
+//                       position by position until the local gate fails;
 //                       integer sums per repetition (exact, order-free).
-// metrics_kernel     -- one CTA per position: fp64 BCE sums, integer pair counts.
+// metrics_kernel     -- one cluster of CTAs per position: fp64 BCE sums, integer
+//                       pair counts.
 #include "rules.cuh"
 
 namespace sdd {
 namespace {
 
 constexpr uint32_t kPurposePerm = 3;
-constexpr int kDiagThreads = 256;
-// The permutation builder's CTAs are small so that 32 of them share an SM:
-// each spends most of its time in one thread's serial swap loop, and the SM
-// interleaves those loops.
-constexpr int kPermThreads = 64;
+// The permutation builder's threads: every phase below is a pass over the n
+// valid blocks between two barriers, so with 256 threads a 2,048-block log
+// takes 8 elements a thread and phase, and seven CTAs (28 KiB each) share an
+// SM.  Bound by issue (72 % of the slots; ~300 warp instructions per 32
+// elements, of which the ten Philox rounds are about 80).  GB300, 2,048 blocks
+// x 32 positions x 100 repetitions: 75 us; with 64 threads a CTA, buckets by a
+// counting sort, ceil(log2 n) pointer-jumping passes and the scores gathered
+// here 265 us.
+constexpr int kPermThreads = 256;
 
 // Logs of at most this many blocks are shuffled by the parallel construction
 // below; longer ones by the serial swap loop.
 constexpr int kPermPar = 4096;
 
-// Shared memory of the permutation builder for B logged blocks: the block
-// list [B], the validity bits of position j [ceil(B/32) words] and their
-// exclusive prefix popcounts [ceil(B/32)]; for B <= kPermPar the parallel
-// construction's arrays: one [B] of 32-bit bucket bounds and four [B] of
-// 16-bit indices (small, so that ~23 CTAs share an SM).
+// Shared memory of the permutation builder for B logged blocks: the validity
+// bits of position j [ceil(B/32) words] and their exclusive prefix popcounts
+// [ceil(B/32)]; for B <= kPermPar the parallel construction's arrays (one [B]
+// of 32-bit list heads, five [B] of 16-bit indices), above it the block list
+// [B] (32-bit).
 __host__ __device__ inline size_t perm_smem_bytes(int B) {
     const size_t words = (static_cast<size_t>(B) + 31) / 32;
-    const size_t par = (B <= kPermPar) ? static_cast<size_t>(B) * (sizeof(int32_t) + 4 * sizeof(int16_t)) : 0;
-    return (static_cast<size_t>(B) + 2 * words) * sizeof(int32_t) + par;
+    const size_t per = (B <= kPermPar) ? sizeof(int32_t) + 5 * sizeof(int16_t) : sizeof(int32_t);
+    return 2 * words * sizeof(int32_t) + static_cast<size_t>(B) * per;
 }
 
-__global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const float *q, const int32_t *L, int B, int gamma,
-                                                                  int n_rep, int conditional, uint64_t seed,
-                                                                  float *pq) {
+// pi: [n_rep][gamma][B] 16-bit block indices (B <= 50,000): block b of
+// position j takes the score of block pi[r][j][b] in repetition r.
+__global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const int32_t *L, int B, int gamma, int conditional,
+                                                                  uint64_t seed, uint16_t *pi) {
     extern __shared__ int32_t s_dyn[];
-    int32_t *s_list = s_dyn;                                               // the valid blocks, then their shuffle
-    uint32_t *s_mask = reinterpret_cast<uint32_t *>(s_dyn + B);            // validity bits
-    int32_t *s_wpre = s_dyn + B + (B + 31) / 32;                           // valid blocks before each word
+    const int words = (B + 31) / 32;
+    uint32_t *s_mask = reinterpret_cast<uint32_t *>(s_dyn);                // validity bits
+    int32_t *s_wpre = s_dyn + words;                                       // valid blocks before each word
+    int32_t *s_rest = s_wpre + words;
     __shared__ __align__(16) int32_t s_k[kPermThreads];   // swap partners of the current batch of slots
     __shared__ int s_n;
     const int r = blockIdx.x / gamma, j = blockIdx.x % gamma;
     const int tid = threadIdx.x, lane = tid & 31;
-    const int words = (B + 31) / 32;
-    float *row = pq + (static_cast<int64_t>(r) * gamma + j) * B;
+    uint16_t *row = pi + (static_cast<int64_t>(r) * gamma + j) * B;
     // validity bits (the loads of several chunks in flight together)
 #pragma unroll 4
     for (int c = 0; c < B; c += kPermThreads) {
@@ -89,240 +96,365 @@ __global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const float *q
     }
     __syncthreads();
     const int n = s_n;
-    // the valid blocks in index order (the order defines the draw)
-    for (int b = tid; b < B; b += kPermThreads) {
+    // the valid blocks in index order (the order defines the draw): block b is
+    // the (s_wpre + popcount)-th of them
+    auto rank_of = [&](int b, bool &valid) {
         const uint32_t m = s_mask[b >> 5], bit = 1u << (b & 31);
-        if (m & bit) s_list[s_wpre[b >> 5] + __popc(m & (bit - 1u))] = b;
-    }
-    __syncthreads();
+        valid = (m & bit) != 0;
+        return s_wpre[b >> 5] + __popc(m & (bit - 1u));
+    };
     // Fisher-Yates from the top: slot i swaps with k_i = floor(w (i + 1) / 2^32),
     // w the first Philox word of counter (i, j, r, purpose), for i = n-1 .. 1.
     const uint2 key = make_uint2(static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32));
-    if (n > 1 && B <= kPermPar) {   // (the shared-memory layout follows B, not n)
+    auto partner = [&](int i) {
+        const uint4 o = philox4x32_10(make_uint4(static_cast<uint32_t>(i), static_cast<uint32_t>(j),
+                                                 static_cast<uint32_t>(r), kPurposePerm),
+                                      key);
+        return static_cast<int32_t>((static_cast<uint64_t>(o.x) * static_cast<uint64_t>(i + 1)) >> 32);
+    };
+    if (B <= kPermPar) {
         // The same permutation without the serial loop.  Step a moves the
         // value then at slot a to slot k_a and fixes slot a.  Let P(s) be the
         // value at slot s just before step s (slot 0: at the end); the last
         // step before a that wrote slot s is the smallest a' > a with
         // k_a' = s, and it wrote P(a').  So, with bucket(s) = {a : k_a = s}:
-        //   P(s) = P(min{a' in bucket(s), a' > s}), or the original s_list[s];
-        //   final[a] = P(min{a' in bucket(k_a), a' > a}), or s_list[k_a];
+        //   P(s) = P(min{a' in bucket(s), a' > s}), or the s-th valid block;
+        //   final[a] = P(min{a' in bucket(k_a), a' > a}), or the k_a-th;
         //   final[0] = P(0).
-        // P follows the "first step above" chains to their ends (pointer
-        // jumping); buckets come from a counting sort, each sorted by index.
-        int32_t *s_cnt = s_wpre + words;                          // bucket sizes, starts, then ends
-        int16_t *s_kk = reinterpret_cast<int16_t *>(s_cnt + B);   // k_a
-        int16_t *s_bkt = s_kk + B;                                // steps by bucket; later the final list
-        int16_t *s_nxt = s_bkt + B;                               // next step of the bucket above a (-1: none)
-        int16_t *s_ptr = s_nxt + B;                               // chain links, then chain ends
-        __shared__ int32_t s_part[kPermThreads];
-        for (int t = tid; t < n; t += kPermThreads) s_cnt[t] = 0;
+        // Each bucket is a linked list in any order (one atomic exchange per
+        // step); both minima are taken by walking a bucket, whose length is
+        // about ln(n / s), and P follows the "first step above" chains to
+        // their ends by pointer jumping, until no pointer moves (the chains
+        // are about as short as the buckets).
+        int32_t *s_head = s_rest;                                  // a bucket's first step (0: none; steps are >= 1)
+        int16_t *s_list = reinterpret_cast<int16_t *>(s_head + B); // the valid blocks
+        int16_t *s_kk = s_list + B;                                // k_a
+        int16_t *s_link = s_kk + B;                                // the bucket's next step (0: none)
+        int16_t *s_nxt = s_link + B;                               // the bucket's first step above a (0: none)
+        int16_t *s_ptr = s_nxt + B;                                // chain links, then chain ends
+        for (int b = tid; b < B; b += kPermThreads) {
+            s_head[b] = 0;
+            bool valid;
+            const int t = rank_of(b, valid);
+            if (valid) s_list[t] = static_cast<int16_t>(b);
+        }
         __syncthreads();
         for (int a = 1 + tid; a < n; a += kPermThreads) {
-            const uint4 o = philox4x32_10(make_uint4(static_cast<uint32_t>(a), static_cast<uint32_t>(j),
-                                                     static_cast<uint32_t>(r), kPurposePerm),
-                                          key);
-            const int k = static_cast<int>((static_cast<uint64_t>(o.x) * static_cast<uint64_t>(a + 1)) >> 32);
+            const int k = partner(a);
             s_kk[a] = static_cast<int16_t>(k);
-            atomicAdd(&s_cnt[k], 1);
+            s_link[a] = static_cast<int16_t>(atomicExch(&s_head[k], a));
         }
         __syncthreads();
-        // bucket starts: exclusive prefix of the sizes (chunks per thread)
-        const int chunk = (n + kPermThreads - 1) / kPermThreads;
-        const int c0 = min(n, tid * chunk), c1 = min(n, c0 + chunk);
-        int sum = 0;
-        for (int t = c0; t < c1; ++t) sum += s_cnt[t];
-        s_part[tid] = sum;
+        for (int t = tid; t < n; t += kPermThreads) {
+            int above = n;   // slot t's chain: it ends at t when no step above t targets t
+            for (int u = s_head[t]; u != 0; u = s_link[u])
+                if (u > t && u < above) above = u;
+            s_ptr[t] = static_cast<int16_t>(above < n ? above : t);
+            if (t > 0) {
+                int nx = n;
+                for (int u = s_head[s_kk[t]]; u != 0; u = s_link[u])
+                    if (u > t && u < nx) nx = u;
+                s_nxt[t] = static_cast<int16_t>(nx < n ? nx : 0);
+            }
+        }
+        __syncthreads();
+        // (in place: a pointer read during a pass is an earlier or later link
+        // of the same chain, so it never passes the chain's end)
+        for (int more = n > 1; more;) {
+            bool moved = false;
+            for (int t = tid; t < n; t += kPermThreads) {
+                const int p = s_ptr[t], pp = s_ptr[p];
+                if (pp != p) {
+                    s_ptr[t] = static_cast<int16_t>(pp);
+                    moved = true;
+                }
+            }
+            more = __syncthreads_or(moved);
+        }
+        for (int b = tid; b < B; b += kPermThreads) {
+            bool valid;
+            const int a = rank_of(b, valid);
+            int src = b;
+            if (valid) {
+                const int na = (a > 0) ? s_nxt[a] : 0;
+                src = s_list[(a == 0) ? s_ptr[0] : (na > 0) ? s_ptr[na] : s_kk[a]];
+            }
+            row[b] = static_cast<uint16_t>(src);
+        }
+        return;
+    }
+    // serial: the partners of kPermThreads slots drawn in parallel, the swaps
+    // then in order
+    int32_t *s_list = s_rest;
+    for (int b = tid; b < B; b += kPermThreads) {
+        bool valid;
+        const int t = rank_of(b, valid);
+        if (valid) s_list[t] = b;
+    }
+    __syncthreads();
+    for (int top = n - 1; top > 0; top -= kPermThreads) {
+        const int i = top - tid;
+        if (i > 0) s_k[tid] = partner(i);
         __syncthreads();
         if (tid == 0) {
-            int run = 0;
-            for (int t = 0; t < kPermThreads; ++t) {
-                const int v = s_part[t];
-                s_part[t] = run;
-                run += v;
-            }
-        }
-        __syncthreads();
-        int run = s_part[tid];
-        for (int t = c0; t < c1; ++t) {
-            const int v = s_cnt[t];
-            s_cnt[t] = run;
-            run += v;
-        }
-        __syncthreads();
-        // scatter (the starts advance to the ends: bucket t is [end(t-1), end(t)))
-        for (int a = 1 + tid; a < n; a += kPermThreads)
-            s_bkt[atomicAdd(&s_cnt[s_kk[a]], 1)] = static_cast<int16_t>(a);
-        __syncthreads();
-        // per slot: its bucket sorted, successors, the first step above the slot
-        for (int t = tid; t < n; t += kPermThreads) {
-            const int b0 = (t > 0) ? s_cnt[t - 1] : 0, b1 = s_cnt[t];
-            for (int u = b0 + 1; u < b1; ++u) {   // insertion sort (buckets hold ~1 step)
-                const int v = s_bkt[u];
-                int w = u - 1;
-                while (w >= b0 && s_bkt[w] > v) {
-                    s_bkt[w + 1] = s_bkt[w];
-                    --w;
-                }
-                s_bkt[w + 1] = static_cast<int16_t>(v);
-            }
-            int above = t;   // the chain ends here when no step above t targets t
-            for (int u = b0; u < b1; ++u) {
-                const int v = s_bkt[u];
-                s_nxt[v] = (u + 1 < b1) ? s_bkt[u + 1] : static_cast<int16_t>(-1);
-                if (above == t && v > t) above = v;
-            }
-            s_ptr[t] = static_cast<int16_t>(above);
-        }
-        __syncthreads();
-        for (int span = 1; span < n; span <<= 1) {   // pointer jumping to the chain ends
-            for (int t = tid; t < n; t += kPermThreads) s_ptr[t] = s_ptr[s_ptr[t]];
-            __syncthreads();
-        }
-        for (int a = tid; a < n; a += kPermThreads) {
-            int v;
-            if (a == 0) {
-                v = s_list[s_ptr[0]];
-            } else {
-                const int na = s_nxt[a];
-                v = (na >= 0) ? s_list[s_ptr[na]] : s_list[s_kk[a]];
-            }
-            s_bkt[a] = static_cast<int16_t>(v);
-        }
-        __syncthreads();
-        for (int a = tid; a < n; a += kPermThreads) s_list[a] = s_bkt[a];
-        __syncthreads();
-    } else {
-        // serial: the partners of kPermThreads slots drawn in parallel, the swaps
-        // then in order
-        for (int top = n - 1; top > 0; top -= kPermThreads) {
-            const int i = top - tid;
-            if (i > 0) {
-                const uint4 o = philox4x32_10(make_uint4(static_cast<uint32_t>(i), static_cast<uint32_t>(j),
-                                                         static_cast<uint32_t>(r), kPurposePerm),
-                                              key);
-                s_k[tid] = static_cast<int32_t>((static_cast<uint64_t>(o.x) * static_cast<uint64_t>(i + 1)) >> 32);
-            }
-            __syncthreads();
-            if (tid == 0) {
-                // slots top, top - 1, ..., top - cnt + 1 (all > 0); x carries the
-                // value at slot a, re-read after each swap (which may have written
-                // slot a - 1), so one shared-memory round trip bounds an iteration;
-                // the partners come four at a time
-                const int cnt = min(kPermThreads, top);
-                int32_t x = s_list[top];
-                for (int u = 0; u < cnt; u += 4) {
-                    const int4 kk = *reinterpret_cast<const int4 *>(s_k + u);
-                    const int ks[4] = {kk.x, kk.y, kk.z, kk.w};
+            // slots top, top - 1, ..., top - cnt + 1 (all > 0); x carries the
+            // value at slot a, re-read after each swap (which may have written
+            // slot a - 1), so one shared-memory round trip bounds an iteration;
+            // the partners come four at a time
+            const int cnt = min(kPermThreads, top);
+            int32_t x = s_list[top];
+            for (int u = 0; u < cnt; u += 4) {
+                const int4 kk = *reinterpret_cast<const int4 *>(s_k + u);
+                const int ks[4] = {kk.x, kk.y, kk.z, kk.w};
 #pragma unroll
-                    for (int h = 0; h < 4; ++h) {
-                        if (u + h >= cnt) break;
-                        const int a = top - u - h, k = ks[h];
-                        const int32_t y = (k == a) ? x : s_list[k];
-                        s_list[k] = x;
-                        s_list[a] = y;
-                        x = s_list[a - 1];
-                    }
+                for (int h = 0; h < 4; ++h) {
+                    if (u + h >= cnt) break;
+                    const int a = top - u - h, k = ks[h];
+                    const int32_t y = (k == a) ? x : s_list[k];
+                    s_list[k] = x;
+                    s_list[a] = y;
+                    x = s_list[a - 1];
                 }
             }
-            __syncthreads();
+        }
+        __syncthreads();
+    }
+    for (int b = tid; b < B; b += kPermThreads) {
+        bool valid;
+        const int a = rank_of(b, valid);
+        row[b] = static_cast<uint16_t>(valid ? s_list[a] : b);
+    }
+}
+
+// Grid: ceil(B / kPrefixThreads) CTAs for each of n_rep + 1 repetitions, the
+// last of which is the logged order.  Neighbouring threads are neighbouring blocks, so a repetition's
+// indices are read in whole lines, and a score is gathered only while the
+// block's local gate holds; the positions go in groups of kPrefixU whose
+// loads are in flight together.  Bound by the gathers' latency.  GB300, 2,048
+// x 32 x 100: 20 us; with a warp per (repetition, block), its lanes on scores
+// 4 B bytes apart, 112 us.
+constexpr int kPrefixThreads = 256;
+constexpr int kPrefixU = 4;
+__global__ void __launch_bounds__(kPrefixThreads) perm_prefix_kernel(const float *q, const uint16_t *pi, int B,
+                                                                     int gamma, int n_rep, int signal, df eta_loc,
+                                                                     df log_eta_c, unsigned long long *sums) {
+    const int per = (B + kPrefixThreads - 1) / kPrefixThreads;
+    const int r = blockIdx.x / per, b = static_cast<int>(blockIdx.x % per) * kPrefixThreads + threadIdx.x;
+    int Kh = 0;
+    if (b < B) {
+        const uint16_t *row = pi + static_cast<int64_t>(r) * gamma * B + b;
+        int kb = 0, best = 0;   // leading positions passing the local gate; the largest prefix meeting Eq. 3
+        bool open = true;
+        df S = df{0.f, 0.f};
+        for (int j0 = 0; j0 < gamma && open; j0 += kPrefixU) {
+            float qj[kPrefixU];
+#pragma unroll
+            for (int u = 0; u < kPrefixU; ++u) {
+                const int j = j0 + u;
+                int src = b;
+                if (r < n_rep && j < gamma) src = __ldg(row + static_cast<int64_t>(j) * B);
+                qj[u] = (j < gamma) ? __ldg(q + static_cast<int64_t>(src) * gamma + j) : qnan();
+            }
+#pragma unroll
+            for (int u = 0; u < kPrefixU; ++u) {
+                // (past gamma: NaN closes the gate)
+                open = open && isfinite(qj[u]) && df_ge(df{qj[u], 0.f}, eta_loc);
+                if (!open) continue;
+                kb = j0 + u + 1;
+                if (signal == SDD_SIG_MARGINAL) continue;
+                S = df_add(S, df{logf(qj[u]), 0.f});
+                const bool pass = (signal == SDD_SIG_RAW) ? df_ge(S, df_mul_f(log_eta_c, static_cast<float>(kb)))
+                                                          : df_ge(S, log_eta_c);
+                if (pass) best = kb;
+            }
+        }
+        Kh = (signal == SDD_SIG_MARGINAL) ? kb : best;
+    }
+    Kh = __reduce_add_sync(0xFFFFFFFFu, Kh);
+    if ((threadIdx.x & 31) == 0 && Kh > 0) atomicAdd(sums + r, static_cast<unsigned long long>(Kh));
+}
+
+// Positionwise metrics.  The pair counts of the AUROC are what costs: a
+// position of a log of B blocks has up to B^2 / 4 (positive, negative) pairs.
+// A cluster of kMetCluster CTAs takes a position; CTA c takes the blocks of
+// its c-th part of the log as the positives (and their BCE terms: fp64
+// logarithms, which issue slowly here, so they too are spread over the SMs)
+// against every negative of the log.  Positives and negatives are compacted
+// into shared memory in tiles (their order does not matter for integer
+// counts); a thread holds kMetR positives in registers against a strided run
+// of the negatives.  Sums meet in CTA 0 by distributed shared memory and are
+// added in rank order, so the results are deterministic.  Bound by the chain
+// of staging, pairs, fp64 logarithms and the cluster's sums.  GB300, 2,048 x
+// 32: 30 us (38 us with a logarithm for each class and the three results on
+// one thread); one CTA per position and one positive per thread against the
+// log in global memory took 1,326 us.
+constexpr int kMetThreads = 256;
+constexpr int kMetCluster = 8;
+constexpr int kMetR = 4;
+constexpr int kMetPos = 1024;    // positives of a tile
+constexpr int kMetNeg = 4096;    // negatives of a tile
+struct MetSums {
+    double bce;
+    unsigned long long np, nn, gt, eq;
+};
+
+__device__ __forceinline__ void st_cluster_u64(uint32_t addr, unsigned long long v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+
+// The valid blocks of [b0, b1) of the wanted class (positive: L >= j + 1),
+// their scores compacted into dst (in any order); *s_cnt receives their number.
+__device__ __forceinline__ void met_stage(const float *q, const int32_t *L, int gamma, int j, int conditional, int b0,
+                                          int b1, bool positive, float *dst, int *s_cnt) {
+    __syncthreads();   // the previous tile has been read
+    if (threadIdx.x == 0) *s_cnt = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    constexpr int U = 4;   // loads of U blocks a thread in flight together
+    for (int c = b0; c < b1; c += U * kMetThreads) {
+        int l[U];
+        float x[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int b = c + u * kMetThreads + static_cast<int>(threadIdx.x);
+            l[u] = (b < b1) ? __ldg(L + b) : 0;
+            x[u] = (b < b1) ? __ldg(q + static_cast<int64_t>(b) * gamma + j) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int b = c + u * kMetThreads + static_cast<int>(threadIdx.x);
+            const bool in = b < b1 && !(conditional && l[u] < j) && (l[u] >= j + 1) == positive;
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+            int at = 0;
+            if (lane == 0 && m) at = atomicAdd(s_cnt, __popc(m));
+            at = __shfl_sync(0xFFFFFFFFu, at, 0);
+            if (in) dst[at + __popc(m & ((1u << lane) - 1u))] = x[u];
         }
     }
-    // block b (the t-th valid block) takes the score of block s_list[t]; others
-    // keep theirs: the permuted scores of position j, gathered here so that the
-    // prefix kernel reads each with one load
-    for (int b = tid; b < B; b += kPermThreads) {
-        const uint32_t m = s_mask[b >> 5], bit = 1u << (b & 31);
-        const int src = (m & bit) ? s_list[s_wpre[b >> 5] + __popc(m & (bit - 1u))] : b;
-        row[b] = __ldg(q + static_cast<int64_t>(src) * gamma + j);
-    }
+    __syncthreads();
 }
 
-__global__ void perm_prefix_kernel(const float *q, const float *pq, int B, int gamma, int n_rep, int signal,
-                                   df eta_loc, df log_eta_c, unsigned long long *sums) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    if (w >= static_cast<int64_t>(n_rep + 1) * B) return;
-    const int r = static_cast<int>(w / B), b = static_cast<int>(w % B);   // r == n_rep: the logged order
-    int kb = gamma, best = 0;
-    df carry = df{0.f, 0.f};
-    for (int c = 0; c < gamma && kb >= c; c += 32) {
-        const int j = c + lane;
-        const bool in = j < gamma;
-        const float qj = !in ? 0.f
-                         : (r < n_rep) ? __ldg(pq + (static_cast<int64_t>(r) * gamma + j) * B + b)
-                                       : __ldg(q + static_cast<int64_t>(b) * gamma + j);
-        const float lq = in ? logf(qj) : 0.f;
-        const df S = df_add(carry, warp_prefix_df(df{lq, 0.f}, lane));
-        carry.hi = __shfl_sync(0xFFFFFFFFu, S.hi, 31);
-        carry.lo = __shfl_sync(0xFFFFFFFFu, S.lo, 31);
-        sched_step(c, lane, gamma, in, qj, false, S, eta_loc, log_eta_c, signal, kb, best);
-    }
-    const int Kh = (signal == SDD_SIG_MARGINAL) ? kb : best;
-    if (lane == 0) atomicAdd(sums + r, static_cast<unsigned long long>(Kh));
-}
-
-__global__ void __launch_bounds__(kDiagThreads) metrics_kernel(const float *q, const int32_t *L, int B, int gamma,
-                                                               int conditional, double *bce, double *bce_base,
-                                                               double *auroc, int32_t *n_pos, int32_t *n_neg) {
-    const int j = blockIdx.x;
-    __shared__ double s_bce[kDiagThreads];
-    __shared__ unsigned long long s_np[kDiagThreads], s_nn[kDiagThreads], s_gt[kDiagThreads], s_eq[kDiagThreads];
-    double sb = 0.0;
-    unsigned long long np = 0, nn = 0, gt = 0, eq = 0;
-    for (int b = threadIdx.x; b < B; b += kDiagThreads) {
+__global__ void __cluster_dims__(kMetCluster, 1, 1) __launch_bounds__(kMetThreads)
+    metrics_kernel(const float *q, const int32_t *L, int B, int gamma, int conditional, double *bce, double *bce_base,
+                   double *auroc, int32_t *n_pos, int32_t *n_neg) {
+    const int j = blockIdx.x / kMetCluster, rank = blockIdx.x % kMetCluster;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ float s_pos[kMetPos], s_neg[kMetNeg];
+    __shared__ int s_np, s_nn;
+    __shared__ MetSums s_w[kMetThreads / 32];
+    __shared__ MetSums s_all[kMetCluster];   // (CTA 0)
+    const int part = (B + kMetCluster - 1) / kMetCluster;
+    const int p0 = min(B, rank * part), p1 = min(B, p0 + part);
+    MetSums a{0.0, 0, 0, 0, 0};
+    for (int b = p0 + tid; b < p1; b += kMetThreads) {
         const int l = __ldg(L + b);
         if (conditional && l < j) continue;
         const bool y = l >= j + 1;
         const double qc = fmin(fmax(static_cast<double>(__ldg(q + static_cast<int64_t>(b) * gamma + j)), 1e-7),
                                1.0 - 1e-7);
-        sb -= y ? log(qc) : log1p(-qc);
-        if (y) {
-            ++np;
-            const float qi = __ldg(q + static_cast<int64_t>(b) * gamma + j);
-            for (int k = 0; k < B; ++k) {   // every valid negative
-                const int lk = __ldg(L + k);
-                if ((conditional && lk < j) || lk >= j + 1) continue;
-                const float qk = __ldg(q + static_cast<int64_t>(k) * gamma + j);
-                gt += qi > qk;
-                eq += qi == qk;
+        // one fp64 logarithm for both classes: 1 - qc = h + l exactly, and
+        // ln(h + l) = ln h + l / h to (l / h)^2 < 2^-104
+        const double h = 1.0 - qc, l2 = (1.0 - h) - qc;
+        const double corr = static_cast<double>(static_cast<float>(l2) / static_cast<float>(h));
+        a.bce -= log(y ? qc : h) + (y ? 0.0 : corr);
+        a.np += y ? 1 : 0;
+        a.nn += y ? 0 : 1;
+    }
+    for (int c = p0; c < p1; c += kMetPos) {
+        met_stage(q, L, gamma, j, conditional, c, min(p1, c + kMetPos), true, s_pos, &s_np);
+        const int P = s_np;
+        if (P == 0) continue;
+        // Q threads side by side over groups of kMetR positives, the others
+        // over the negatives: Q the power of two at or above the groups
+        const int groups = (P + kMetR - 1) / kMetR;
+        int Q = 1;
+        while (Q < groups && Q < kMetThreads) Q <<= 1;
+        const int g0 = tid & (Q - 1), stripe = tid / Q, stripes = kMetThreads / Q;
+        for (int n0 = 0; n0 < B; n0 += kMetNeg) {
+            met_stage(q, L, gamma, j, conditional, n0, min(B, n0 + kMetNeg), false, s_neg, &s_nn);
+            const int N = s_nn;
+            for (int g = g0; g < groups; g += Q) {
+                float p[kMetR];
+                uint32_t gt = 0, ge = 0;   // (at most kMetR kMetNeg each)
+#pragma unroll
+                for (int u = 0; u < kMetR; ++u) {
+                    // (NaN compares false: a slot past the tile counts nothing)
+                    p[u] = (g * kMetR + u < P) ? s_pos[g * kMetR + u] : qnan();
+                }
+#pragma unroll 4
+                for (int k = stripe; k < N; k += stripes) {
+                    const float v = s_neg[k];
+#pragma unroll
+                    for (int u = 0; u < kMetR; ++u) {
+                        gt += p[u] > v ? 1u : 0u;
+                        ge += p[u] >= v ? 1u : 0u;
+                    }
+                }
+                a.gt += gt;
+                a.eq += ge - gt;
             }
-        } else {
-            ++nn;
         }
     }
-    s_bce[threadIdx.x] = sb;
-    s_np[threadIdx.x] = np;
-    s_nn[threadIdx.x] = nn;
-    s_gt[threadIdx.x] = gt;
-    s_eq[threadIdx.x] = eq;
+    // fixed-order sums: lanes, warps, CTAs
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a.bce += __shfl_down_sync(0xFFFFFFFFu, a.bce, off);
+        a.np += __shfl_down_sync(0xFFFFFFFFu, a.np, off);
+        a.nn += __shfl_down_sync(0xFFFFFFFFu, a.nn, off);
+        a.gt += __shfl_down_sync(0xFFFFFFFFu, a.gt, off);
+        a.eq += __shfl_down_sync(0xFFFFFFFFu, a.eq, off);
+    }
+    if (lane == 0) s_w[warp] = a;
     __syncthreads();
-    for (int h = kDiagThreads / 2; h > 0; h >>= 1) {   // fixed-order tree: deterministic sums
-        if (threadIdx.x < h) {
-            s_bce[threadIdx.x] += s_bce[threadIdx.x + h];
-            s_np[threadIdx.x] += s_np[threadIdx.x + h];
-            s_nn[threadIdx.x] += s_nn[threadIdx.x + h];
-            s_gt[threadIdx.x] += s_gt[threadIdx.x + h];
-            s_eq[threadIdx.x] += s_eq[threadIdx.x + h];
+    if (tid == 0) {
+#pragma unroll
+        for (int w = 1; w < kMetThreads / 32; ++w) {
+            a.bce += s_w[w].bce;
+            a.np += s_w[w].np;
+            a.nn += s_w[w].nn;
+            a.gt += s_w[w].gt;
+            a.eq += s_w[w].eq;
         }
-        __syncthreads();
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(dst) : "r"(smem_addr(&s_all[rank])));
+        st_cluster_u64(dst, static_cast<unsigned long long>(__double_as_longlong(a.bce)));
+        st_cluster_u64(dst + 8, a.np);
+        st_cluster_u64(dst + 16, a.nn);
+        st_cluster_u64(dst + 24, a.gt);
+        st_cluster_u64(dst + 32, a.eq);
     }
-    if (threadIdx.x == 0) {
-        const double P = static_cast<double>(s_np[0]), N = static_cast<double>(s_nn[0]), n = P + N;
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (rank == 0 && lane == 0 && warp < 3) {
+        // (a warp for each result: their fp64 chains run side by side)
+        MetSums t = s_all[0];
+#pragma unroll
+        for (int c = 1; c < kMetCluster; ++c) {
+            t.bce += s_all[c].bce;
+            t.np += s_all[c].np;
+            t.nn += s_all[c].nn;
+            t.gt += s_all[c].gt;
+            t.eq += s_all[c].eq;
+        }
+        const double P = static_cast<double>(t.np), N = static_cast<double>(t.nn), n = P + N;
         const double nan = __longlong_as_double(0x7FF8000000000000ll);
-        bce[j] = (n > 0) ? s_bce[0] / n : nan;
-        const double pr = (n > 0) ? P / n : nan;
-        bce_base[j] = (n > 0) ? ((pr > 0.0 && pr < 1.0) ? -(pr * log(pr) + (1.0 - pr) * log1p(-pr)) : 0.0) : nan;
-        auroc[j] = (P > 0 && N > 0) ? (static_cast<double>(s_gt[0]) + 0.5 * static_cast<double>(s_eq[0])) / (P * N)
-                                    : nan;
-        if (n_pos) n_pos[j] = static_cast<int32_t>(s_np[0]);
-        if (n_neg) n_neg[j] = static_cast<int32_t>(s_nn[0]);
+        if (warp == 0) {
+            bce[j] = (n > 0) ? t.bce / n : nan;
+            if (n_pos) n_pos[j] = static_cast<int32_t>(t.np);
+            if (n_neg) n_neg[j] = static_cast<int32_t>(t.nn);
+        } else if (warp == 1) {
+            const double pr = (n > 0) ? P / n : nan;
+            bce_base[j] = (n > 0) ? ((pr > 0.0 && pr < 1.0) ? -(pr * log(pr) + (1.0 - pr) * log1p(-pr)) : 0.0) : nan;
+        } else {
+            auroc[j] =
+                (P > 0 && N > 0) ? (static_cast<double>(t.gt) + 0.5 * static_cast<double>(t.eq)) / (P * N) : nan;
+        }
     }
 }
 
 }  // namespace
 
 cudaError_t launch_perm_diag(const float *q, const int32_t *L, int B, int gamma, int signal, df eta_loc,
-                             df log_eta_c, int n_rep, uint64_t seed, float *pq, unsigned long long *sums,
+                             df log_eta_c, int n_rep, uint64_t seed, uint16_t *pi, unsigned long long *sums,
                              cudaStream_t stream) {
     cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * (n_rep + 1), stream);
     if (e != cudaSuccess) return e;
@@ -333,22 +465,22 @@ cudaError_t launch_perm_diag(const float *q, const int32_t *L, int B, int gamma,
         if (e != cudaSuccess) return e;
     }
     if (n_rep > 0) {
-        perm_build_kernel<<<n_rep * gamma, kPermThreads, smem, stream>>>(q, L, B, gamma, n_rep,
-                                                                        signal == SDD_SIG_CONDITIONAL, seed, pq);
+        perm_build_kernel<<<n_rep * gamma, kPermThreads, smem, stream>>>(L, B, gamma, signal == SDD_SIG_CONDITIONAL,
+                                                                        seed, pi);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    const int64_t warps = static_cast<int64_t>(n_rep + 1) * B;
-    perm_prefix_kernel<<<static_cast<unsigned>((warps * 32 + 255) / 256), 256, 0, stream>>>(
-        q, pq, B, gamma, n_rep, signal, eta_loc, log_eta_c, sums);
+    const int per = (B + kPrefixThreads - 1) / kPrefixThreads;
+    perm_prefix_kernel<<<static_cast<unsigned>(per) * static_cast<unsigned>(n_rep + 1), kPrefixThreads, 0, stream>>>(
+        q, pi, B, gamma, n_rep, signal, eta_loc, log_eta_c, sums);
     return cudaGetLastError();
 }
 
 cudaError_t launch_position_metrics(const float *q, const int32_t *L, int B, int gamma, int conditional, double *bce,
                                     double *bce_base, double *auroc, int32_t *n_pos, int32_t *n_neg,
                                     cudaStream_t stream) {
-    metrics_kernel<<<gamma, kDiagThreads, 0, stream>>>(q, L, B, gamma, conditional, bce, bce_base, auroc, n_pos,
-                                                       n_neg);
+    metrics_kernel<<<gamma * kMetCluster, kMetThreads, 0, stream>>>(q, L, B, gamma, conditional, bce, bce_base, auroc,
+                                                                    n_pos, n_neg);
     return cudaGetLastError();
 }
 
