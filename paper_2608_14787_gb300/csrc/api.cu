@@ -151,13 +151,47 @@ void init_scan(ScanParams &p, const Work &w, sdd_dtype_t dtype, int B, int gamma
     p.status = status;
 }
 
-// Fill in the totals of a ScanParams whose groups are set.
+// The draw geometry of nb blocks over `budget` decide teams of nt threads:
+// each draw row of RV vectors is cut into nseg segments of whole nt-vector chunks, as
+// many as keep nb * nseg teams within the budget (at least two vectors per
+// thread, at most kDrawMaxSeg segments).
+void draw_segments(int RV, int nb, int budget, int nt, int32_t &nseg, int32_t &seg_vec) {
+    const int want = std::max(1, std::min(kDrawMaxSeg, budget / std::max(nb, 1)));
+    const int per_thread = std::max(2, (RV + nt * want - 1) / (nt * want));
+    seg_vec = per_thread * nt;
+    nseg = (RV + seg_vec - 1) / seg_vec;
+}
+
+// The decide kernel's team.  After a pass of whole pieces (kWholeMin or more of
+// them to a row, so few rows) a block's CTAs are wide enough to merge a row's
+// partials by groups of threads and to hold fewer, wider draw segments.
+void set_team(ScanParams &p, const Work &w) {
+    DecideParams &d = p.dec;
+    d.team = kDecThreads;
+    if (p.rows <= 0 || p.W % p.rows != 0 || p.W / p.rows < kWholeMin) return;
+    int32_t nseg = 1, seg_vec = 0;
+    draw_segments(p.RV, p.grp[0].nb, w.sms, kDecThreadsWhole, nseg, seg_vec);
+    // (the workspace holds max(dec_ctas, B) kDecThreads prefixes)
+    if (static_cast<int64_t>(std::max(p.grp[0].nb * nseg, w.sms)) * kDecThreadsWhole >
+        static_cast<int64_t>(std::max(w.dec_ctas, p.B)) * kDecThreads)
+        return;
+    d.team = kDecThreadsWhole;
+    if (!d.enabled) return;
+    d.dec_ctas = w.sms;
+    d.nseg = nseg;
+    d.seg_vec = seg_vec;
+}
+
+// Fill in the totals of a ScanParams whose groups are set, and the decide
+// kernel's geometry (its decisions are set).
 void finish_params(ScanParams &p, const Work &w) {
     p.rows0 = static_cast<int64_t>(p.grp[0].nb) * p.grp[0].npos;
     p.rows = p.rows0 + (p.n_groups > 1 ? static_cast<int64_t>(p.grp[1].nb) * p.grp[1].npos : 0);
     p.T = p.rows * p.RV;
     p.W = scan_warps(w.W_max, p.T, p.rows);
+    p.ctas = w.W_max / kWarpsPerCta;
     set_divisors(p);
+    set_team(p, w);
 }
 
 // The streaming kernel over the rows of p.
@@ -165,8 +199,7 @@ sdd_status_t run_scan(const ScanParams &p, cudaStream_t stream) {
     if (p.T == 0) return SDD_OK;
     if (static_cast<double>(p.C) * static_cast<double>(p.W) >= 9.007199254740992e15)   // 2^53
         return fail(SDD_ERR_UNSUPPORTED, "%lld vectors of logits exceed the index arithmetic", (long long)p.T);
-    const int grid = static_cast<int>((static_cast<int64_t>(p.W) + kWarpsPerCta - 1) / kWarpsPerCta);
-    cudaError_t e = launch_scan(p, grid, stream);
+    cudaError_t e = launch_scan(p, stream);
     if (e != cudaSuccess) return cuda_fail(e, "scan launch");
     return SDD_OK;
 }
@@ -184,17 +217,6 @@ sdd_status_t run_decide_shard(const ScanParams &p, cudaStream_t stream) {
     cudaError_t e = launch_decide(p, stream);
     if (e != cudaSuccess) return cuda_fail(e, "decide launch");
     return SDD_OK;
-}
-
-// The draw geometry of nb blocks over `budget` decide teams of nt threads:
-// each draw row of RV vectors is cut into nseg segments of whole nt-vector chunks, as
-// many as keep nb * nseg teams within the budget (at least two vectors per
-// thread, at most kDrawMaxSeg segments).
-void draw_segments(int RV, int nb, int budget, int nt, int32_t &nseg, int32_t &seg_vec) {
-    const int want = std::max(1, std::min(kDrawMaxSeg, budget / std::max(nb, 1)));
-    const int per_thread = std::max(2, (RV + nt * want - 1) / (nt * want));
-    seg_vec = per_thread * nt;
-    nseg = (RV + seg_vec - 1) / seg_vec;
 }
 
 // Block decisions and, for the sampling rule, the draw geometry over the
@@ -1176,7 +1198,7 @@ sdd_status_t sdd_block_pipelined(const sdd_block_args *next, const sdd_block_arg
     }
     if (static_cast<double>(pn.C) * static_cast<double>(pn.W) >= 9.007199254740992e15)   // 2^53
         return fail(SDD_ERR_UNSUPPORTED, "%lld vectors of logits exceed the index arithmetic", (long long)pn.T);
-    const int grid = static_cast<int>((static_cast<int64_t>(pn.W) + pn.wpc - 1) / pn.wpc);
+    const int grid = std::min(pn.W, pn.ctas);
     // prev's draw segments over this grid's CTAs, one (block, segment) item each
     if (!ep) draw_segments(pp.RV, pp.grp[0].nb, grid, 32 * pn.warp0, pp.dec.nseg, pp.dec.seg_vec);
     const cudaError_t e = launch_pipe(&pn, ep ? nullptr : &pp, grid, st);

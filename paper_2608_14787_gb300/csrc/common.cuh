@@ -430,6 +430,19 @@ __device__ __forceinline__ SoftState soft_merge(const SoftState &a, const SoftSt
     return o;
 }
 
+// The state `off` lanes above (every lane of the warp calls it).
+__device__ __forceinline__ SoftState soft_shfl_down(const SoftState &v, int off) {
+    SoftState o;
+    o.m = __shfl_down_sync(0xFFFFFFFFu, v.m, off);
+    o.r = __shfl_down_sync(0xFFFFFFFFu, v.r, off);
+    o.t2 = __shfl_down_sync(0xFFFFFFFFu, v.t2, off);
+    o.sh = __shfl_down_sync(0xFFFFFFFFu, v.sh, off);
+    o.sl = __shfl_down_sync(0xFFFFFFFFu, v.sl, off);
+    o.amax = __shfl_down_sync(0xFFFFFFFFu, v.amax, off);
+    o.rank = __shfl_down_sync(0xFFFFFFFFu, v.rank, off);
+    return o;
+}
+
 __device__ __forceinline__ SoftState soft_warp_reduce(SoftState v) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {

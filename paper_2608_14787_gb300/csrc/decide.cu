@@ -14,14 +14,15 @@ namespace {
 
 // One CTA per (listed block, draw segment), behind the streaming grid that
 // wrote the partials (FEAT, SHARD: as decide_cta).  Separate instantiations,
-// so that the fused round keeps the smallest kernel.
-template <int DT, bool FEAT, bool SHARD = false>
-__global__ void __launch_bounds__(kDecThreads) decide_kernel(const __grid_constant__ ScanParams p) {
-    extern __shared__ float s_pref_all[];   // [nseg][kDecThreads]: every segment's prefixes (last CTA)
+// so that the fused round keeps the smallest kernel.  NT = kDecThreadsWhole
+// after a streaming pass of whole pieces (many of them to a row, few blocks).
+template <int DT, bool FEAT, bool SHARD = false, int NT = kDecThreads>
+__global__ void __launch_bounds__(NT) decide_kernel(const __grid_constant__ ScanParams p) {
+    extern __shared__ float s_pref_all[];   // [nseg][NT]: every segment's prefixes (last CTA)
     griddep_wait();   // launched behind the streaming grid that wrote the partials
     const PartView pv = part_view(p);
-    const DecGeom geo = dec_geom(p, pv, p.dec.enabled && p.dec.do_strict && !p.dec.greedy && !SHARD);
-    decide_cta<DT, FEAT, SHARD>(p, pv, geo, s_pref_all);
+    const DecGeom geo = dec_geom<NT>(p, pv, p.dec.enabled && p.dec.do_strict && !p.dec.greedy && !SHARD);
+    decide_cta<DT, FEAT, SHARD, NT>(p, pv, geo, s_pref_all);
 }
 
 // Vocabulary-sharded draw, one CTA per block, after every slice's masses of
@@ -228,6 +229,14 @@ __global__ void uniforms_kernel(uint64_t seed, const uint32_t *j, const uint32_t
 
 }  // namespace
 
+namespace {
+// [features][bf16]
+void (*const kDecideWhole[2][2])(ScanParams) = {{decide_kernel<SDD_F32, false, false, kDecThreadsWhole>,
+                                                 decide_kernel<SDD_BF16, false, false, kDecThreadsWhole>},
+                                                {decide_kernel<SDD_F32, true, false, kDecThreadsWhole>,
+                                                 decide_kernel<SDD_BF16, true, false, kDecThreadsWhole>}};
+}  // namespace
+
 int decide_max_ctas_per_sm() {
     int n = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, decide_kernel<SDD_BF16, false>, kDecThreads, 0);
@@ -244,6 +253,12 @@ cudaError_t decide_prepare_device() {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
     }
+    constexpr int bytes_whole = kDrawMaxSeg * kDecThreadsWhole * static_cast<int>(sizeof(float));
+    for (const auto &row : kDecideWhole)
+        for (auto k : row) {
+            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes_whole);
+            if (e != cudaSuccess) return e;
+        }
     void (*const draws[])(ShardParams) = {shard_draw_kernel<SDD_BF16>, shard_draw_kernel<SDD_F32>};
     for (auto k : draws) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -259,13 +274,15 @@ cudaError_t launch_decide(const ScanParams &p, cudaStream_t stream) {
     // a device block count: a one-dimensional grid cut on the device (dec_geom)
     const bool dev_geom = draw && p.nb_dev != nullptr && p.shard == nullptr;
     const int nseg = draw ? (dev_geom ? std::min(kDrawMaxSeg, std::max(p.dec.dec_ctas, 1)) : p.dec.nseg) : 1;
-    const size_t smem = draw ? static_cast<size_t>(nseg) * kDecThreads * sizeof(float) : 0;
+    const int team = (p.dec.team == kDecThreadsWhole) ? kDecThreadsWhole : kDecThreads;
+    const size_t smem = draw ? static_cast<size_t>(nseg) * team * sizeof(float) : 0;
     const dim3 grid = dev_geom ? dim3(static_cast<unsigned>(std::max(p.dec.dec_ctas, nb))) : dim3(nb, nseg);
     const bool bf = p.dtype == SDD_BF16, feat = p.feat != nullptr;
     void (*const k)(ScanParams) = (p.shard != nullptr)
                                       ? (bf ? decide_kernel<SDD_BF16, false, true> : decide_kernel<SDD_F32, false, true>)
                                   : feat ? (bf ? decide_kernel<SDD_BF16, true> : decide_kernel<SDD_F32, true>)
                                          : (bf ? decide_kernel<SDD_BF16, false> : decide_kernel<SDD_F32, false>);
+    if (team == kDecThreadsWhole) return launch_dependent(kDecideWhole[feat][bf], grid, dim3(team), smem, stream, p);
     return launch_dependent(k, grid, dim3(kDecThreads), smem, stream, p);
 }
 

@@ -515,6 +515,7 @@ __device__ int segment_find(const DrawCtx &c, const float *s_pref_all, int sel, 
 struct DecGeom {
     int i, seg, nseg, seg_vec;
 };
+template <int NT = kDecThreads>
 __device__ __forceinline__ DecGeom dec_geom(const ScanParams &p, const PartView &pv, bool draw) {
     DecGeom g;
     if (p.nb_dev == nullptr || !draw) {
@@ -526,8 +527,8 @@ __device__ __forceinline__ DecGeom dec_geom(const ScanParams &p, const PartView 
     }
     const int nb = static_cast<int>(max(pv.nb, static_cast<int64_t>(1)));
     const int want = max(1, min(kDrawMaxSeg, min(p.dec.dec_ctas, static_cast<int>(gridDim.x)) / nb));
-    const int per_thread = max(2, (p.RV + kDecThreads * want - 1) / (kDecThreads * want));
-    g.seg_vec = per_thread * kDecThreads;
+    const int per_thread = max(2, (p.RV + NT * want - 1) / (NT * want));
+    g.seg_vec = per_thread * NT;
     g.nseg = (p.RV + g.seg_vec - 1) / g.seg_vec;
     g.i = static_cast<int>(blockIdx.x) / g.nseg;
     g.seg = static_cast<int>(blockIdx.x) % g.nseg;
@@ -585,7 +586,7 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
     const int64_t ob = static_cast<int64_t>(b) * gamma;
     const int64_t bo = static_cast<int64_t>(b) * (gamma + 1);
 
-    // ---- phase 1: facts of every row of the block, one row per thread ----
+    // ---- phase 1: facts of every row of the block ----
     // the drafted tokens, guard flags and the block's schedule inputs (gamma <=
     // 2 NT: at most two positions per thread) are loaded in the same batch as
     // the rows' partials below and stored after them: one round trip
@@ -605,28 +606,41 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
             D_b = d.D_in ? d.D_in[b] : 0;
         }
     }
-    for (int s = tid; s < nd + nt; s += NT) {
-        if (s < nd) {
-            const int j = s;
+    // a row's partials are merged by one thread, or, when rows have more pieces
+    // than a thread loads at once, by a group of 2 or 4: the group that needs
+    // the fewest rounds of loads over the block's rows
+    int lg = 0;   // log2 of the group
+    if (!SHARD && p.pieces > 4) {
+        const int rounds1 = ((nd + nt + NT - 1) / NT) * ((p.pieces + 3) >> 2);
+        const int rounds2 = ((2 * (nd + nt) + NT - 1) / NT) * ((p.pieces + 7) >> 3);
+        const int rounds4 = ((4 * (nd + nt) + NT - 1) / NT) * ((p.pieces + 15) >> 4);
+        lg = (rounds4 < rounds2 && rounds4 < rounds1) ? 2 : (rounds2 < rounds1) ? 1 : 0;
+    }
+    const int first = tid >> lg, step = NT >> lg;
+    for (int s0 = 0; s0 < nd + nt; s0 += step) {
+        const int s = s0 + first;
+        const bool in = s < nd + nt, drow = s < nd;
+        const int j = drow ? s : s - nd;
+        SoftState acc;
+        float g, top[5];
+        bool bad;
+        if (!SHARD) {
+            // (every thread of a warp takes part: the groups exchange by shuffles)
+            const int gi = drow ? max(gd, 0) : gt;
+            const int64_t r = (gi > 0 ? pv.rows0 : 0) + static_cast<int64_t>(i) * (drow ? gamma : gamma + 1) + j;
+            const bool merge = in && (!drow || has_d);
+            merge_row_group<FEAT>(p, pv, r, merge, FEAT && leader && drow, lg, acc, g, bad, top);
+        }
+        if (!in || (tid & ((1 << lg) - 1)) != 0) continue;
+        if (drow) {
             RowFacts f;
             if (has_d) {
                 const ScanGroup &G = p.grp[gd];
-                SoftState acc;
-                float g;
-                bool bad;
-                const int64_t r = (gd ? pv.rows0 : 0) + static_cast<int64_t>(i) * G.npos + j;
-                if (SHARD) {
-                    merge_row_shards(p, r, -1, false, acc, g, bad);
-                    f = row_final(p, G, j, b, acc, g, bad, leader);
-                } else if (FEAT && leader) {
-                    float top[5];
-                    merge_row_t<true>(p, pv, r, acc, g, bad, top);
-                    f = row_final(p, G, j, b, acc, g, bad, leader);
-                    feat_final(G, static_cast<int64_t>(b) * p.gamma + j, top, f.lse);
-                } else {
-                    merge_row(p, pv, r, acc, g, bad);
-                    f = row_final(p, G, j, b, acc, g, bad, leader);
-                }
+                if (SHARD)
+                    merge_row_shards(p, (gd ? pv.rows0 : 0) + static_cast<int64_t>(i) * G.npos + j, -1, false, acc, g,
+                                     bad);
+                f = row_final(p, G, j, b, acc, g, bad, leader);
+                if (FEAT && leader) feat_final(G, static_cast<int64_t>(b) * p.gamma + j, top, f.lse);
             } else {
                 // stand-alone acceptance: the caller's drafter LSE and the token's drafter logit
                 f = facts_invalid();
@@ -638,16 +652,10 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
             }
             put_drafter(F, j, f);
         } else {
-            const int j = s - nd;
             const ScanGroup &G = p.grp[gt];
-            SoftState acc;
-            float g;
-            bool bad;
-            const int64_t r = (gt ? pv.rows0 : 0) + static_cast<int64_t>(i) * G.npos + j;
             if (SHARD)
-                merge_row_shards(p, r, (j < gamma) ? __ldg(d.tokens + ob + j) : -1, j < gamma, acc, g, bad);
-            else
-                merge_row(p, pv, r, acc, g, bad);
+                merge_row_shards(p, (gt ? pv.rows0 : 0) + static_cast<int64_t>(i) * G.npos + j,
+                                 (j < gamma) ? __ldg(d.tokens + ob + j) : -1, j < gamma, acc, g, bad);
             put_target(F, j, row_final(p, G, j, b, acc, g, bad, leader));
         }
     }

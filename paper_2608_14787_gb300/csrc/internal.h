@@ -51,7 +51,14 @@ inline FastDiv make_fastdiv(uint64_t d) {
 // segment); each draw segment is a run of whole 256-vector chunks of the draw
 // row, at most kDrawMaxSeg per block (the last CTA of a block stages every
 // segment's kDecThreads prefixes in shared memory: 1 KiB per segment).
+// After a pass of whole pieces (scan_warps) the kernel runs kDecThreadsWhole
+// threads: rows then have 8 to 16 partials each and there are few of them, so
+// that a group of four threads can take a row (merge_row_group; every four
+// partials that one thread merges cost ~1.2 us), and a block's draw needs half
+// the segments.  GB300, a round of one 32 x 151,936 bf16 block 26.5 -> 25.6 us,
+// of one 8 x 32,000 fp32 block 22.4 -> 17.7 us (pipelined 22.9 -> 14.7 us).
 constexpr int kDecThreads = 256;
+constexpr int kDecThreadsWhole = 512;
 constexpr int kDrawMaxSeg = 64;
 
 // Vocabulary-sharded draw: what the decide kernel leaves, per block, for the
@@ -98,6 +105,7 @@ struct DecideParams {
     int32_t *commit_tokens, *commit_n;
     long long *agreement;
     // sampling draw (residual / bonus inverse CDF), workspace
+    int32_t team;                  // the decide kernel's threads: kDecThreads or kDecThreadsWhole
     int32_t nseg, seg_vec;         // segments per block and vectors per segment
     int32_t dec_ctas;              // decide CTAs resident at once (the draw's one-wave budget)
     float *res_pref;               // [nb, nseg, kDecThreads] per-thread inclusive prefix sums
@@ -136,6 +144,8 @@ struct ScanParams {
     int32_t kcap;            // rank saturation (>= 1)
     int32_t B;
     int32_t W;               // active warps
+    int32_t pieces;          // pieces of a row at most (warps that stream parts of it)
+    int32_t ctas;            // CTAs of a full streaming grid (one per SM)
     int64_t rows0;           // rows of group 0
     int64_t rows;            // rows of all groups
     int64_t T;               // total vectors = rows * RV
@@ -147,10 +157,10 @@ struct ScanParams {
     int64_t R, P[2];
     int64_t T0, C;
     FastDiv divC, divW, divRV, divNpos[2], divWt[2], divP[2];   // division by C, W, RV, grp[g].npos, wt[g], P[g]
-    // The streaming warps of a CTA: warps warp0 .. warp0 + wpc - 1, global
-    // streaming warp blockIdx.x * wpc + (warp - warp0) (set_divisors: all 16;
-    // the pipelined round: warps kPipeWarps-15, the others run the previous
-    // round's decide work).
+    // The streaming warps of a CTA: warps warp0 .. warp0 + wpc - 1
+    // (set_divisors: all 16; the pipelined round: the warps behind the decide
+    // team's).  The call's W warps spread evenly over the grid's CTAs
+    // (scan_warp).
     int32_t warp0, wpc;
     const int32_t *tokens;   // [B, gamma]
     // When set, the number of listed blocks is read from this device word at
@@ -184,8 +194,8 @@ struct ScheduleParams {
     int32_t *K_hat, *K, *D_out;
 };
 
-// The streaming kernel (grid = warps / kWarpsPerCta CTAs).
-cudaError_t launch_scan(const ScanParams &p, int grid, cudaStream_t stream);
+// The streaming kernel: p.W warps over min(p.W, p.ctas) CTAs.
+cudaError_t launch_scan(const ScanParams &p, cudaStream_t stream);
 // Failure-detection test hooks of the streaming kernel, read at each launch:
 // the ring waits' poll limit (0 = kWaitPolls) and the dropped first copy.
 void set_scan_wait_hooks(uint32_t polls, int drop_copy);
@@ -249,8 +259,28 @@ constexpr int64_t kRowStartVec = 400;
 // on GB300, a one-block round at V = 151,936 took 31.5 instead of 34.5 us
 // and the 8 x 32,000 fp32 block 27.9 instead of 68 us (cap 8: 35.8 / 26.6;
 // cap 32: 33.4 / 32.1); the 16-block round is unchanged.
+//
+// A call with few rows cuts every row into the same whole number of pieces, so
+// that each warp streams exactly one piece and pays for one piece's end (a
+// weighted cut makes most warps cross a row: 3 us of the ~15 us that such a
+// pass takes), and its warps spread over all SMs (scan_warp).  From kWholeMin
+// pieces to a row the warps that this leaves out are under 1 in 9, which costs
+// less than the second piece's end; with 2 pieces to a row (the pipelined
+// 16-block round, 2,080 of 2,128 warps) the equal cut lost to the weighted one
+// (63.1 against 61.2 us).  GB300, streaming pass of one 32 x 151,936 bf16
+// block: 15.1 us cut by cost, 12.7 us in 16 pieces a row (8: 16.1, 24 and 32:
+// 13.5); the 8 x 32,000 fp32 block 9.6 -> 7.2 us.
 constexpr int64_t kPiecesPerRow = 16;
+constexpr int64_t kWholeMin = 8;
+// The pieces of every row in a call cut into whole pieces, or 0.
+__host__ __device__ inline int64_t whole_pieces(int64_t W_max, int64_t T, int64_t rows) {
+    int64_t k = rows > 0 ? W_max / rows : 0;
+    k = k < kPiecesPerRow ? k : kPiecesPerRow;
+    return (k >= kWholeMin && 2 * rows * k <= T) ? k : 0;
+}
 __host__ __device__ inline int32_t scan_warps(int64_t W_max, int64_t T, int64_t rows) {
+    const int64_t k = whole_pieces(W_max, T, rows);
+    if (k > 0) return static_cast<int32_t>(rows * k);
     int64_t w = W_max < T / 2 ? W_max : T / 2;
     if (w > rows * kPiecesPerRow) w = rows * kPiecesPerRow;
     return static_cast<int32_t>(w > 1 ? w : 1);
@@ -277,7 +307,11 @@ constexpr int32_t kPipeCostDrafter = 21, kPipeCostTarget = 18;
 // and W are set (host), all 16 warps of a CTA streaming.  The magic divisions
 // are exact while C * W < 2^53 (the callers check it).
 inline void set_divisors(ScanParams &p, int32_t cost_drafter = kCostDrafter, int32_t cost_target = kCostTarget) {
-    const bool mixed = p.n_groups == 2 && p.grp[0].kind != p.grp[1].kind;
+    // a short call's rows are cut into whole pieces: no weights
+    const bool whole = p.rows > 0 && p.W % p.rows == 0 && p.W / p.rows >= kWholeMin;
+    p.pieces = (p.nb_dev || p.rows <= 0) ? static_cast<int32_t>(kPiecesPerRow)
+                                         : static_cast<int32_t>((p.W + p.rows - 1) / p.rows + (whole ? 0 : 1));
+    const bool mixed = p.n_groups == 2 && p.grp[0].kind != p.grp[1].kind && !whole;
     for (int g = 0; g < 2; ++g) p.wt[g] = mixed ? (p.grp[g].kind == 0 ? cost_drafter : cost_target) : 1;
     const int64_t wmax = std::max(p.wt[0], p.wt[1]), wmin = std::min(p.wt[0], p.wt[1]);
     // The row-start cost must leave every warp at least one vector start: a
@@ -287,7 +321,7 @@ inline void set_divisors(ScanParams &p, int32_t cost_drafter = kCostDrafter, int
     // (R + 2 wmax).  Rows too short for that (and too short to be cut at all)
     // get no row-start cost.
     int64_t R = kRowStartVec * wmax;
-    if (p.RV < 2 * kPiecesPerRow || wmin * p.RV + R < kPiecesPerRow * (R + 2 * wmax)) R = 0;
+    if (whole || p.RV < 2 * kPiecesPerRow || wmin * p.RV + R < kPiecesPerRow * (R + 2 * wmax)) R = 0;
     p.R = R;
     for (int g = 0; g < 2; ++g) p.P[g] = p.wt[g] * p.RV + R;
     p.T0 = p.rows0 * p.RV;

@@ -73,9 +73,7 @@ __global__ void __launch_bounds__(kThreads, 1) pipe_kernel(const __grid_constant
     }
     constexpr int kTeamWarps = TEAM / 32, kStreamWarps = kWarpsPerCta - kTeamWarps;
     const int warp = threadIdx.x >> 5;
-    const int64_t gw = static_cast<int64_t>(blockIdx.x) * kStreamWarps + (warp - kTeamWarps);
-    if (pp.has_next && gw < pp.next.W)
-        scan_warp<DTN, false, kPipeStages>(pp.next, smem, gw, warp - kTeamWarps, kStreamWarps);
+    if (pp.has_next) scan_warp<DTN, false, kPipeStages>(pp.next, smem, warp - kTeamWarps, kStreamWarps);
 }
 
 using PipeKernel = void (*)(PipeParams);

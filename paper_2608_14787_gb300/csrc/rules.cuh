@@ -12,7 +12,7 @@
 //    K_min, staleness and guards;
 //  * periodic_khat -- the confidence-free periodic baseline of the appendix's
 //    periodic-skipping paragraph (an attempt every P rounds, same guards);
-//  * merge_row_t<true> / feat_final -- the extended features of App. A.7: a
+//  * merge_row_group<true> / feat_final -- the extended features of App. A.7: a
 //    drafter row's five largest entries merged from its pieces' lists (loaded
 //    with its partials), then the probability margin and the top-5 mass.
 //
@@ -54,16 +54,36 @@ __device__ __forceinline__ Partial load_partial(const Partial *p) {
     return u.q;
 }
 
+// A descending list's insertion of z.
+__device__ __forceinline__ void insert5(float (&t)[5], float z) {
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const float hi = fmaxf(t[k], z), lo = fminf(t[k], z);
+        t[k] = hi;
+        z = lo;
+    }
+}
+
 // Merged state of global row r, whose pieces were streamed by warps fw..lw
-// (partial of warp w at index r + w), merged in warp order, four loads in
-// flight at a time.  The row's first piece carries its token logit; any piece
-// flags an out-of-range token.  FEAT (drafter rows of the feature call): also
-// the row's five largest entries t, merged from the pieces' lists (p.feat,
-// indexed like the partials) loaded in the same batches.
+// (partial of warp w at index r + w), by a group of 2^lg neighbouring threads:
+// each merges a run of the pieces in warp order, four loads in flight at a
+// time, and the runs are merged in order by shuffles; the group's first thread
+// holds the result.  Every thread of the warp calls it; `on` says whether its
+// group has a row.  The row's first piece carries its token logit; any piece
+// flags an out-of-range token.  FEAT with `feat` set (drafter rows of the
+// feature call): also the row's five largest entries t, merged from the
+// pieces' lists (p.feat, indexed like the partials) loaded in the same batches.
 template <bool FEAT>
-__device__ __forceinline__ void merge_row_t(const ScanParams &p, const PartView &pv, int64_t r, SoftState &acc,
-                                            float &g, bool &tok_bad, float (&t)[5]) {
-    const int64_t fw = part_owner(p, pv, r * p.RV), lw = part_owner(p, pv, (r + 1) * p.RV - 1);
+__device__ __forceinline__ void merge_row_group(const ScanParams &p, const PartView &pv, int64_t r, bool on, bool feat,
+                                                int lg, SoftState &acc, float &g, bool &tok_bad, float (&t)[5]) {
+    int64_t fw = 0, lw = -1;
+    if (on) {
+        fw = part_owner(p, pv, r * p.RV);
+        lw = part_owner(p, pv, (r + 1) * p.RV - 1);
+    }
+    const int at = static_cast<int>(threadIdx.x) & ((1 << lg) - 1);
+    const int run = (static_cast<int>(lw - fw) + (1 << lg)) >> lg;   // pieces of a run
+    const int64_t wa = fw + at * run, wb = min(lw, wa + run - 1);
     acc = soft_identity();
     g = qnan();
     tok_bad = false;
@@ -71,21 +91,21 @@ __device__ __forceinline__ void merge_row_t(const ScanParams &p, const PartView 
 #pragma unroll
         for (int k = 0; k < 5; ++k) t[k] = -INFINITY;
     }
-    for (int64_t w0 = fw; w0 <= lw; w0 += 4) {
+    for (int64_t w0 = wa; w0 <= wb; w0 += 4) {
         Partial pt[4];
         uint4 fv[4][2];   // FEAT: the pieces' top-5 lists, loaded in the same batch
 #pragma unroll
         for (int u = 0; u < 4; ++u)
-            if (w0 + u <= lw) {
+            if (w0 + u <= wb) {
                 pt[u] = load_partial(p.partials + r + w0 + u);
-                if (FEAT) {
+                if (FEAT && feat) {
                     fv[u][0] = __ldcg(reinterpret_cast<const uint4 *>(p.feat + r + w0 + u));
                     fv[u][1] = __ldcg(reinterpret_cast<const uint4 *>(p.feat + r + w0 + u) + 1);
                 }
             }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            if (w0 + u > lw) break;
+            if (w0 + u > wb) break;
             if (w0 + u == fw) g = pt[u].g;
             tok_bad |= pt[u].rank < 0;
             SoftState o;
@@ -97,28 +117,27 @@ __device__ __forceinline__ void merge_row_t(const ScanParams &p, const PartView 
             o.amax = pt[u].amax;
             o.rank = max(pt[u].rank, 0);
             acc = soft_merge(acc, o);
-            if (FEAT) {
-                const float f[5] = {__uint_as_float(fv[u][0].x), __uint_as_float(fv[u][0].y),
-                                    __uint_as_float(fv[u][0].z), __uint_as_float(fv[u][0].w),
-                                    __uint_as_float(fv[u][1].x)};
-#pragma unroll
-                for (int i = 0; i < 5; ++i) {
-                    float z = f[i];
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) {   // insert z into the descending list
-                        const float hi = fmaxf(t[k], z), lo = fminf(t[k], z);
-                        t[k] = hi;
-                        z = lo;
-                    }
-                }
+            if (FEAT && feat) {
+                insert5(t, __uint_as_float(fv[u][0].x));
+                insert5(t, __uint_as_float(fv[u][0].y));
+                insert5(t, __uint_as_float(fv[u][0].z));
+                insert5(t, __uint_as_float(fv[u][0].w));
+                insert5(t, __uint_as_float(fv[u][1].x));
             }
         }
     }
-}
-__device__ __forceinline__ void merge_row(const ScanParams &p, const PartView &pv, int64_t r, SoftState &acc, float &g,
-                                          bool &tok_bad) {
-    float t[5];
-    merge_row_t<false>(p, pv, r, acc, g, tok_bad, t);
+    for (int off = 1; off < (1 << lg); off <<= 1) {
+        // the run `off` threads above follows this one
+        acc = soft_merge(acc, soft_shfl_down(acc, off));
+        tok_bad = (__shfl_down_sync(0xFFFFFFFFu, tok_bad ? 1 : 0, off) != 0) || tok_bad;
+        if (FEAT) {
+            float z[5];
+#pragma unroll
+            for (int k = 0; k < 5; ++k) z[k] = __shfl_down_sync(0xFFFFFFFFu, t[k], off);
+#pragma unroll
+            for (int k = 0; k < 5; ++k) insert5(t, z[k]);
+        }
+    }
 }
 
 // Vocabulary-sharded rows: the merged state of row r from the S slices'

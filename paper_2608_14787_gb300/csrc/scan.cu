@@ -1,4 +1,5 @@
 // scan.cu -- the streaming kernel (the per-warp work is in scan.cuh).
+#include <algorithm>
 #include <atomic>
 
 #include "scan.cuh"
@@ -12,12 +13,10 @@ namespace {
 template <int DT, bool FEAT>
 __global__ void __launch_bounds__(kThreads, 1) scan_kernel(const __grid_constant__ ScanParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
-    const int64_t gw = static_cast<int64_t>(blockIdx.x) * kWarpsPerCta + (threadIdx.x >> 5);
-    if (gw >= p.W) return;
     // launched as a programmatic dependent of whatever precedes it in the
     // stream: nothing is read or written before that work has completed
     griddep_wait();
-    scan_warp<DT, FEAT>(p, smem, gw, threadIdx.x >> 5, kWarpsPerCta);
+    scan_warp<DT, FEAT>(p, smem, threadIdx.x >> 5, blockDim.x >> 5);
 }
 
 }  // namespace
@@ -51,7 +50,7 @@ void set_scan_wait_hooks(uint32_t polls, int drop_copy) {
     g_drop_copy.store(drop_copy ? 1 : 0, std::memory_order_relaxed);
 }
 
-cudaError_t launch_scan(const ScanParams &p, int grid, cudaStream_t stream) {
+cudaError_t launch_scan(const ScanParams &p, cudaStream_t stream) {
     const bool bf = p.dtype == SDD_BF16, feat = p.feat != nullptr;
     void (*const k)(ScanParams) = feat ? (bf ? scan_kernel<SDD_BF16, true> : scan_kernel<SDD_F32, true>)
                                        : (bf ? scan_kernel<SDD_BF16, false> : scan_kernel<SDD_F32, false>);
@@ -59,7 +58,8 @@ cudaError_t launch_scan(const ScanParams &p, int grid, cudaStream_t stream) {
     const uint32_t polls = g_wait_polls.load(std::memory_order_relaxed);
     q.wait_polls = polls ? polls : kWaitPolls;
     q.drop_copy = g_drop_copy.load(std::memory_order_relaxed);
-    return launch_dependent(k, dim3(grid), dim3(kThreads), kScanSmem, stream, q);
+    const int grid = std::min(p.W, p.ctas), warps = (p.W + grid - 1) / grid;
+    return launch_dependent(k, dim3(grid), dim3(32 * warps), ring_bytes(kStages, warps), stream, q);
 }
 
 }  // namespace sdd

@@ -446,20 +446,22 @@ __device__ __forceinline__ float token_logit(const ScanParams &p, const PartView
     return fmax_nan(logit_at<DT>(row_base(p, pv, r), x.t), clamp_floor());
 }
 
-// The streaming work of one warp of the CTA, streaming warp gw (below p.W;
-// blockIdx.x * p.wpc + warp - p.warp0), once the work ahead of it in the
-// stream has completed.  smem is the CTA's ring area, ring_bytes(STAGES,
-// n_rings): one ring of STAGES tiles per streaming warp, then their barriers;
-// this warp's is ring ring_idx.  FEAT: also the five largest logits of
+// The streaming work of streaming warp w of the CTA, once the work ahead of it
+// in the stream has completed.  smem is the CTA's ring area,
+// ring_bytes(STAGES, n_rings): one ring of STAGES tiles per streaming warp,
+// then their barriers; this warp's is ring w.  FEAT: also the five largest logits of
 // every drafter row piece (extended features); without it the code is
 // unchanged.
 template <int DT, bool FEAT, int STAGES = kStages>
-__device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *smem, int64_t gw, int ring_idx,
-                                          int n_rings) {
+__device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *smem, int w, int n_rings) {
     constexpr int kStages = STAGES;
     const int lane = threadIdx.x & 31;
     const PartView pv = part_view(p);
-    if (gw >= pv.W) return;   // (a device block count can leave warps without work)
+    // the call's warps spread evenly over the CTAs (a call too small for every
+    // warp, or a device block count, leaves warps of each CTA without work)
+    const int wpc = (pv.W + gridDim.x - 1) / gridDim.x;
+    const int64_t gw = static_cast<int64_t>(blockIdx.x) * wpc + w;
+    if (w >= wpc || gw >= pv.W) return;
     // The sampling draw's arrival counters of this call's blocks start at zero
     // (the decide kernel behind this one reads them only after this grid has
     // completed), so the workspace needs no zero fill and calls of any shape
@@ -469,8 +471,8 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
     constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
     const int tail = p.V % EPV;  // valid entries of the last vector of a row (0 = full)
 
-    unsigned char *ring = smem + ring_idx * (kStages * kTileBytes);
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + n_rings * kStages * kTileBytes) + ring_idx * kStages;
+    unsigned char *ring = smem + w * (kStages * kTileBytes);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + n_rings * kStages * kTileBytes) + w * kStages;
     if (lane == 0) {
 #pragma unroll
         for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);

@@ -1,0 +1,74 @@
+"""Rounds whose rows are cut into whole pieces (8 to 16 warps to a row) and the
+rounds just outside that rule, against the oracle: blocks of 1 to 3 positions
+up to 304 rows (the last whole cut on 152 SMs), odd vocabularies whose pieces
+end inside a vector tile, rows too short for 16 pieces, the post-verify half
+with its block count on the device, and the pipelined chain."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2608_14787_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _check(sdd, orc, rnd, blk, seed, round_):
+    zd, zt, x = synth.bf16_bits(blk.z_d), synth.bf16_bits(blk.z_t), blk.x.cpu().numpy()
+    st = orc.row_stats(zd, tokens=x)
+    rtol = 2e-3 if blk.z_d.dtype == torch.bfloat16 else 1e-5     # the parity tests' tolerances
+    np.testing.assert_allclose(rnd.q.cpu().numpy(), st.q, rtol=rtol, atol=1e-7)
+    np.testing.assert_allclose(rnd.lse.cpu().numpy(), st.lse, rtol=1e-6)
+    np.testing.assert_allclose(rnd.entropy.cpu().numpy(), st.entropy, rtol=rtol, atol=1e-7)
+    np.testing.assert_array_equal(rnd.argmax.cpu().numpy(), st.argmax)
+    for b in range(x.shape[0]):
+        L, tok, margin = orc.verify_strict(zt[b], zd[b], x[b], seed=seed, b=b, round_=round_)
+        if margin >= 1e-6:
+            assert int(rnd.L_strict[b]) == L and np.array_equal(rnd.tokens_strict[b].cpu().numpy(), tok), b
+        Lk, tk, _ = orc.verify_topk(orc.target_facts(zt[b], x[b]), x[b], 2)
+        assert int(rnd.L_topk[0, b]) == Lk and np.array_equal(rnd.tokens_topk[0, b].cpu().numpy(), tk)
+
+
+SHAPES = [(1, 1, 8), (1, 1, 40), (1, 8, 1003), (1, 32, 20011), (3, 17, 4001), (8, 18, 2500), (9, 17, 2500), (60, 2, 3001),
+          (100, 1, 1999), (102, 1, 1999)]
+
+
+@pytest.mark.parametrize("B,gamma,V", SHAPES)
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_small_rounds(sdd, orc, B, gamma, V, dtype):
+    blk = synth.make_block("c3", device="cuda", B=B, gamma=gamma, V=-(-V // 8) * 8, dtype=dtype, round_=B)
+    blk.z_d, blk.z_t, blk.x = blk.z_d[..., :V], blk.z_t[..., :V], blk.x.clamp(max=V - 1)
+    rnd = sdd.BlockRound(B, gamma, V, dtype=dtype, ks=(2,), K_min=0)
+    rnd.set_inputs(blk.z_d, blk.z_t, blk.x, seed=5, round_=2)
+    rnd.run()
+    _check(sdd, orc, rnd, blk, 5, 2)
+    # the two halves apart, the verified blocks listed on the device
+    conf = sdd.confidence(blk.z_d, blk.x)
+    assert torch.equal(conf.argmax, rnd.argmax)
+    # (cut differently: each side within 2^-22 of the sums' value and a rounding to fp32)
+    torch.testing.assert_close(conf.q, rnd.q, rtol=1e-6, atol=0)
+    K = (torch.arange(B, device="cuda") % 3 == 1).to(torch.int32)
+    rows, n = sdd.select_rows(K)
+    L, tok, _ = sdd.verify_strict_listed(blk.z_t, blk.x, rows, n, z_d=blk.z_d, draft=conf, seed=5, round_=2)
+    keep = K == 0
+    assert torch.equal(L[keep], rnd.L_strict[keep]) and torch.equal(tok[keep], rnd.tokens_strict[keep])
+    assert bool((L[~keep] == -2).all())
+
+
+def test_small_round_features(sdd, orc):
+    blk = synth.make_block("c2", device="cuda", V=20016, round_=3)
+    conf = sdd.confidence(blk.z_d, blk.x, features=True)
+    margin, top5 = orc.row_features(synth.bf16_bits(blk.z_d))
+    np.testing.assert_allclose(conf.top5.cpu().numpy(), top5, rtol=2e-3)
+    p1 = conf.maxprob.cpu().numpy()
+    assert np.all(np.abs(conf.margin.cpu().numpy() - margin) <= 2e-3 * p1)
+
+
+def test_small_pipelined_chain(sdd, orc):
+    blks = [synth.make_block("c3", device="cuda", B=2, gamma=9, V=8008, round_=r) for r in range(3)]
+    rnds = [sdd.BlockRound(2, 9, 8008, ks=(2,), K_min=0) for _ in blks]
+    for r, (b, q) in enumerate(zip(blks, rnds)):
+        q.set_inputs(b.z_d, b.z_t, b.x, seed=1, round_=r)
+        sdd.block_pipelined(q, rnds[r - 1] if r else None)
+    sdd.block_pipelined(None, rnds[-1])
+    for r, (b, q) in enumerate(zip(blks, rnds)):
+        _check(sdd, orc, q, b, 1, r)
