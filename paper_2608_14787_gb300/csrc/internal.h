@@ -162,6 +162,7 @@ struct ScanParams {
     // team's).  The call's W warps spread evenly over the grid's CTAs
     // (scan_warp).
     int32_t warp0, wpc;
+    int32_t spread;          // warps of a CTA that have work: ceil(W / CTAs) (set at launch; not with nb_dev)
     const int32_t *tokens;   // [B, gamma]
     // When set, the number of listed blocks is read from this device word at
     // launch (at most grp[g].nb, which then sizes the grid): rows, T, T0, C
@@ -240,14 +241,14 @@ cudaError_t launch_uniforms(uint64_t seed, const uint32_t *j, const uint32_t *b,
                             const uint32_t *purpose, int64_t n, float *u, cudaStream_t stream);
 // Relative per-vector cost of streaming a drafter row (online softmax plus
 // the entropy accumulator) and a target row (online softmax plus the rank
-// count), measured on GB300: 10 : 9.
+// count), measured on GB300 (streaming pass of 16 blocks): 10 : 9 51.1 us,
+// 7 : 6 52.1, 11 : 9 53.4, 4 : 3 54.5.
 constexpr int32_t kCostDrafter = 10, kCostTarget = 9;
 // Extra cost of a row's first vector, in vectors of the heavier group: the
 // end of a warp's piece of a row (exact argmax re-read, reduction, partial)
-// and the next piece's start.  Per-warp globaltimer stamps (one 16-block
-// round): warps whose range crosses a row boundary ended 3.2 us after those
-// whose range does not.  Measured on GB300 (16-block round, back to back):
-// 0 -> 69.08 us, 200 -> 68.68, 400 -> 68.62, 700 -> 69.21.
+// and the next piece's start.  Measured on GB300 (back to back, 16 blocks):
+// round 64.27 / 64.13 / 64.01 us with 0 / 200 / 400, pipelined 55.99 / 55.89 /
+// 55.14, confidence 33.1 / 33.1 / 32.6.
 constexpr int64_t kRowStartVec = 400;
 
 // Warps of a launch over T vectors in `rows` rows with at most W_max warps:
@@ -299,8 +300,8 @@ constexpr int64_t kPipeSmallBytes = int64_t(64) << 20;
 // The pipelined pass's cost weights (drafter, target vector), as kCostDrafter
 // and kCostTarget for the streaming kernel: on fourteen warps beside the
 // decide work the drafter rows' entropy work weighs more (GB300, 16-block
-// round: 10 : 9 62.3 us, 21 : 18 61.2, 11 : 9 61.5, 23 : 18 62.2, 12 : 9 63.5;
-// with 10 : 9 the CTAs streaming drafter rows ended ~2.5 us after the others).
+// round: 21 : 18 55.1 us, 22 : 18 56.0, 24 : 18 57.4, 26 : 18 59.5; 10 : 9 ended
+// the CTAs of drafter rows ~2.5 us after the others).
 constexpr int32_t kPipeCostDrafter = 21, kPipeCostTarget = 18;
 
 // The cost weights and division constants of a launch whose groups, rows, T
@@ -425,7 +426,9 @@ __device__ __forceinline__ PartView part_view(const ScanParams &p) {
 // owns the costs [floor(w C / W), floor((w+1) C / W)) and so the vectors whose
 // cost interval starts there: [start(w), start(w+1)) with start(w) the first
 // vector of cost >= floor(w C / W).  Requires C W < 2^53 (checked by the host).
-__device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartView &v, int64_t w) {
+// Also the row r (of both groups) that holds start(w) and its vector k there.
+__device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartView &v, int64_t w, int64_t &row,
+                                              int32_t &kv) {
     const int64_t c = fast_div(w * v.C, v.divW);
     const int64_t c0 = v.rows0 * p.P[0];   // the cost of group 0
     const int g = (c <= c0) ? 0 : 1;
@@ -434,6 +437,9 @@ __device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartVie
     const int64_t rem = cg - r * p.P[g];
     int64_t k = 0;
     if (rem > 0) k = (rem <= p.R) ? 1 : fast_div(rem - p.R + p.wt[g] - 1, p.divWt[g]);
+    const bool next = k == p.RV;   // (the row's end: the next row's start)
+    row = (g ? v.rows0 : 0) + r + (next ? 1 : 0);
+    kv = next ? 0 : static_cast<int32_t>(k);
     return (g ? v.T0 : 0) + r * p.RV + k;
 }
 // The warp owning vector v.

@@ -128,6 +128,7 @@ cudaError_t launch_pipe(const ScanParams *next, const ScanParams *prev, int grid
     pp.next = *next;
     pp.has_next = 1;
     pp.next.wait_polls = kWaitPolls;
+    pp.next.spread = (next->W + grid - 1) / std::max(grid, 1);
     size_t smem = static_cast<size_t>(ti ? pipe_rings(kPipeTeamSmall) : pipe_rings(kPipeTeam));
     if (prev) {
         pp.prev = *prev;

@@ -57,9 +57,10 @@ cudaError_t launch_scan(const ScanParams &p, cudaStream_t stream) {
     ScanParams q = p;
     const uint32_t polls = g_wait_polls.load(std::memory_order_relaxed);
     q.wait_polls = polls ? polls : kWaitPolls;
+    q.spread = (p.W + std::min(p.W, p.ctas) - 1) / std::min(p.W, p.ctas);
     q.drop_copy = g_drop_copy.load(std::memory_order_relaxed);
-    const int grid = std::min(p.W, p.ctas), warps = (p.W + grid - 1) / grid;
-    return launch_dependent(k, dim3(grid), dim3(32 * warps), ring_bytes(kStages, warps), stream, q);
+    return launch_dependent(k, dim3(std::min(p.W, p.ctas)), dim3(32 * q.spread), ring_bytes(kStages, q.spread), stream,
+                            q);
 }
 
 }  // namespace sdd

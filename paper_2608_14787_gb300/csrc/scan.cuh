@@ -125,31 +125,6 @@ __device__ __noinline__ int count_before(const uint4 *tile, int n, int k0, int l
     return cnt;
 }
 
-// Resolve a lane's argmax: the first of its entries equal to m inside the tile
-// that starts at vector k0 of the row (re-read from global memory, all loads
-// issued before the first compare; the row's padding and entries past V are
-// excluded).
-template <int DT>
-__device__ __noinline__ int first_index(const char *rowp, int k0, int lane, int RV, int V, float m) {
-    constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
-    uint4 w[kVPL];
-#pragma unroll
-    for (int i = 0; i < kVPL; ++i) {
-        const int vec = k0 + lane + 32 * i;
-        w[i] = (vec < RV) ? __ldg(reinterpret_cast<const uint4 *>(rowp) + vec) : make_uint4(0, 0, 0, 0);
-    }
-#pragma unroll
-    for (int i = 0; i < kVPL; ++i) {
-        const int vec = k0 + lane + 32 * i;
-        if (vec >= RV) break;
-        const uint4 c = clamp_vec<DT>(w[i]);
-#pragma unroll
-        for (int e = 0; e < EPV; ++e)
-            if (vec * EPV + e < V && vec_elem<DT>(c, e) == m) return vec * EPV + e;
-    }
-    return INT32_MAX;
-}
-
 // Process one full tile: the lane's vectors are lane, lane+32, ... of the tile.
 // Sums are relative to the integer reference st.r (log2 units), so a new
 // maximum rescales by an exact power of two.  A new maximum only records the
@@ -420,30 +395,59 @@ __device__ __forceinline__ void group_top5(const char *rowp, int kb, int ke, int
     }
 }
 
-// Drafted token of global row r, if the row has one (load issued, not waited on).
-struct RowTok {
-    int t;
-    bool has;
+// What a warp needs of a row that its range touches, held one row per lane
+// (RowWindow: rows first .. first + 31): computed for all the rows at once,
+// with their token loads in flight together, when the warp starts.  The first
+// tile of a full grid used to land 5.4 us after the kernel's wait (the range's
+// ends, the rows and two dependent token loads one after another, ahead of the
+// first tile's wait): with the two ends on two lanes, the rows on lanes and
+// the token logits fetched behind the first copies 3.6 us.  Together with the
+// piece's end below (2.4 -> 0.8 us) a 16-block streaming pass takes 51.1
+// instead of 55.1 us (6.18 TB/s), one block 10.1 instead of 12.6 us.
+struct RowWindow {
+    int64_t first;
+    const char *base;   // the row's logits
+    int32_t tok;        // its drafted token (-1: none or out of range)
+    float g;            // the token's clamped logit (NaN if none)
+    uint32_t flags;     // kRowDrafter, kRowBadTok
 };
-__device__ __forceinline__ RowTok row_token(const ScanParams &p, const PartView &pv, int64_t r) {
-    RowTok x{0, false};
-    if (r < pv.rows) {
+constexpr uint32_t kRowDrafter = 1, kRowBadTok = 2;
+
+// Rows first + lane up to `last`; the token logits are loaded by window_logits.
+__device__ __forceinline__ void window_rows(const ScanParams &p, const PartView &pv, int64_t first, int64_t last,
+                                            int lane, RowWindow &w) {
+    w.first = first;
+    w.base = nullptr;
+    w.tok = -1;
+    w.flags = 0;
+    const int64_t r = first + lane;
+    if (r <= last) {
         int gi, j, b;
         int64_t lr;
         bool ok;
         row_locate(p, pv, r, gi, lr, j, b, ok);
+        const ScanGroup &G = p.grp[gi];
+        w.base = G.base + (static_cast<int64_t>(b) * G.npos + j) * G.stride_bytes;
+        w.flags = (G.kind == 0) ? kRowDrafter : 0u;
         if (j < p.gamma) {
-            x.t = __ldg(p.tokens + static_cast<int64_t>(b) * p.gamma + j);
-            x.has = true;
+            w.tok = __ldg(p.tokens + static_cast<int64_t>(b) * p.gamma + j);
+            w.flags |= kRowBadTok;   // (until window_logits has seen it)
         }
     }
-    return x;
 }
-// Clamped logit of row r at its drafted token (NaN if none or out of range).
 template <int DT>
-__device__ __forceinline__ float token_logit(const ScanParams &p, const PartView &pv, int64_t r, RowTok x) {
-    if (!x.has || x.t < 0 || x.t >= p.V) return __int_as_float(0x7FC00000);
-    return fmax_nan(logit_at<DT>(row_base(p, pv, r), x.t), clamp_floor());
+__device__ __forceinline__ void window_logits(const ScanParams &p, RowWindow &w) {
+    w.g = __int_as_float(0x7FC00000);
+    if ((w.flags & kRowBadTok) && w.tok >= 0 && w.tok < p.V) {
+        w.flags &= ~kRowBadTok;
+        w.g = fmax_nan(logit_at<DT>(w.base, w.tok), clamp_floor());
+    } else {
+        w.tok = -1;
+    }
+}
+__device__ __forceinline__ const char *shfl_ptr(const char *ptr, int src) {
+    return reinterpret_cast<const char *>(
+        __shfl_sync(0xFFFFFFFFu, reinterpret_cast<unsigned long long>(ptr), src));
 }
 
 // The streaming work of streaming warp w of the CTA, once the work ahead of it
@@ -459,7 +463,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
     const PartView pv = part_view(p);
     // the call's warps spread evenly over the CTAs (a call too small for every
     // warp, or a device block count, leaves warps of each CTA without work)
-    const int wpc = (pv.W + gridDim.x - 1) / gridDim.x;
+    const int wpc = p.nb_dev ? (pv.W + gridDim.x - 1) / gridDim.x : p.spread;
     const int64_t gw = static_cast<int64_t>(blockIdx.x) * wpc + w;
     if (w >= wpc || gw >= pv.W) return;
     // The sampling draw's arrival counters of this call's blocks start at zero
@@ -480,11 +484,17 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
     }
     __syncwarp();
 
-    const int64_t v0 = part_start(p, pv, gw), v1 = part_start(p, pv, gw + 1);
-    Cursor pc{v0, fast_div(v0, p.divRV), 0};
-    pc.k = static_cast<int32_t>(v0 - pc.r * p.RV);
+    // the range's two ends by two lanes at once, then the rows it touches
+    int64_t rs;
+    int32_t ks;
+    const int64_t vs = part_start(p, pv, gw + (lane & 1), rs, ks);
+    const int64_t v0 = __shfl_sync(0xFFFFFFFFu, vs, 0), v1 = __shfl_sync(0xFFFFFFFFu, vs, 1);
+    Cursor pc{v0, __shfl_sync(0xFFFFFFFFu, rs, 0), __shfl_sync(0xFFFFFFFFu, ks, 0)};
+    const int64_t r_last = __shfl_sync(0xFFFFFFFFu, rs, 1) - (__shfl_sync(0xFFFFFFFFu, ks, 1) == 0 ? 1 : 0);
     Cursor cc = pc;
-    const char *prow = row_base(p, pv, pc.r);
+    RowWindow win;
+    window_rows(p, pv, pc.r, r_last, lane, win);
+    const char *prow = shfl_ptr(win.base, 0);
     const uint64_t pol = l2_evict_first_policy();   // the logits are read once
     uint32_t pending = 0;  // slots with a copy in flight
     uint32_t phase = 0;    // parity bit per slot
@@ -511,23 +521,20 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
         if (pc.k == p.RV && pc.v < v1) {
             pc.k = 0;
             pc.r += 1;
-            prow = row_base(p, pv, pc.r);
+            prow = (pc.r - win.first < 32) ? shfl_ptr(win.base, static_cast<int>(pc.r - win.first))
+                                           : row_base(p, pv, pc.r);
         }
     };
     for (int s = 0; s < kStages && pc.v < v1; ++s) issue(s);
 
-    // Drafted tokens and their logits run ahead of the stream: the token two
-    // rows ahead and the logit one row ahead are in flight while the current
-    // piece streams, so no piece start waits on a dependent pair of loads.
-    RowTok tokA = row_token(p, pv, cc.r), tokB = row_token(p, pv, cc.r + 1);
-    float gA = token_logit<DT>(p, pv, cc.r, tokA);
+    window_logits<DT>(p, win);   // (behind the first copies)
 
     SoftState st = soft_identity();
     uint32_t ck[5];        // FEAT: the lane's five largest tile maxima of the piece (keys) ...
     int ct[5];             // ... and their tiles' first vectors (drafter rows)
     int kb = 0;            // FEAT: the piece's first vector in the row
     float s_hi = 0.f, s_lo = 0.f;   // the lane's exp-sum as an fp32 pair
-    bool in_piece = false;
+    bool in_piece = false, fresh = false;   // fresh: the piece's token has not been fetched yet
     bool ent = false;      // warp-uniform: drafter row (entropy accumulator, clamped entries)
     int tok = -1;          // drafted token of the current row (-1: none or out of range)
     bool tok_bad = false;  // the row has a drafted token outside [0, V)
@@ -551,23 +558,16 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
             }
             s_hi = 0.f;
             s_lo = 0.f;
-            int gi, j, b;
-            int64_t lr;
-            bool ok;
-            row_locate(p, pv, cc.r, gi, lr, j, b, ok);
-            const ScanGroup &G = p.grp[gi];
-            crow = G.base + (static_cast<int64_t>(b) * G.npos + j) * G.stride_bytes;
-            ent = G.kind == 0;
-            const bool tok_ok = tokA.has && tokA.t >= 0 && tokA.t < p.V;
-            tok = tok_ok ? tokA.t : -1;
-            tok_bad = tokA.has && !tok_ok;
-            g = gA;
-            // advance the prefetch: logit of the next row, token of the one after
-            gA = token_logit<DT>(p, pv, cc.r + 1, tokB);
-            tokA = tokB;
-            tokB = row_token(p, pv, cc.r + 2);
-            rank_on = !ent && tok >= 0;
+            if (cc.r - win.first >= 32) {   // (a range of more than 32 rows)
+                window_rows(p, pv, cc.r, r_last, lane, win);
+                window_logits<DT>(p, win);
+            }
+            const int at = static_cast<int>(cc.r - win.first);
+            crow = shfl_ptr(win.base, at);
+            ent = (__shfl_sync(0xFFFFFFFFu, win.flags, at) & kRowDrafter) != 0;
+            rank_on = false;
             wrank = 0;
+            fresh = true;
             in_piece = true;
         }
         // warp-uniform outcome: a phase that one lane saw complete is complete for all
@@ -581,6 +581,16 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
         const float cm = ent ? process_tile<DT, true>(tile, cc.k, lane, st, s_hi, s_lo)
                              : process_tile<DT, false>(tile, cc.k, lane, st, s_hi, s_lo);
         if (FEAT && ent) group_update(cm, cc.k, ck, ct);
+        if (fresh) {
+            // the token's logit is first needed here: its load had the first
+            // tile's copy and arithmetic to arrive
+            const int at = static_cast<int>(cc.r - win.first);
+            tok = __shfl_sync(0xFFFFFFFFu, win.tok, at);
+            g = __shfl_sync(0xFFFFFFFFu, win.g, at);
+            tok_bad = (__shfl_sync(0xFFFFFFFFu, win.flags, at) & kRowBadTok) != 0;
+            rank_on = !ent && tok >= 0;
+            fresh = false;
+        }
         if (rank_on) {
             const bool want = cm >= g;
             if (__any_sync(0xFFFFFFFFu, want)) {
@@ -600,25 +610,46 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
         cc.v += n;
         cc.k += n;
         if (row_end || cc.v == v1) {
-            // end of this warp's piece of row cc.r: exact argmax of the piece,
-            // then the warp's partial state
-            float M = st.m;
+            // end of this warp's piece of row cc.r: its maximum M, the first
+            // index that attains it, and the lanes' sums against M.  The lanes
+            // that hold M re-read their vectors of its tile while the sums
+            // are added.
+            const float M = fkey_inv(__reduce_max_sync(0xFFFFFFFFu, fkey(st.m)));
+            const bool holds = st.m == M && st.amax != INT32_MAX;
+            const int va = (holds ? st.amax : 0) + lane;
+            uint4 aw[kVPL];
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) M = fmax_nan(M, __shfl_xor_sync(0xFFFFFFFFu, M, off));
-            int idx = INT32_MAX;
-            auto resolve = [&]() {
-                if (st.m == M && st.amax != INT32_MAX) idx = first_index<DT>(crow, st.amax, lane, p.RV, p.V, M);
-            };
+            for (int i = 0; i < kVPL; ++i) {
+                const int vec = va + 32 * i;
+                aw[i] = (holds && vec < p.RV) ? __ldg(reinterpret_cast<const uint4 *>(crow) + vec)
+                                              : make_uint4(0, 0, 0, 0);
+            }
             float top[5];
-            if (FEAT && ent)
-                group_top5<DT>(crow, kb, cc.k, p.V, lane, ck, ct, top, resolve);   // (cc.k: the piece's end)
-            else
-                resolve();
-            st.amax = idx;
-            st.rank = (lane == 0) ? wrank : 0;
-            st.sh = s_hi;
-            st.sl = s_lo;
-            const SoftState red = soft_warp_reduce(st);
+            if (FEAT && ent) group_top5<DT>(crow, kb, cc.k, p.V, lane, ck, ct, top, [] {});   // (cc.k: the piece's end)
+            // every reference is a power of two below M's, so the rescaling is
+            // exact; each step adds two lanes' double-floats the same way on
+            // both, so all lanes agree
+            const float rM = ceilf(M * kLog2e);
+            const float sc = pow2f_int(st.r - rM);
+            float t2 = sc * fmaf((st.m - M) * kLog2e, s_hi + s_lo, st.t2);
+            float sh = s_hi * sc, sl = s_lo * sc;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                float h, e;
+                two_sum(sh, __shfl_xor_sync(0xFFFFFFFFu, sh, off), h, e);
+                fast_two_sum(h, e + (sl + __shfl_xor_sync(0xFFFFFFFFu, sl, off)), sh, sl);
+                t2 += __shfl_xor_sync(0xFFFFFFFFu, t2, off);
+            }
+            int idx = INT32_MAX;
+#pragma unroll
+            for (int i = kVPL - 1; i >= 0; --i) {
+                const int vec = va + 32 * i;
+                const uint4 c = clamp_vec<DT>(aw[i]);
+#pragma unroll
+                for (int e = EPV - 1; e >= 0; --e)
+                    if (vec * EPV + e < p.V && vec_elem<DT>(c, e) == M) idx = vec * EPV + e;
+            }
+            idx = __reduce_min_sync(0xFFFFFFFFu, holds ? idx : INT32_MAX);
             if (FEAT && ent) {
                 if (lane == 0) {
                 FeatPartial fp;
@@ -630,13 +661,13 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
             }
             if (lane == 0) {
                 Partial pt;
-                pt.m = red.m;
-                pt.r = red.r;
-                pt.t2 = red.t2;
-                pt.sh = red.sh;
-                pt.sl = red.sl;
-                pt.amax = red.amax;
-                pt.rank = tok_bad ? -1 : red.rank;
+                pt.m = M;
+                pt.r = rM;
+                pt.t2 = t2;
+                pt.sh = sh;
+                pt.sl = sl;
+                pt.amax = idx;
+                pt.rank = tok_bad ? -1 : wrank;
                 pt.g = g;
                 p.partials[cc.r + gw] = pt;
             }
