@@ -277,9 +277,9 @@ __device__ __forceinline__ float process_tile(const uint4 *tile, int k0, int lan
 // which those five groups' maxima reach, so an entry outside them can only
 // tie the fifth largest entry.  While the piece streams, each lane keeps its
 // five largest tile maxima (order-preserving integer keys) with the tiles'
-// first vectors -- one compare per tile; at the piece's end the warp merges
-// the lanes' lists (five integer max reductions), re-reads the five groups
-// (40 vectors) from global memory and takes their five largest entries.
+// numbers; at the piece's end the warp merges the lanes' lists (five integer
+// max reductions), re-reads the five groups (40 vectors, in halves over the
+// lanes) from global memory and takes their five largest entries.
 __device__ __forceinline__ uint32_t fkey(float f) {
     const uint32_t u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
@@ -288,96 +288,101 @@ __device__ __forceinline__ float fkey_inv(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
 }
 
-// The lane's tile maximum cm of the tile starting at row vector k0 into its
-// list (ck descending, ct the tiles; key 0 = empty).
-__device__ __forceinline__ void group_update(float cm, int k0, uint32_t (&ck)[5], int (&ct)[5]) {
+// The lane's list: ck descending, 0 = empty.  bf16 logits (exact in the upper
+// half of a key): the key's upper half and, below it, the tile's number in the
+// piece -- 16 bits, as a piece is at most a sixteenth of a row of 2 GiB, or a
+// full grid's share of the device's memory (under 2^16 tiles of 4 KiB) -- so
+// that an insertion is five pairs of integer max and min and takes no branch
+// (~14 instructions a tile; with the tile numbers in registers of their own
+// the update took 81, as nearly every tile has a lane that inserts).  fp32:
+// the keys in ck, the tiles' numbers in ct.
+template <int DT>
+__device__ __forceinline__ void group_update(float cm, uint32_t tile, uint32_t (&ck)[5], uint32_t (&ct)[5]) {
+    if (DT == SDD_BF16) {
+        uint32_t key = (fkey(cm) & 0xFFFF0000u) | (tile & 0xFFFFu);
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            const uint32_t lo = min(ck[j], key);
+            ck[j] = max(ck[j], key);
+            key = lo;
+        }
+        return;
+    }
     uint32_t key = fkey(cm);
     if (key <= ck[4]) return;
-    int k = k0;
 #pragma unroll
     for (int j = 0; j < 5; ++j)
         if (key > ck[j]) {
-            const uint32_t tk = ck[j];
-            const int tt = ct[j];
+            const uint32_t tk = ck[j], tt = ct[j];
             ck[j] = key;
-            ct[j] = k;
+            ct[j] = tile;
             key = tk;
-            k = tt;
+            tile = tt;
         }
 }
 
 // The five largest clamped entries (descending; -inf where the piece has
 // fewer) of the piece [kb, ke) of row rowp, warp-uniform, from the lanes'
-// group lists.  The 40 vectors of the five groups are loaded (two per lane)
-// before `between` runs, so their round trip overlaps whatever it waits on.
-template <int DT, class Between>
+// group lists.
+template <int DT>
 __device__ __forceinline__ void group_top5(const char *rowp, int kb, int ke, int V, int lane, uint32_t (&ck)[5],
-                                           int (&ct)[5], float (&t)[5], Between between) {
+                                           uint32_t (&ct)[5], float (&t)[5]) {
     constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
     // (the rounds are rolled loops shifting their results in: this code runs
     // once per piece, and its instructions are fetched while L2 is busy)
-    int gl[5], gk[5];   // the five groups: lane and tile
+    int gv[5];   // the five groups' first vectors (-1: none)
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
-        gl[k] = 0;
-        gk[k] = -1;
+        gv[k] = -1;
         t[k] = -INFINITY;
     }
 #pragma unroll 1
     for (int k = 0; k < 5; ++k) {
-        const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, ck[0]);
+        const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, ck[0]);   // 0: every list is empty
         const int owner = __ffs(__ballot_sync(0xFFFFFFFFu, ck[0] == m)) - 1;
-        const int tile = __shfl_sync(0xFFFFFFFFu, ct[0], owner);   // -1 when every list is empty
+        const uint32_t tile = (DT == SDD_BF16) ? (m & 0xFFFFu) : __shfl_sync(0xFFFFFFFFu, ct[0], owner);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            gl[j] = gl[j + 1];
-            gk[j] = gk[j + 1];
-        }
-        gl[4] = owner;
-        gk[4] = tile;
+        for (int j = 0; j < 4; ++j) gv[j] = gv[j + 1];
+        gv[4] = (m != 0u) ? kb + static_cast<int>(tile) * kTileVec + owner : -1;
         if (lane == owner) {
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 ck[j] = ck[j + 1];
-                ct[j] = ct[j + 1];
+                if (DT != SDD_BF16) ct[j] = ct[j + 1];
             }
             ck[4] = 0u;
-            ct[4] = -1;
         }
     }
-    // vector u (0..39) of the groups: group u / 8, its (u % 8)-th vector;
-    // lane q takes u = q and u = q + 32
-    int vec[2];
-    uint4 w[2];
+    // half-vector u (0..79) of the groups: group u / 16, half u % 2 of its
+    // (u % 16) / 2-th vector; lane q takes u = q, q + 32 and q + 64
+    constexpr int HPV = EPV / 2;   // entries of a half-vector
+    int vec[3];
+    uint2 w[3];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int u = lane + 32 * h;
-        const int g = u >> 3, j = u & 7;
-        int gk_ = -1, gl_ = 0;
+    for (int h = 0; h < 3; ++h) {
+        const int u = lane + 32 * h, g = u >> 4;
+        int first = -1;
 #pragma unroll
         for (int k = 0; k < 5; ++k)
-            if (g == k) {
-                gk_ = gk[k];
-                gl_ = gl[k];
-            }
-        const int v = (gk_ >= 0) ? gk_ + gl_ + 32 * j : -1;
-        vec[h] = (u < 40 && v >= kb && v < ke) ? v : -1;
-        w[h] = (vec[h] >= 0) ? __ldg(reinterpret_cast<const uint4 *>(rowp) + vec[h]) : make_uint4(0, 0, 0, 0);
+            if (g == k) first = gv[k];
+        const int v = first + 32 * ((u & 15) >> 1);
+        vec[h] = (first >= 0 && v < ke) ? v : -1;
+        w[h] = (vec[h] >= 0) ? __ldg(reinterpret_cast<const uint2 *>(rowp) + 2 * vec[h] + (u & 1)) : make_uint2(0, 0);
     }
-    between();
-    float e[2 * EPV];
+    float e[3 * HPV];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const uint4 c = clamp_vec<DT>(w[h]);
+    for (int h = 0; h < 3; ++h) {
+        const uint4 c = clamp_vec<DT>(make_uint4(w[h].x, w[h].y, 0, 0));
+        const int first = vec[h] * EPV + ((lane & 1) ? HPV : 0);   // (u and the lane have the same parity)
 #pragma unroll
-        for (int j = 0; j < EPV; ++j)
-            e[h * EPV + j] = (vec[h] >= 0 && vec[h] * EPV + j < V) ? vec_elem<DT>(c, j) : -INFINITY;
+        for (int j = 0; j < HPV; ++j)
+            e[h * HPV + j] = (vec[h] >= 0 && first + j < V) ? vec_elem<DT>(c, j) : -INFINITY;
     }
 #pragma unroll 1
     for (int k = 0; k < 5; ++k) {   // five rounds: the warp's largest remaining entry
         float lm = e[0];
 #pragma unroll
-        for (int j = 1; j < 2 * EPV; ++j) lm = fmaxf(lm, e[j]);
+        for (int j = 1; j < 3 * HPV; ++j) lm = fmaxf(lm, e[j]);
         const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, fkey(lm));
 #pragma unroll
         for (int j = 0; j < 4; ++j) t[j] = t[j + 1];
@@ -386,8 +391,8 @@ __device__ __forceinline__ void group_top5(const char *rowp, int kb, int ke, int
         if (lane == owner) {
             bool done = false;
 #pragma unroll
-            for (int j = 0; j < 2 * EPV; ++j)
-                if (!done && fkey(e[j]) == m) {
+            for (int j = 0; j < 3 * HPV; ++j)
+                if (!done && e[j] == lm) {
                     e[j] = -INFINITY;
                     done = true;
                 }
@@ -531,7 +536,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
 
     SoftState st = soft_identity();
     uint32_t ck[5];        // FEAT: the lane's five largest tile maxima of the piece (keys) ...
-    int ct[5];             // ... and their tiles' first vectors (drafter rows)
+    uint32_t ct[5];        // ... fp32: their tiles' numbers in the piece (drafter rows)
     int kb = 0;            // FEAT: the piece's first vector in the row
     float s_hi = 0.f, s_lo = 0.f;   // the lane's exp-sum as an fp32 pair
     bool in_piece = false, fresh = false;   // fresh: the piece's token has not been fetched yet
@@ -552,7 +557,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
 #pragma unroll
                 for (int k = 0; k < 5; ++k) {
                     ck[k] = 0u;
-                    ct[k] = -1;
+                    ct[k] = 0u;
                 }
                 kb = cc.k;
             }
@@ -580,7 +585,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
         if (n < kTileVec || (row_end && tail)) pad_tile<DT>(tile, n, lane, row_end, tail);
         const float cm = ent ? process_tile<DT, true>(tile, cc.k, lane, st, s_hi, s_lo)
                              : process_tile<DT, false>(tile, cc.k, lane, st, s_hi, s_lo);
-        if (FEAT && ent) group_update(cm, cc.k, ck, ct);
+        if (FEAT && ent) group_update<DT>(cm, static_cast<uint32_t>(cc.k - kb) / kTileVec, ck, ct);
         if (fresh) {
             // the token's logit is first needed here: its load had the first
             // tile's copy and arithmetic to arrive
@@ -625,7 +630,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
                                               : make_uint4(0, 0, 0, 0);
             }
             float top[5];
-            if (FEAT && ent) group_top5<DT>(crow, kb, cc.k, p.V, lane, ck, ct, top, [] {});   // (cc.k: the piece's end)
+            if (FEAT && ent) group_top5<DT>(crow, kb, cc.k, p.V, lane, ck, ct, top);   // (cc.k: the piece's end)
             // every reference is a power of two below M's, so the rescaling is
             // exact; each step adds two lanes' double-floats the same way on
             // both, so all lanes agree
