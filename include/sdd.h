@@ -457,9 +457,10 @@ SDD_API sdd_status_t sdd_survival_mlp(const void *h, int M, int K, const void *W
  *   s    [M] fp32 output.
  *   workspace  device scratch of sdd_scorer_workspace_size(M) bytes, 16-byte
  *        aligned (receives the first layer's partials, then a2).
- * Two launches on the stream: the first layer (K split over a 4-CTA cluster as
- * in sdd_survival_mlp), then layers 2 and 3 and the head, a 4-CTA cluster per
- * 128 positions (each CTA 64 of the 256 columns of both layers).  Needs an
+ * Up to three launches on the stream: whole waves of 128-position tiles, one
+ * per SM, in one; for the tiles left over the first layer (K split over a
+ * cluster as in sdd_survival_mlp), then layers 2 and 3 and the head, a 4-CTA
+ * cluster per tile (each CTA 64 of the 256 columns of both layers).  Needs an
  * sm_10x device; a bounded wait that gives up sets SDD_DEV_TIMEOUT in *status.
  */
 SDD_API sdd_status_t sdd_scorer_deep(const void *h, int Kh, const void *f, int M, const void *W1, const float *b1,

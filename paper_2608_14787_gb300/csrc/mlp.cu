@@ -8,7 +8,8 @@
 //
 // and the scalar-feature block f of the deep scorer's input.
 //
-// First layer (mlp_kernel): a cluster of S = 4 CTAs per 128-row tile splits K;
+// Up to a quarter of the SMs' worth of 128-row tiles (a decode round's batch):
+// first layer (mlp_kernel): a cluster of S = 4 CTAs per 128-row tile splits K;
 // each CTA streams its K quarter through a four-stage ring of 48 KiB (A tile
 // 128 x 64, B tile 256 x 64, K-major, 128-byte swizzle) filled by 2D TMA, one
 // thread issues tcgen05.mma.kind::f16 (M = 128, N = 256, K = 16) into a
@@ -18,6 +19,9 @@
 // Layers 2-3 of the deep scorer (mlp_tail_kernel): a cluster of four CTAs per
 // tile, each computing 64 output columns of both layers, a2 through the
 // workspace and back by TMA.
+// Larger batches (mlp_plan): whole waves of one tile per SM run unsplit
+// (mlp_kernel with S = 1; the deep scorer all layers in one CTA,
+// mlp_deep_kernel), the tiles left over as above with S = 4 or 2.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -50,6 +54,11 @@ struct MlpParams {
     uint16_t *act;          // [M, 256] bf16 bits: GELU(W1 x + b1) (activation mode)
     float *ws;              // [tiles][S][256][128] fp32: partial accumulators (column-major per source CTA)
     int32_t *status;
+    int32_t tile0;          // the launch's first tile
+    // The launch follows another of the same layer over other tiles: it need
+    // not wait for that one to start, only to end (so that whatever waits for
+    // this launch has waited for both).
+    int32_t late_wait;
 };
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
@@ -156,6 +165,61 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 
 __device__ __forceinline__ float gelu_erf(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 
+// The first layer's main loop over K slices [kt0, kt0 + nk) of the tile at row
+// m0: warp 0 lane 0 fills the ring, warp 1 lane 0 issues the products into the
+// 256 TMEM columns at tmem; `done` completes with the accumulator.  The ring
+// is idle when both lanes have left (once `done` has completed).
+__device__ __forceinline__ void mlp_mainloop(unsigned char *smem, uint64_t *full, uint64_t *empty, uint64_t *done,
+                                             const CUtensorMap *tmA, const CUtensorMap *tmA2, const CUtensorMap *tmB,
+                                             int Ka, int m0, int kt0, int nk, uint32_t tmem, int *s_abort) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp == 0 && lane == 0) {
+        // TMA producer: stage s holds K slice kt0 + t of the A tile (rows
+        // m0..m0+127) and of the B tile (all 256 hidden units)
+        int t = 0;
+        for (; t < nk; ++t) {
+            const int s = t % kMlpStages;
+            const uint32_t ph = static_cast<uint32_t>(t / kMlpStages) & 1u;
+            if (t >= kMlpStages && !mbar_wait_bounded(&empty[s], ph ^ 1u, kWaitPolls)) {
+                *s_abort = 1;
+                break;
+            }
+            mbar_arrive_expect_tx(&full[s], kStageBytes);
+            const uint32_t a = smem_addr(smem + s * kStageBytes);
+            const int k = (kt0 + t) * kMlpBK;
+            if (k < Ka)
+                tma_load_2d(a, tmA, k, m0, smem_addr(&full[s]));
+            else
+                tma_load_2d(a, tmA2, k - Ka, m0, smem_addr(&full[s]));
+            tma_load_2d(a + kATileBytes, tmB, k, 0, smem_addr(&full[s]));
+        }
+        // let every issued load land before the ring is reused or the CTA
+        // leaves (already true unless a wait gave up): the last load per stage
+        for (int s = 0; s < kMlpStages && s < t; ++s) {
+            const int last = ((t - 1 - s) / kMlpStages) * kMlpStages + s;
+            (void)mbar_wait_bounded(&full[s], static_cast<uint32_t>(last / kMlpStages) & 1u, kWaitPolls);
+        }
+    } else if (warp == 1 && lane == 0) {
+        // MMA issuer: four K = 16 steps per stage, the 128-byte rows advanced
+        // by 32 bytes per step
+        for (int t = 0; t < nk; ++t) {
+            const int s = t % kMlpStages;
+            const uint32_t ph = static_cast<uint32_t>(t / kMlpStages) & 1u;
+            if (!mbar_wait_bounded(&full[s], ph, kWaitPolls)) {
+                *s_abort = 1;
+                break;
+            }
+            tc_fence_after();
+            const uint32_t a = smem_addr(smem + s * kStageBytes), b = a + kATileBytes;
+#pragma unroll
+            for (int kk = 0; kk < kMlpBK / 16; ++kk)
+                umma_f16(tmem, umma_desc_sw128(a + kk * 32), umma_desc_sw128(b + kk * 32), (t | kk) != 0 ? 1u : 0u);
+            umma_commit(smem_addr(&empty[s]));   // the stage is free once these MMAs have read it
+        }
+        umma_commit(smem_addr(done));            // the accumulator is complete
+    }
+}
+
 // Grid: (M tiles x S) CTAs in clusters of S along x (S = 1, 2 or 4 splits of
 // K).  CTA rank r of a cluster multiplies K slices [r nk/S, (r+1) nk/S) of its
 // 128-row tile into its own TMEM.  Columns [q W, (q+1) W) of the tile (W =
@@ -187,9 +251,10 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     __shared__ float s_b1[kMlpN], s_w2[kMlpN];   // epilogue constants, widened once per CTA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = (S > 1) ? cluster_rank() : 0u;
-    const int m0 = (blockIdx.x / S) * kMlpBM;
-    const int nk = p.K / kMlpBK / S;           // K slices of this CTA
-    const int kt0 = static_cast<int>(rank) * nk;
+    const int m0 = (p.tile0 + static_cast<int>(blockIdx.x) / S) * kMlpBM;
+    const int slices = p.K / kMlpBK;
+    const int kt0 = static_cast<int>(rank) * slices / S;                // K slices of this CTA
+    const int nk = (static_cast<int>(rank) + 1) * slices / S - kt0;
 
     if (tid == 0) {
         for (int s = 0; s < kMlpStages; ++s) {
@@ -209,7 +274,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     }
     // launched as a programmatic dependent: the setup above overlaps the end
     // of the work ahead in the stream; nothing is read before that completes
-    griddep_wait();
+    // (with late_wait the launch ahead waited for it before it let this start)
+    if (!p.late_wait) griddep_wait();
     for (int n = tid; n < kMlpN; n += kMlpThreads) {
         s_b1[n] = __ldg(p.b1 + n);
         s_w2[n] = HEAD ? __uint_as_float(static_cast<uint32_t>(__ldg(p.w2 + n)) << 16) : 0.f;
@@ -219,51 +285,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    if (warp == 0 && lane == 0) {
-        // TMA producer: stage s holds K slice kt0 + t of the A tile (rows
-        // m0..m0+127) and of the B tile (all 256 hidden units)
-        int t = 0;
-        for (; t < nk; ++t) {
-            const int s = t % kMlpStages;
-            const uint32_t ph = static_cast<uint32_t>(t / kMlpStages) & 1u;
-            if (t >= kMlpStages && !mbar_wait_bounded(&empty[s], ph ^ 1u, kWaitPolls)) {
-                s_abort = 1;
-                break;
-            }
-            mbar_arrive_expect_tx(&full[s], kStageBytes);
-            const uint32_t a = smem_addr(smem + s * kStageBytes);
-            const int k = (kt0 + t) * kMlpBK;
-            if (k < p.Ka)
-                tma_load_2d(a, &tmA, k, m0, smem_addr(&full[s]));
-            else
-                tma_load_2d(a, &tmA2, k - p.Ka, m0, smem_addr(&full[s]));
-            tma_load_2d(a + kATileBytes, &tmB, k, 0, smem_addr(&full[s]));
-        }
-        // let every issued load land before the ring is reused or the CTA
-        // leaves (already true unless a wait gave up): the last load per stage
-        for (int s = 0; s < kMlpStages && s < t; ++s) {
-            const int last = ((t - 1 - s) / kMlpStages) * kMlpStages + s;
-            (void)mbar_wait_bounded(&full[s], static_cast<uint32_t>(last / kMlpStages) & 1u, kWaitPolls);
-        }
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer: four K = 16 steps per stage, the 128-byte rows advanced
-        // by 32 bytes per step
-        for (int t = 0; t < nk; ++t) {
-            const int s = t % kMlpStages;
-            const uint32_t ph = static_cast<uint32_t>(t / kMlpStages) & 1u;
-            if (!mbar_wait_bounded(&full[s], ph, kWaitPolls)) {
-                s_abort = 1;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t a = smem_addr(smem + s * kStageBytes), b = a + kATileBytes;
-#pragma unroll
-            for (int kk = 0; kk < kMlpBK / 16; ++kk)
-                umma_f16(tmem, umma_desc_sw128(a + kk * 32), umma_desc_sw128(b + kk * 32), (t | kk) != 0 ? 1u : 0u);
-            umma_commit(smem_addr(&empty[s]));   // the stage is free once these MMAs have read it
-        }
-        umma_commit(smem_addr(done));            // the accumulator is complete
-    }
+    mlp_mainloop(smem, full, empty, done, &tmA, &tmA2, &tmB, p.Ka, m0, kt0, nk, tmem, &s_abort);
     __syncwarp();
 
     // Exchange through the workspace.  CTA q of the cluster finishes the
@@ -303,14 +325,14 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
             mbar_arrive_expect_tx(xfer, (S - 1) * kBlock);
             for (int r = 0; r < S; ++r)
                 if (r != static_cast<int>(rank))
-                    bulk_load(smem_addr(smem + r * kBlock),
+                    bulk_load(smem_addr(smem + (r - (r > static_cast<int>(rank) ? 1 : 0)) * kBlock),
                               ws_tile + (static_cast<int64_t>(r) * kMlpN + static_cast<int>(rank) * W) * kMlpBM, kBlock,
                               smem_addr(xfer));
         }
     }
     const bool okx = (S == 1) || __all_sync(0xFFFFFFFFu, mbar_wait_bounded(xfer, 0u, kWaitPolls));
     if (!okx) s_abort = 1;
-    const float *recv = reinterpret_cast<const float *>(smem);   // [S][W columns][128 rows]
+    const float *recv = reinterpret_cast<const float *>(smem);   // [S - 1 other CTAs][W columns][128 rows]
 
     // epilogue: z = the partials summed in rank order, then bias and GELU;
     // this warp's columns [rank W + part W / 4, + W / 4) of its 32 rows
@@ -321,25 +343,22 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
          c += 16) {
         uint32_t own[16];
         tmem_ld16_or0(ok, tbase + c, own);
-        float rem[S][16];
+        float g[16];   // the partials' sum, then the activations
 #pragma unroll
-        for (int r = 0; r < S; ++r)
-            if (r != static_cast<int>(rank)) {
-                const float *src = recv + (r * W + c - static_cast<int>(rank) * W) * kMlpBM + row;
+        for (int r = 0; r < S; ++r) {
+            const bool mine = r == static_cast<int>(rank);
+            const float *src = recv + ((r - (r > static_cast<int>(rank) ? 1 : 0)) * W + c - static_cast<int>(rank) * W) *
+                                          kMlpBM + row;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) rem[r][j] = src[j * kMlpBM];
+            for (int j = 0; j < 16; ++j) {
+                const float x = mine ? __uint_as_float(own[j]) : src[j * kMlpBM];
+                g[j] = (r == 0) ? x : g[j] + x;
             }
-        float g[16];
+        }
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-            float z = 0.f;
-#pragma unroll
-            for (int r = 0; r < S; ++r) {
-                const float x = (r == static_cast<int>(rank)) ? __uint_as_float(own[j]) : rem[r][j];
-                z = (r == 0) ? x : z + x;
-            }
             const int n = c + j;
-            g[j] = gelu_erf(z + s_b1[n]);
+            g[j] = gelu_erf(g[j] + s_b1[n]);
             if (HEAD) t2 = fmaf(s_w2[n], g[j], t2);
         }
         if (!HEAD && ok && grow < p.M) {
@@ -381,6 +400,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     __syncthreads();
     if (tid == 0 && s_abort) status_or(p.status, SDD_DEV_TIMEOUT);
     if (S > 1 && tid == 0 && !okx) (void)mbar_wait_bounded(xfer, 0u, kWaitPolls);   // copies still in flight
+    if (p.late_wait) griddep_wait();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
@@ -407,12 +427,16 @@ constexpr uint32_t kTailWSlice = kTailN * kMlpBK * 2;      // 8 KiB: 64 rows x 6
 constexpr int kTailSlices = kMlpN / kMlpBK;                // 4
 constexpr uint32_t kTailA = kTailSlices * kTailASlice;     // 64 KiB
 constexpr uint32_t kTailW = kTailSlices * kTailWSlice;     // 32 KiB
-constexpr int kTailSmem = kTailA + 2 * kTailW + 1024 + 256;
+// PAIR: W3 takes W2's place, so that two CTAs share an SM (launches of more
+// CTAs than SMs: one's round trips run under the other's epilogue); otherwise
+// both are loaded ahead.
+constexpr int tail_smem(bool pair) { return static_cast<int>(kTailA + (pair ? 1 : 2) * kTailW) + 1024 + 256; }
 constexpr uint32_t kTailTmemCols = 128;
 constexpr int kTailThreads = 512;   // 16 warps: four per TMEM lane quarter, 16 columns each
 
 struct TailParams {
     int32_t M;
+    int32_t tile0;          // the launch's first tile
     const float *b2, *b3;   // [256]
     const uint16_t *w4;     // [256] bf16 bits
     float b4;
@@ -421,7 +445,8 @@ struct TailParams {
     int32_t *status;
 };
 
-__global__ void __launch_bounds__(kTailThreads, 1) mlp_tail_kernel(const __grid_constant__ CUtensorMap tmAct,
+template <bool PAIR>
+__global__ void __launch_bounds__(kTailThreads, PAIR ? 2 : 1) mlp_tail_kernel(const __grid_constant__ CUtensorMap tmAct,
                                                                  const __grid_constant__ CUtensorMap tmW2,
                                                                  const __grid_constant__ CUtensorMap tmW3,
                                                                  const __grid_constant__ CUtensorMap tmAct2,
@@ -429,8 +454,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) mlp_tail_kernel(const __grid_
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                             ~static_cast<uintptr_t>(1023));
-    unsigned char *bufA = smem, *bufW2 = smem + kTailA, *bufW3 = smem + kTailA + kTailW;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(smem + kTailA + 2 * kTailW);
+    unsigned char *bufA = smem, *bufW2 = smem + kTailA;   // a1, then a2; W2
+    unsigned char *bufW3 = PAIR ? bufW2 : bufW2 + kTailW;
+    uint64_t *bar = reinterpret_cast<uint64_t *>(bufW3 + kTailW);
     uint64_t *fullA = bar, *fullW2 = bar + 1, *fullW3 = bar + 2, *mma2 = bar + 3, *mma3 = bar + 4, *fullA2 = bar + 5;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar + 6);
     __shared__ int s_abort;
@@ -439,7 +465,7 @@ __global__ void __launch_bounds__(kTailThreads, 1) mlp_tail_kernel(const __grid_
     __shared__ float s_head[kTailCluster][kMlpBM];  // (CTA 0) each CTA's dot product of each row
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t rank = cluster_rank();
-    const int m0 = (blockIdx.x / kTailCluster) * kMlpBM;
+    const int m0 = (p.tile0 + static_cast<int>(blockIdx.x) / kTailCluster) * kMlpBM;
     const int n0 = static_cast<int>(rank) * kTailN;
     for (int n = tid; n < kTailN; n += kTailThreads) {
         s_b2[n] = __ldg(p.b2 + n0 + n);
@@ -462,14 +488,17 @@ __global__ void __launch_bounds__(kTailThreads, 1) mlp_tail_kernel(const __grid_
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    auto load_w3 = [&] {
+        mbar_arrive_expect_tx(fullW3, kTailW);
+        for (int c = 0; c < kTailSlices; ++c)
+            tma_load_2d(smem_addr(bufW3 + c * kTailWSlice), &tmW3, c * kMlpBK, n0, smem_addr(fullW3));
+    };
     if (tid == 0) {
         // the weights do not depend on the first layer: loaded while it finishes
         mbar_arrive_expect_tx(fullW2, kTailW);
         for (int c = 0; c < kTailSlices; ++c)
             tma_load_2d(smem_addr(bufW2 + c * kTailWSlice), &tmW2, c * kMlpBK, n0, smem_addr(fullW2));
-        mbar_arrive_expect_tx(fullW3, kTailW);
-        for (int c = 0; c < kTailSlices; ++c)
-            tma_load_2d(smem_addr(bufW3 + c * kTailWSlice), &tmW3, c * kMlpBK, n0, smem_addr(fullW3));
+        if (!PAIR) load_w3();
     }
     // launched as a programmatic dependent of the first layer: a1 (and the
     // workspace, which a2 overwrites) only once that grid has completed
@@ -503,6 +532,9 @@ __global__ void __launch_bounds__(kTailThreads, 1) mlp_tail_kernel(const __grid_
     const uint32_t tlane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(mma2, 0u, kWaitPolls));
     tc_fence_after();
+    // layer 2's products have read W2: W3 into its place, under the epilogue
+    const bool w3_issued = !PAIR || ok;   // (thread 0's)
+    if (PAIR && tid == 0 && ok) load_w3();
     {
         uint32_t v[16];
         tmem_ld16_or0(ok, tlane + part * 16, v);
@@ -567,11 +599,182 @@ __global__ void __launch_bounds__(kTailThreads, 1) mlp_tail_kernel(const __grid_
                                                 s_head[3][row]) + p.b4)));
     if (tid == 0) {
         // every load this CTA issued has landed before its shared memory goes away
-        for (int i : {0, 1, 2, 5}) (void)mbar_wait_bounded(&bar[i], 0u, kWaitPolls);
+        for (int i : {0, 1, 5}) (void)mbar_wait_bounded(&bar[i], 0u, kWaitPolls);
+        if (w3_issued) (void)mbar_wait_bounded(fullW3, 0u, kWaitPolls);
         if (s_abort || !ok) status_or(p.status, SDD_DEV_TIMEOUT);
     }
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTailTmemCols)
+                     : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// The deep scorer of one 128-row tile in one CTA (whole waves of tiles): the
+// first layer with K not split, then layers 2 and 3 and the head without a1,
+// a2 or partial sums leaving the SM.  After the main loop the ring's 192 KiB
+// hold the activations (64 KiB, written by the epilogues in the operands'
+// swizzled layout) and one 256 x 256 weight matrix (128 KiB: W2 as soon as the
+// main loop's products have read the ring, W3 once layer 2's have read W2,
+// each under the epilogue before it).  TMEM columns 0-255 hold z1, 256-511 z2,
+// 0-255 z3.  a1 is also written to p.act.
+//
+// Bound by the main loop's operands (2.9 MB into each SM, ~22 us) and then by
+// the issue of 3 x 32 K erf-form GELUs an SM.  GB300, K = 3584 + 256: 50.9 us
+// for 128 tiles (16,384 rows) against 93.8 us with K split four ways, clusters
+// of four and a second launch for the tail (61.4 us with K not split and the
+// tail in a second launch); 20,000 rows 69.3 against 116 us.
+// ---------------------------------------------------------------------------
+struct DeepParams {
+    int32_t M, K, Ka, tile0;
+    const float *b1, *b2, *b3;   // [256]
+    const uint16_t *w4;          // [256] bf16 bits
+    float b4;
+    uint16_t *act;               // [M, 256] bf16 bits: a1
+    float *out;                  // [M]
+    int32_t *status;
+};
+constexpr uint32_t kDeepW = 4u * kBTileBytes;   // 128 KiB: a 256 x 256 bf16 matrix, four 64-column slices
+static_assert(kTailA + kDeepW == kMlpStages * kStageBytes, "activations and weights share the ring");
+
+// Address of the 16-byte chunk of columns 8 c8 .. 8 c8 + 7 of a row in the
+// swizzled activations (64-column slices of 128 rows x 128 bytes).
+__device__ __forceinline__ unsigned char *act_chunk(unsigned char *buf, int row, int c8) {
+    return buf + (c8 >> 3) * kTailASlice + row * 128 + (((c8 & 7) ^ (row & 7)) << 4);
+}
+
+__global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_constant__ CUtensorMap tmA,
+                                                                 const __grid_constant__ CUtensorMap tmA2,
+                                                                 const __grid_constant__ CUtensorMap tmB,
+                                                                 const __grid_constant__ CUtensorMap tmW2,
+                                                                 const __grid_constant__ CUtensorMap tmW3,
+                                                                 const __grid_constant__ DeepParams p) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
+                                                            ~static_cast<uintptr_t>(1023));
+    unsigned char *bufA = smem, *bufW = smem + kTailA;
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kMlpStages * kStageBytes);
+    uint64_t *empty = full + kMlpStages;
+    uint64_t *done = empty + kMlpStages;   // z1, then z2, z3
+    uint64_t *fullW = done + 3;            // W2, W3
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fullW + 2);
+    __shared__ int s_abort;
+    __shared__ float s_b[3][kMlpN], s_w4[kMlpN];
+    __shared__ float s_part[3][kMlpBM];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = (p.tile0 + static_cast<int>(blockIdx.x)) * kMlpBM;
+
+    if (tid == 0) {
+        for (int i = 0; i < 2 * kMlpStages + 5; ++i) mbar_init(&full[i], 1);
+        fence_mbar_init();
+        s_abort = 0;
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
+                     "r"(2 * kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    griddep_wait();
+    for (int n = tid; n < kMlpN; n += kMlpThreads) {
+        s_b[0][n] = __ldg(p.b1 + n);
+        s_b[1][n] = __ldg(p.b2 + n);
+        s_b[2][n] = __ldg(p.b3 + n);
+        s_w4[n] = __uint_as_float(static_cast<uint32_t>(__ldg(p.w4 + n)) << 16);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    mlp_mainloop(smem, full, empty, done, &tmA, &tmA2, &tmB, p.Ka, m0, 0, p.K / kMlpBK, tmem, &s_abort);
+    __syncwarp();
+
+    // warp w: TMEM lanes 32 (w % 4) .. + 31 (tile rows), columns 64 (w / 4) .. + 63
+    const int quarter = warp & 3, part = warp >> 2;
+    const int row = quarter * 32 + lane, grow = m0 + row;
+    const uint32_t tlane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    bool ok = true;
+    float t = 0.f;   // this thread's part of the head's dot product
+    int w_issued = 0;
+#pragma unroll 1
+    for (int layer = 0; layer < 3; ++layer) {
+        // z of this layer is complete, and its products have read their operands
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&done[layer], 0u, kWaitPolls)) && ok;
+        tc_fence_after();
+        if (!ok) s_abort = 1;
+        if (layer == 0) {
+            // (every warp: a CTA's threads have all passed the main loop)
+            __syncthreads();   // the producer has left the ring
+            griddep_launch_dependents();
+        }
+        if (tid == 0 && layer < 2 && ok) {
+            mbar_arrive_expect_tx(&fullW[layer], kDeepW);
+            for (int c = 0; c < kTailSlices; ++c)
+                tma_load_2d(smem_addr(bufW + c * kBTileBytes), layer == 0 ? &tmW2 : &tmW3, c * kMlpBK, 0,
+                            smem_addr(&fullW[layer]));
+            w_issued = layer + 1;
+        }
+        const uint32_t z = tlane + (layer == 1 ? kTmemCols : 0u) + part * 64;
+        const float *bias = s_b[layer];
+#pragma unroll 1
+        for (int c = 0; c < 64; c += 16) {
+            uint32_t v[16];
+            tmem_ld16_or0(ok, z + c, v);
+            float g[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) g[j] = gelu_erf(__uint_as_float(v[j]) + bias[part * 64 + c + j]);
+            if (layer == 2) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) t = fmaf(s_w4[part * 64 + c + j], g[j], t);
+                continue;
+            }
+            uint32_t w[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) w[q] = pack_bf16x2(g[2 * q], g[2 * q + 1]);
+            const int c8 = part * 8 + (c >> 3);
+            *reinterpret_cast<uint4 *>(act_chunk(bufA, row, c8)) = make_uint4(w[0], w[1], w[2], w[3]);
+            *reinterpret_cast<uint4 *>(act_chunk(bufA, row, c8 + 1)) = make_uint4(w[4], w[5], w[6], w[7]);
+            if (layer == 0 && ok && grow < p.M) {
+                uint4 *dst = reinterpret_cast<uint4 *>(p.act + static_cast<int64_t>(grow) * kMlpN + part * 64 + c);
+                dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+            }
+        }
+        if (layer == 2) break;
+        fence_proxy_async_smem();   // the activations, before the tensor cores read them
+        tc_fence_before();
+        __syncthreads();
+        if (warp == 1 && lane == 0) {
+            tc_fence_after();
+            if (ok && mbar_wait_bounded(&fullW[layer], 0u, kWaitPolls)) {
+                const uint32_t d = tmem + (layer == 0 ? kTmemCols : 0u);
+#pragma unroll 1
+                for (int c = 0; c < kTailSlices; ++c)
+#pragma unroll
+                    for (int kk = 0; kk < kMlpBK / 16; ++kk)
+                        umma_f16(d, umma_desc_sw128(smem_addr(bufA + c * kTailASlice) + kk * 32),
+                                 umma_desc_sw128(smem_addr(bufW + c * kBTileBytes) + kk * 32),
+                                 (c | kk) != 0 ? 1u : 0u);
+            } else {
+                s_abort = 1;
+            }
+            umma_commit(smem_addr(&done[layer + 1]));   // (arrives at once when nothing was issued)
+        }
+        __syncwarp();
+    }
+    if (part > 0) s_part[part - 1][row] = t;
+    tc_fence_before();
+    __syncthreads();
+    if (part == 0 && ok && grow < p.M) {
+        t = ((t + s_part[0][row]) + s_part[1][row]) + s_part[2][row];
+        p.out[grow] = 1.f / (1.f + expf(-(t + p.b4)));
+    }
+    if (tid == 0) {
+        // every weight load has landed before the shared memory goes away
+        for (int i = 0; i < w_issued; ++i) (void)mbar_wait_bounded(&fullW[i], 0u, kWaitPolls);
+        if (s_abort) status_or(p.status, SDD_DEV_TIMEOUT);
+    }
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * kTmemCols)
                      : "memory");
 }
 
@@ -610,7 +813,7 @@ struct MapCache {
         int K, box;
         CUtensorMap map;
     };
-    static constexpr int kSlots = 8;
+    static constexpr int kSlots = 16;
     Entry e[kSlots];
     int n = 0, next = 0;
     std::mutex mu;
@@ -631,27 +834,59 @@ struct MapCache {
 MapCache g_maps;
 constexpr int kMaxDevices = 64;
 std::atomic<int> g_attr_ready[kMaxDevices];
+std::atomic<int> g_sms[kMaxDevices];
 
 // Per-device opt-in of every kernel here to its dynamic shared memory.
-cudaError_t mlp_prepare() {
+cudaError_t mlp_prepare(int *sm_count) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (g_attr_ready[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    if (g_attr_ready[dev].load(std::memory_order_acquire)) {
+        *sm_count = g_sms[dev].load(std::memory_order_relaxed);
+        return cudaSuccess;
+    }
     for (auto fn : {mlp_kernel<1, true>, mlp_kernel<2, true>, mlp_kernel<4, true>, mlp_kernel<1, false>,
                     mlp_kernel<2, false>, mlp_kernel<4, false>}) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
         if (e != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(mlp_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmem);
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    g_sms[dev].store(sms, std::memory_order_relaxed);
+    e = cudaFuncSetAttribute(mlp_tail_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem(false));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mlp_tail_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem(true));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_deep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
     if (e != cudaSuccess) return e;
     g_attr_ready[dev].store(1, std::memory_order_release);
+    *sm_count = sms;
     return cudaSuccess;
 }
 
+// How M rows' tiles are run: `full` of them, whole waves of one tile per SM,
+// with K not split (no operand read twice, nothing exchanged), and the `rest`
+// after them with K split S ways, as far as the SMs reach (one wave again; a
+// wave with S = 4, 2, 1 takes 13.5, 18.4 and 33.7 us at K = 3584).  A rest of
+// more than half the SMs runs unsplit too (it is then part of `full`).  GB300,
+// one-layer scorer, K = 3584, against all tiles split four ways: 8,192 rows
+// 18.4 / 26.4 us, 12,000 25.2 / 43.7, 16,384 33.7 / 58.0, 20,000 43.6 / 71.9,
+// 32,768 65.8 / 111.7.
+struct MlpPlan {
+    int full, rest, S;
+};
+MlpPlan mlp_plan(int M, int K, int sms) {
+    const int tiles = (M + kMlpBM - 1) / kMlpBM, nk = K / kMlpBK;
+    MlpPlan q{tiles / sms * sms, tiles % sms, 1};
+    if (q.rest > 0) q.S = (4 * q.rest <= sms && nk >= 4) ? 4 : (2 * q.rest <= sms && nk >= 2) ? 2 : 1;
+    if (q.S == 1) q = MlpPlan{tiles, 0, 1};
+    return q;
+}
+
 // The first layer: A = [A1 | A2] (A2 may be absent: Ka = K), W1 [256, K].
-// head: fused GELU / w2 / sigmoid into out; else bf16 activations into act.
+// head: fused GELU / w2 / sigmoid into out; else bf16 activations into act, of
+// the plan's rest only (its whole waves are mlp_deep_kernel's).
 cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, const void *W1, const float *b1,
                           const void *w2, float b2, float *out, uint16_t *act, bool head, float *ws, int32_t *status,
                           cudaStream_t stream, const char **why) {
@@ -661,11 +896,9 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
         *why = "cuTensorMapEncodeTiled failed";
         return cudaErrorInvalidValue;
     }
-    cudaError_t e = mlp_prepare();
+    int sms = 0;
+    cudaError_t e = mlp_prepare(&sms);
     if (e != cudaSuccess) return e;
-    // split K four ways when the slices divide evenly (more SMs, no reloads)
-    const int nk = K / kMlpBK;
-    const int S = (nk % 4 == 0 && nk >= 8) ? 4 : (nk % 2 == 0 && nk >= 4) ? 2 : 1;
     MlpParams p;
     p.M = M;
     p.K = K;
@@ -677,28 +910,35 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
     p.act = act;
     p.ws = ws;
     p.status = status;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(((M + kMlpBM - 1) / kMlpBM) * S);
-    cfg.blockDim = dim3(kMlpThreads);
-    cfg.dynamicSmemBytes = kMlpSmem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = S;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // setup overlaps the work ahead
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    if (head) {
-        if (S == 4) return cudaLaunchKernelEx(&cfg, mlp_kernel<4, true>, tmA, tmA2, tmB, p);
-        if (S == 2) return cudaLaunchKernelEx(&cfg, mlp_kernel<2, true>, tmA, tmA2, tmB, p);
-        return cudaLaunchKernelEx(&cfg, mlp_kernel<1, true>, tmA, tmA2, tmB, p);
+    // Tiles [t0, t0 + n) with K split S ways.
+    auto launch = [&](int t0, int n, int S, bool late) {
+        p.tile0 = t0;
+        p.late_wait = late ? 1 : 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(n * S);
+        cfg.blockDim = dim3(kMlpThreads);
+        cfg.dynamicSmemBytes = kMlpSmem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[2];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = S;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // setup overlaps the work ahead
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 2;
+        const auto kernel = S == 4   ? (head ? mlp_kernel<4, true> : mlp_kernel<4, false>)
+                            : S == 2 ? (head ? mlp_kernel<2, true> : mlp_kernel<2, false>)
+                                     : (head ? mlp_kernel<1, true> : mlp_kernel<1, false>);
+        return cudaLaunchKernelEx(&cfg, kernel, tmA, tmA2, tmB, p);
+    };
+    const MlpPlan plan = mlp_plan(M, K, sms);
+    if (head && plan.full > 0) {
+        e = launch(0, plan.full, 1, false);
+        if (e != cudaSuccess) return e;
     }
-    if (S == 4) return cudaLaunchKernelEx(&cfg, mlp_kernel<4, false>, tmA, tmA2, tmB, p);
-    if (S == 2) return cudaLaunchKernelEx(&cfg, mlp_kernel<2, false>, tmA, tmA2, tmB, p);
-    return cudaLaunchKernelEx(&cfg, mlp_kernel<1, false>, tmA, tmA2, tmB, p);
+    return plan.rest > 0 ? launch(plan.full, plan.rest, plan.S, plan.full > 0) : cudaSuccess;
 }
 
 }  // namespace
@@ -722,8 +962,47 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
                                const char **why) {
     *why = nullptr;
     if (M == 0) return cudaSuccess;
-    cudaError_t e = launch_layer1(h, Kh, f, M, Kh + kMlpN, W1, b1, nullptr, 0.f, nullptr, act, false,
-                                  static_cast<float *>(ws), status, stream, why);
+    int sms = 0;
+    cudaError_t e = mlp_prepare(&sms);
+    if (e != cudaSuccess) return e;
+    const int K = Kh + kMlpN;
+    const MlpPlan plan = mlp_plan(M, K, sms);
+    if (plan.full > 0) {
+        CUtensorMap tmA, tmA2, tmB, tmW2, tmW3;
+        if (!g_maps.get(&tmA, h, M, Kh, kMlpBM) || !g_maps.get(&tmA2, f, M, kMlpN, kMlpBM) ||
+            !g_maps.get(&tmB, W1, kMlpN, K, kMlpN) || !g_maps.get(&tmW2, W2, kMlpN, kMlpN, kMlpN) ||
+            !g_maps.get(&tmW3, W3, kMlpN, kMlpN, kMlpN)) {
+            *why = "cuTensorMapEncodeTiled failed";
+            return cudaErrorInvalidValue;
+        }
+        DeepParams d;
+        d.M = M;
+        d.K = K;
+        d.Ka = Kh;
+        d.tile0 = 0;
+        d.b1 = b1;
+        d.b2 = b2;
+        d.b3 = b3;
+        d.w4 = static_cast<const uint16_t *>(w4);
+        d.b4 = b4;
+        d.act = act;
+        d.out = out;
+        d.status = status;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(plan.full);
+        cfg.blockDim = dim3(kMlpThreads);
+        cfg.dynamicSmemBytes = kMlpSmem;
+        cfg.stream = stream;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelEx(&cfg, mlp_deep_kernel, tmA, tmA2, tmB, tmW2, tmW3, d);
+        if (e != cudaSuccess || plan.rest == 0) return e;
+    }
+    e = launch_layer1(h, Kh, f, M, K, W1, b1, nullptr, 0.f, nullptr, act, false, static_cast<float *>(ws), status,
+                      stream, why);
     if (e != cudaSuccess || *why) return e;
     const int64_t rows_pad = ((static_cast<int64_t>(M) + kMlpBM - 1) / kMlpBM) * kMlpBM;
     CUtensorMap tmAct, tmW2, tmW3, tmAct2;
@@ -732,8 +1011,10 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
         *why = "cuTensorMapEncodeTiled failed";
         return cudaErrorInvalidValue;
     }
+    const bool pair = plan.rest * kTailCluster > sms;
     TailParams p;
     p.M = M;
+    p.tile0 = plan.full;
     p.b2 = b2;
     p.b3 = b3;
     p.w4 = static_cast<const uint16_t *>(w4);
@@ -742,9 +1023,9 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
     p.out = out;
     p.status = status;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(((M + kMlpBM - 1) / kMlpBM) * kTailCluster);
+    cfg.gridDim = dim3(plan.rest * kTailCluster);
     cfg.blockDim = dim3(kTailThreads);
-    cfg.dynamicSmemBytes = kTailSmem;
+    cfg.dynamicSmemBytes = tail_smem(pair);
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -755,7 +1036,7 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, mlp_tail_kernel, tmAct, tmW2, tmW3, tmAct2, p);
+    return cudaLaunchKernelEx(&cfg, pair ? mlp_tail_kernel<true> : mlp_tail_kernel<false>, tmAct, tmW2, tmW3, tmAct2, p);
 }
 
 // ---------------------------------------------------------------------------

@@ -1,0 +1,44 @@
+"""The scorers where their launch changes shape: batches just inside and past
+one CTA per SM (38 tiles of 128 rows on 152 SMs) and of several waves with a
+ragged last tile, and K whose slices of 64 do not divide by four (and under
+four of them), against fp64.  Tolerances as derived in the scorers' own tests."""
+import pytest
+import torch
+
+from paper_2608_14787_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _gelu(z):
+    return 0.5 * z * (1 + torch.erf(z / 2 ** 0.5))
+
+
+@pytest.mark.parametrize("M,K", [(38 * 128, 512), (38 * 128 + 1, 512), (76 * 128 - 5, 448), (20001, 320), (700, 192),
+                                 (20001, 64), (300, 3520)])
+def test_mlp(sdd, M, K):
+    W1, b1, w2, b2 = synth.make_mlp(device="cuda", hidden=K)
+    h = synth.make_hidden(M, device="cuda", seed=3, hidden=K)
+    status = sdd.new_status()
+    s = sdd.survival_mlp(h, W1, b1, w2, float(b2), status=status)
+    again = sdd.survival_mlp(h, W1, b1, w2, float(b2), status=status)
+    want = torch.sigmoid(_gelu(h.double() @ W1.double().T + b1.double()) @ w2.double() + b2.double())
+    assert int(status.item()) == 0 and torch.equal(s, again)
+    torch.testing.assert_close(s.double(), want, rtol=0, atol=5e-5)
+
+
+@pytest.mark.parametrize("M,Kh", [(38 * 128, 256), (38 * 128 + 1, 256), (12345, 192), (20001, 64), (20001, 704)])
+def test_deep(sdd, M, Kh):
+    w = synth.make_scorer_deep(device="cuda", hidden=Kh)
+    W1, b1, W2, b2, W3, b3, w4, b4 = w
+    h = synth.make_hidden(M, device="cuda", seed=5, hidden=Kh)
+    f = synth.make_features(M, device="cuda")
+    status = sdd.new_status()
+    s = sdd.scorer_deep(h, f, *w, status=status)
+    again = sdd.scorer_deep(h, f, *w, status=status)
+    u = torch.cat([h, f], 1).double()
+    for W, b in ((W1, b1), (W2, b2), (W3, b3)):
+        u = _gelu(u @ W.double().T + b.double())
+    want = torch.sigmoid(u @ w4.double() + b4)
+    assert int(status.item()) == 0 and torch.equal(s, again)
+    torch.testing.assert_close(s.double(), want, rtol=0, atol=3e-4)
