@@ -12,11 +12,15 @@
 // accepted, p_t of the bonus row: each team sums its segment of the draw row
 // and publishes its per-thread prefix sums; the last to finish (atomic
 // arrival, no waiting) locates the segment, then the thread, from those sums,
-// and searches that thread's run with one warp.  Last, every other rule
-// (lenience, top-k; greedy strict), the skip schedule and the agreement
-// counters, one warp per rule or threshold pair, shared round robin by the
-// block's segment teams under the sampling rule; the segment-0 team writes
-// the commits.
+// and searches that thread's run with one warp.  Every other rule (lenience,
+// top-k; greedy strict), the skip schedule and the agreement counters go one
+// warp per rule or threshold pair, shared round robin by the block's segment
+// teams under the sampling rule -- in the last team to arrive beside the warp
+// that locates the draw; the segment-0 team writes the commits of skipped
+// blocks.  GB300, decide kernel of one 32 x 151,936 bf16 block 12.6 -> 11.6 us,
+// of one 8 x 32,000 fp32 block 10.4 -> 9.5 us against those tasks after the
+// draw, pair 0's schedule ahead of it and the partials' owners computed for
+// rows of whole pieces.
 #pragma once
 
 #include "rules.cuh"
@@ -677,6 +681,61 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
     if (!dec) return;
     const bool sched = d.do_sched && has_d;
 
+    // The tasks that follow from the facts, a warp each.  Rule r > 0 (lenience,
+    // top-k):
+    const int R = 1 + d.n_ell + d.n_k;
+    auto rule_task = [&](int r) {
+        const int L = rule_first_reject(d, F, r, b, lane);
+        const int corr = F.t_am[L];   // target argmax at the first rejection, or of the bonus row
+        const bool len = r <= d.n_ell;
+        const int64_t o = static_cast<int64_t>(len ? r - 1 : r - 1 - d.n_ell) * p.B + b;
+        int32_t *Lo = len ? d.L_len : d.L_topk, *no = len ? d.n_len : d.n_topk;
+        int32_t *to = len ? d.tok_len : d.tok_topk;
+        if (lane == 0) {
+            if (Lo) Lo[o] = L;
+            if (no) no[o] = L + 1;
+        }
+        if (to) write_tokens(lane, gamma, to + o * (gamma + 1), F.x, L, corr);
+    };
+    // Threshold pair t's schedule and, with `write`, its outputs and agreement
+    // counters (strict L in s_L[0]); pair 0's K also goes to s_K0:
+    auto pair_task = [&](int t, bool write) {
+        int Kh, K, Do;
+        sched_pair(d, F, t, s_force != 0, s_D, lane, Kh, K, Do);
+        if (lane == 0 && t == 0) s_K0 = K;
+        if (lane == 0 && write) {
+            const int64_t o = static_cast<int64_t>(t) * p.B + b;
+            if (d.K_hat) d.K_hat[o] = Kh;
+            if (d.K) d.K[o] = K;
+            if (d.D_out) d.D_out[o] = Do;
+            if (d.agreement && K > 0 && d.do_strict) {
+                const int L = s_L[0];
+                unsigned long long *a = reinterpret_cast<unsigned long long *>(d.agreement + 4 * t);
+                atomicAdd(a + 0, static_cast<unsigned long long>(min(K, L)));
+                atomicAdd(a + 1, static_cast<unsigned long long>(K));
+                atomicAdd(a + 2, static_cast<unsigned long long>(K <= L ? 1 : 0));
+                atomicAdd(a + 3, 1ull);
+            }
+        }
+    };
+    // Under the sampling rule the block's draw segments share the tasks round
+    // robin (every team holds the block's facts): rule r goes to team r mod
+    // nseg, pair t to team (R + t) mod nseg.  This team's share by its warps
+    // w of nw; k0: also pair 0's K into s_K0 (the teams that write commits).
+    auto tasks = [&](int w, int nw, bool k0) {
+        const int extra = (sched && k0) ? 1 : 0;
+#pragma unroll 1
+        for (int i = w;; i += nw) {
+            const int task = seg + (i - extra) * nseg;   // rules, then pairs
+            const bool own = i >= extra;
+            if (own && task >= R + (sched ? d.n_tau : 0)) break;
+            if (!own || task >= R)
+                pair_task(own ? task - R : 0, own);
+            else if (task > 0)   // (rule 0, strict, is the draw's)
+                rule_task(task);
+        }
+    };
+
     if (sampling) {
         // ---- phase 2 (every CTA): the strict accepted length L ----
         if (warp == 0) {
@@ -685,7 +744,7 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
                 s_L[0] = L;
                 s_corr[0] = F.t_am[L];
             }
-        } else if (warp == 1 && sched) {
+        } else if (SHARD && warp == 1 && sched) {
             // pair 0 decides whether this block commits its verified tokens
             int Kh, K, Do;
             sched_pair(d, F, 0, s_force != 0, s_D, lane, Kh, K, Do);
@@ -829,22 +888,30 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
             }
             dec_sync<NT>();
         }
+        float u = 0.f;   // the draw's uniform (warp 0 of the last to arrive)
         if (s_is_last) {
             // the last segment to arrive completes the draw: every segment's
             // prefixes in one round trip (a segment's total is its last prefix)
             const float4 *src =
                 reinterpret_cast<const float4 *>(d.res_pref + static_cast<int64_t>(i) * nseg * NT);
             for (int q = tid; q < nseg * (NT / 4); q += NT) cp_async16(s_pref_all + 4 * q, src + q);
+            const uint32_t jj = (L < gamma) ? static_cast<uint32_t>(L + 1) : static_cast<uint32_t>(gamma + 1);
+            if (warp == 0)
+                u = philox_uniform(d.seed, jj, static_cast<uint32_t>(b), d.round,
+                                   (L < gamma) ? kPurposeResid : kPurposeBonus);
             cp_async_wait_all();
             dec_sync<NT>();
+        }
+        // this team's tasks; in the last to arrive beside warp 0, which locates
+        // the draw (each was 0.7 us of that team's time after it)
+        const bool last = s_is_last != 0;
+        if (!last || warp > 0) tasks(last ? warp - 1 : warp, last ? NW - 1 : NW, last || leader);
+        if (last) {
             if (warp == 0) {
                 // R = sum of the segment totals and their inclusive prefix sums
                 // (double-floats); the first segment whose prefix exceeds u * R
                 int last_seg;   // the last segment of positive mass
                 const df Rm = segment_cum<NT>(s_pref_all, nseg, s_cum, lane, last_seg);
-                const uint32_t jj = (L < gamma) ? static_cast<uint32_t>(L + 1) : static_cast<uint32_t>(gamma + 1);
-                const float u = philox_uniform(d.seed, jj, static_cast<uint32_t>(b), d.round,
-                                               (L < gamma) ? kPurposeResid : kPurposeBonus);
                 const df target = df_mul_f(Rm, u);
                 int sel = -1;
                 if (Rm.hi > 0.f) {
@@ -899,23 +966,26 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
                 }
             }
         }
+        if (!leader) return;
+        dec_sync<NT>();
+        if (warp == 0 && sched && s_K0 > 0) {
+            // a skipped block commits x_1..x_K (pair 0)
+            if (lane == 0 && d.commit_n) d.commit_n[b] = s_K0;
+            if (d.commit_tokens) write_tokens(lane, gamma, d.commit_tokens + bo, F.x, s_K0, -1);
         }
-        if (SHARD && !leader) return;
+        return;
+        }
+        if (!leader) return;
         dec_sync<NT>();
     }
 
-    // ---- every other rule (a warp per rule), the schedule (a warp per
-    // threshold pair) and the agreement counters: under the sampling rule the
-    // block's draw segments share these tasks round robin (every team holds
-    // the block's facts), otherwise the one team takes them all; then the
-    // leader writes the remaining commits ----
-    const int R = 1 + d.n_ell + d.n_k;
-    const int S = (sampling && !SHARD) ? nseg : 1, me = (sampling && !SHARD) ? seg : 0;
-    for (int ir = warp;; ir += NW) {
-        const int r = me + ir * S;   // this team's share of the rules
-        if (r >= R) break;
-        if (r == 0) {
-            if (!d.do_strict || sampling) continue;   // sampling: completed by the draw
+    // ---- greedy strict, or a sharded round after its draw masses: one team
+    // takes every rule (a warp per rule), then the schedule (a warp per
+    // threshold pair) and the agreement counters, then the commits ----
+    for (int r = warp; r < R; r += NW) {
+        if (r > 0) {
+            rule_task(r);
+        } else if (d.do_strict && !sampling) {
             const int L = rule_first_reject(d, F, 0, b, lane);
             if (lane == 0) {
                 s_L[0] = L;
@@ -924,45 +994,11 @@ __device__ __forceinline__ void decide_cta(const ScanParams &p, const PartView &
                 if (d.n_strict) d.n_strict[b] = L + 1;
             }
             if (d.tok_strict) write_tokens(lane, gamma, d.tok_strict + bo, F.x, L, F.t_am[L]);
-        } else {
-            const int L = rule_first_reject(d, F, r, b, lane);
-            const int corr = F.t_am[L];   // target argmax at the first rejection, or of the bonus row
-            const bool len = r <= d.n_ell;
-            const int64_t o = static_cast<int64_t>(len ? r - 1 : r - 1 - d.n_ell) * p.B + b;
-            int32_t *Lo = len ? d.L_len : d.L_topk, *no = len ? d.n_len : d.n_topk;
-            int32_t *to = len ? d.tok_len : d.tok_topk;
-            if (lane == 0) {
-                if (Lo) Lo[o] = L;
-                if (no) no[o] = L + 1;
-            }
-            if (to) write_tokens(lane, gamma, to + o * (gamma + 1), F.x, L, corr);
         }
     }
     if (!sched) return;
     dec_sync<NT>();   // s_L[0] of a greedy strict rule
-    const int t0 = ((me - R) % S + S) % S;   // pair t goes to team (R + t) mod S
-    for (int it = warp;; it += NW) {
-        const int t = t0 + it * S;
-        if (t >= d.n_tau) break;
-        int Kh, K, Do;
-        sched_pair(d, F, t, s_force != 0, s_D, lane, Kh, K, Do);
-        if (lane == 0) {
-            if (t == 0) s_K0 = K;
-            const int64_t o = static_cast<int64_t>(t) * p.B + b;
-            if (d.K_hat) d.K_hat[o] = Kh;
-            if (d.K) d.K[o] = K;
-            if (d.D_out) d.D_out[o] = Do;
-            if (d.agreement && K > 0 && d.do_strict) {
-                const int L = s_L[0];
-                unsigned long long *a = reinterpret_cast<unsigned long long *>(d.agreement + 4 * t);
-                atomicAdd(a + 0, static_cast<unsigned long long>(min(K, L)));
-                atomicAdd(a + 1, static_cast<unsigned long long>(K));
-                atomicAdd(a + 2, static_cast<unsigned long long>(K <= L ? 1 : 0));
-                atomicAdd(a + 3, 1ull);
-            }
-        }
-    }
-    if (!leader) return;
+    for (int t = warp; t < d.n_tau; t += NW) pair_task(t, true);
     dec_sync<NT>();
     if (warp == 0) {
         // tokens committed by a fused round: a skipped block commits x_1..x_K

@@ -144,6 +144,7 @@ struct ScanParams {
     int32_t kcap;            // rank saturation (>= 1)
     int32_t B;
     int32_t W;               // active warps
+    int32_t whole;           // every row is cut into this many pieces (0: cut by cost, or a device block count)
     int32_t pieces;          // pieces of a row at most (warps that stream parts of it)
     int32_t ctas;            // CTAs of a full streaming grid (one per SM)
     int64_t rows0;           // rows of group 0
@@ -310,6 +311,7 @@ constexpr int32_t kPipeCostDrafter = 21, kPipeCostTarget = 18;
 inline void set_divisors(ScanParams &p, int32_t cost_drafter = kCostDrafter, int32_t cost_target = kCostTarget) {
     // a short call's rows are cut into whole pieces: no weights
     const bool whole = p.rows > 0 && p.W % p.rows == 0 && p.W / p.rows >= kWholeMin;
+    p.whole = (whole && !p.nb_dev) ? static_cast<int32_t>(p.W / p.rows) : 0;
     p.pieces = (p.nb_dev || p.rows <= 0) ? static_cast<int32_t>(kPiecesPerRow)
                                          : static_cast<int32_t>((p.W + p.rows - 1) / p.rows + (whole ? 0 : 1));
     const bool mixed = p.n_groups == 2 && p.grp[0].kind != p.grp[1].kind && !whole;

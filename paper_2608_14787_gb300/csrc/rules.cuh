@@ -78,8 +78,13 @@ __device__ __forceinline__ void merge_row_group(const ScanParams &p, const PartV
                                                 int lg, SoftState &acc, float &g, bool &tok_bad, float (&t)[5]) {
     int64_t fw = 0, lw = -1;
     if (on) {
-        fw = part_owner(p, pv, r * p.RV);
-        lw = part_owner(p, pv, (r + 1) * p.RV - 1);
+        if (p.whole > 0) {   // every row in p.whole pieces
+            fw = r * p.whole;
+            lw = fw + p.whole - 1;
+        } else {
+            fw = part_owner(p, pv, r * p.RV);
+            lw = part_owner(p, pv, (r + 1) * p.RV - 1);
+        }
     }
     const int at = static_cast<int>(threadIdx.x) & ((1 << lg) - 1);
     const int run = (static_cast<int>(lw - fw) + (1 << lg)) >> lg;   // pieces of a run
