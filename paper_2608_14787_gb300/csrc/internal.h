@@ -144,6 +144,7 @@ struct ScanParams {
     int32_t kcap;            // rank saturation (>= 1)
     int32_t B;
     int32_t W;               // active warps
+    int32_t units;           // the pipelined pass's weighted warps: the total of their shares (0: equal shares)
     int32_t whole;           // every row is cut into this many pieces (0: cut by cost, or a device block count)
     int32_t pieces;          // pieces of a row at most (warps that stream parts of it)
     int32_t ctas;            // CTAs of a full streaming grid (one per SM)
@@ -305,6 +306,31 @@ constexpr int64_t kPipeSmallBytes = int64_t(64) << 20;
 // the CTAs of drafter rows ~2.5 us after the others).
 constexpr int32_t kPipeCostDrafter = 21, kPipeCostTarget = 18;
 
+// Shares of the pipelined pass's warps (a CTA's streaming warps 0..13, behind a
+// decide team of two): warps 2 and 3 of every four run on the two schedulers
+// that hold three streaming warps and a decide warp, the others on the two
+// that hold four.  With equal shares the latter ended 3.3 us later (52.7
+// against 49.4 us of a 16-block round).  GB300, that round: equal 55.3 us, 12 :
+// 13 54.6, 15 : 16 and 20 : 21 54.7 (two more warps a CTA, all schedulers alike
+// at 96 registers: 59.4).
+constexpr int kShareSlow = 12, kShareFast = 13;
+constexpr int kShareFour = 2 * kShareSlow + 2 * kShareFast;   // warps 4 i .. 4 i + 3
+constexpr int kShareWarps = 14;
+constexpr int kShareCta = 3 * kShareFour + 2 * kShareSlow;
+// The share units ahead of streaming warp w of the grid, and the warp that
+// holds unit u.
+__host__ __device__ inline int64_t share_start(int64_t w) {
+    const uint32_t cta = static_cast<uint32_t>(w) / kShareWarps, i = static_cast<uint32_t>(w) % kShareWarps;
+    return static_cast<int64_t>(cta) * kShareCta + (i >> 2) * kShareFour + (i & 3) * kShareSlow +
+           ((i & 3) == 3 ? kShareFast - kShareSlow : 0);
+}
+__host__ __device__ inline int64_t share_warp(int64_t u) {
+    const uint32_t cta = static_cast<uint32_t>(u) / kShareCta, o = static_cast<uint32_t>(u) % kShareCta;
+    const uint32_t four = o / kShareFour, x = o % kShareFour;
+    return static_cast<int64_t>(cta) * kShareWarps + 4 * four + (x >= kShareSlow) + (x >= 2 * kShareSlow) +
+           (x >= 2 * kShareSlow + kShareFast);
+}
+
 // The cost weights and division constants of a launch whose groups, rows, T
 // and W are set (host), all 16 warps of a CTA streaming.  The magic divisions
 // are exact while C * W < 2^53 (the callers check it).
@@ -332,6 +358,7 @@ inline void set_divisors(ScanParams &p, int32_t cost_drafter = kCostDrafter, int
     p.divC = make_fastdiv(static_cast<uint64_t>(p.C > 0 ? p.C : 1));
     for (int g = 0; g < 2; ++g) p.divWt[g] = make_fastdiv(static_cast<uint64_t>(p.wt[g]));
     for (int g = 0; g < 2; ++g) p.divP[g] = make_fastdiv(static_cast<uint64_t>(p.P[g] > 0 ? p.P[g] : 1));
+    p.units = 0;
     p.divW = make_fastdiv(static_cast<uint64_t>(p.W > 0 ? p.W : 1));
     p.divRV = make_fastdiv(static_cast<uint64_t>(p.RV > 0 ? p.RV : 1));
     for (int g = 0; g < 2; ++g) p.divNpos[g] = make_fastdiv(static_cast<uint64_t>(p.grp[g].npos > 0 ? p.grp[g].npos : 1));
@@ -429,9 +456,11 @@ __device__ __forceinline__ PartView part_view(const ScanParams &p) {
 // cost interval starts there: [start(w), start(w+1)) with start(w) the first
 // vector of cost >= floor(w C / W).  Requires C W < 2^53 (checked by the host).
 // Also the row r (of both groups) that holds start(w) and its vector k there.
+// SHARES: the launch's warps may have shares (p.units; W is then the units').
+template <bool SHARES>
 __device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartView &v, int64_t w, int64_t &row,
                                               int32_t &kv) {
-    const int64_t c = fast_div(w * v.C, v.divW);
+    const int64_t c = fast_div((SHARES && p.units ? share_start(w) : w) * v.C, v.divW);
     const int64_t c0 = v.rows0 * p.P[0];   // the cost of group 0
     const int g = (c <= c0) ? 0 : 1;
     const int64_t cg = g ? c - c0 : c;
@@ -451,6 +480,7 @@ __device__ __forceinline__ int64_t part_owner(const ScanParams &p, const PartVie
     const int64_t r = fast_div(u, p.divRV);
     const int64_t k = u - r * p.RV;
     const int64_t cost = (g ? pv.rows0 * p.P[0] : 0) + r * p.P[g] + (k > 0 ? p.R + k * p.wt[g] : 0);
+    if (p.units) return share_warp(fast_div((cost + 1) * p.units - 1, pv.divC));
     return fast_div((cost + 1) * pv.W - 1, pv.divC);
 }
 

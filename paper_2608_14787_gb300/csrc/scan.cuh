@@ -460,8 +460,8 @@ __device__ __forceinline__ const char *shfl_ptr(const char *ptr, int src) {
 // ring_bytes(STAGES, n_rings): one ring of STAGES tiles per streaming warp,
 // then their barriers; this warp's is ring w.  FEAT: also the five largest logits of
 // every drafter row piece (extended features); without it the code is
-// unchanged.
-template <int DT, bool FEAT, int STAGES = kStages>
+// unchanged.  SHARES: the warps may have unequal shares (the pipelined round).
+template <int DT, bool FEAT, int STAGES = kStages, bool SHARES = false>
 __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *smem, int w, int n_rings) {
     constexpr int kStages = STAGES;
     const int lane = threadIdx.x & 31;
@@ -492,7 +492,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
     // the range's two ends by two lanes at once, then the rows it touches
     int64_t rs;
     int32_t ks;
-    const int64_t vs = part_start(p, pv, gw + (lane & 1), rs, ks);
+    const int64_t vs = part_start<SHARES>(p, pv, gw + (lane & 1), rs, ks);
     const int64_t v0 = __shfl_sync(0xFFFFFFFFu, vs, 0), v1 = __shfl_sync(0xFFFFFFFFu, vs, 1);
     Cursor pc{v0, __shfl_sync(0xFFFFFFFFu, rs, 0), __shfl_sync(0xFFFFFFFFu, ks, 0)};
     const int64_t r_last = __shfl_sync(0xFFFFFFFFu, rs, 1) - (__shfl_sync(0xFFFFFFFFu, ks, 1) == 0 ? 1 : 0);
