@@ -332,9 +332,9 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 
 // Launch `kernel` behind the previous work of `stream` as a programmatic
 // dependent grid (host side).
-template <class Params>
-inline cudaError_t launch_dependent(void (*kernel)(Params), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                    const Params &p) {
+template <class... Params, class... Args>
+inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                    const Args &...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -345,7 +345,7 @@ inline cudaError_t launch_dependent(void (*kernel)(Params), dim3 grid, dim3 bloc
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
 // ---------------------------------------------------------------------------

@@ -46,6 +46,7 @@ __global__ void __launch_bounds__(kDecThreads) shard_draw_kernel(const __grid_co
     __shared__ int s_sel, s_col, s_thr, s_last, s_tok, s_seg;
     __shared__ df s_rem, s_rem2;
     extern __shared__ float s_pref_all[];   // [nseg][kDecThreads]: the decide's prefixes of this slice's draw row
+    griddep_wait();
     if (tid == 0) {
         s_thr = INT32_MAX;
         s_last = -1;
@@ -152,7 +153,10 @@ __global__ void __launch_bounds__(kDecThreads) shard_draw_kernel(const __grid_co
     }
 }
 
+// (This kernel and the small ones below are launched as programmatic
+// dependents, so that their launch overlaps the end of the work ahead.)
 __global__ void schedule_kernel(const __grid_constant__ ScheduleParams p) {
+    griddep_wait();
     const int lane = threadIdx.x & 31;
     const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     if (w >= static_cast<int64_t>(p.B) * p.n_tau) return;
@@ -194,6 +198,7 @@ __global__ void schedule_kernel(const __grid_constant__ ScheduleParams p) {
 }
 
 __global__ void agreement_kernel(const int32_t *K, const int32_t *L, int B, int n_tau, long long *acc) {
+    griddep_wait();
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= static_cast<int64_t>(B) * n_tau) return;
     const int t = static_cast<int>(idx / B), b = static_cast<int>(idx % B);
@@ -208,6 +213,7 @@ __global__ void agreement_kernel(const int32_t *K, const int32_t *L, int B, int 
 
 __global__ void commit_kernel(const int32_t *K, const int32_t *x, const int32_t *vt, const int32_t *vn, int B,
                               int gamma, int32_t *out_t, int32_t *out_n) {
+    griddep_wait();
     const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (idx >= static_cast<int64_t>(B) * (gamma + 1)) return;
     const int b = static_cast<int>(idx / (gamma + 1)), j = static_cast<int>(idx % (gamma + 1));
@@ -223,6 +229,7 @@ __global__ void commit_kernel(const int32_t *K, const int32_t *x, const int32_t 
 
 __global__ void uniforms_kernel(uint64_t seed, const uint32_t *j, const uint32_t *b, const uint64_t *round,
                                 const uint32_t *purpose, int64_t n, float *u) {
+    griddep_wait();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i < n) u[i] = philox_uniform(seed, j[i], b[i], round[i], purpose[i]);
 }
@@ -292,6 +299,7 @@ __global__ void __launch_bounds__(1024) select_rows_kernel(const int32_t *K, int
     __shared__ int s_warp[32];
     __shared__ int s_base;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    griddep_wait();
     if (tid == 0) s_base = 0;
     __syncthreads();
     for (int c0 = 0; c0 < B; c0 += 1024) {
@@ -315,49 +323,44 @@ __global__ void __launch_bounds__(1024) select_rows_kernel(const int32_t *K, int
 }
 
 cudaError_t launch_select_rows(const int32_t *K, int B, int32_t *rows, int32_t *n_rows, cudaStream_t stream) {
-    select_rows_kernel<<<1, 1024, 0, stream>>>(K, B, rows, n_rows);
-    return cudaGetLastError();
+    return launch_dependent(select_rows_kernel, dim3(1), dim3(1024), 0, stream, K, B, rows, n_rows);
 }
 
 cudaError_t launch_shard_draw(const ShardParams &sp, cudaStream_t stream) {
     if (sp.B == 0) return cudaSuccess;
     const size_t smem = static_cast<size_t>(sp.nseg) * kDecThreads * sizeof(float);
-    if (sp.dtype == SDD_BF16)
-        shard_draw_kernel<SDD_BF16><<<sp.B, kDecThreads, smem, stream>>>(sp);
-    else
-        shard_draw_kernel<SDD_F32><<<sp.B, kDecThreads, smem, stream>>>(sp);
-    return cudaGetLastError();
+    return launch_dependent(sp.dtype == SDD_BF16 ? shard_draw_kernel<SDD_BF16> : shard_draw_kernel<SDD_F32>, dim3(sp.B),
+                            dim3(kDecThreads), smem, stream, sp);
 }
 
 cudaError_t launch_schedule(const ScheduleParams &p, cudaStream_t stream) {
     const int64_t warps = static_cast<int64_t>(p.B) * p.n_tau;
     if (warps == 0) return cudaSuccess;
     const int64_t blocks = (warps * 32 + 255) / 256;
-    schedule_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(schedule_kernel, dim3(static_cast<unsigned>(blocks)), dim3(256), 0, stream, p);
 }
 
 cudaError_t launch_agreement(const int32_t *K, const int32_t *L, int B, int n_tau, long long *acc,
                              cudaStream_t stream) {
     const int64_t n = static_cast<int64_t>(B) * n_tau;
     if (n == 0) return cudaSuccess;
-    agreement_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(K, L, B, n_tau, acc);
-    return cudaGetLastError();
+    return launch_dependent(agreement_kernel, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, stream, K, L, B,
+                            n_tau, acc);
 }
 
 cudaError_t launch_commit(const int32_t *K, const int32_t *x, const int32_t *vt, const int32_t *vn, int B,
                           int gamma, int32_t *out_t, int32_t *out_n, cudaStream_t stream) {
     const int64_t n = static_cast<int64_t>(B) * (gamma + 1);
     if (n == 0) return cudaSuccess;
-    commit_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(K, x, vt, vn, B, gamma, out_t, out_n);
-    return cudaGetLastError();
+    return launch_dependent(commit_kernel, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, stream, K, x, vt, vn,
+                            B, gamma, out_t, out_n);
 }
 
 cudaError_t launch_uniforms(uint64_t seed, const uint32_t *j, const uint32_t *b, const uint64_t *round,
                             const uint32_t *purpose, int64_t n, float *u, cudaStream_t stream) {
     if (n == 0) return cudaSuccess;
-    uniforms_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(seed, j, b, round, purpose, n, u);
-    return cudaGetLastError();
+    return launch_dependent(uniforms_kernel, dim3(static_cast<unsigned>((n + 255) / 256)), dim3(256), 0, stream, seed, j, b,
+                            round, purpose, n, u);
 }
 
 }  // namespace sdd

@@ -59,6 +59,7 @@ __host__ __device__ inline size_t perm_smem_bytes(int B) {
 __global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const int32_t *L, int B, int gamma, int conditional,
                                                                   uint64_t seed, uint16_t *pi) {
     extern __shared__ int32_t s_dyn[];
+    griddep_wait();
     const int words = (B + 31) / 32;
     uint32_t *s_mask = reinterpret_cast<uint32_t *>(s_dyn);                // validity bits
     int32_t *s_wpre = s_dyn + words;                                       // valid blocks before each word
@@ -238,6 +239,7 @@ constexpr int kPrefixU = 4;
 __global__ void __launch_bounds__(kPrefixThreads) perm_prefix_kernel(const float *q, const uint16_t *pi, int B,
                                                                      int gamma, int n_rep, int signal, df eta_loc,
                                                                      df log_eta_c, unsigned long long *sums) {
+    griddep_wait();
     const int per = (B + kPrefixThreads - 1) / kPrefixThreads;
     const int r = blockIdx.x / per, b = static_cast<int>(blockIdx.x % per) * kPrefixThreads + threadIdx.x;
     int Kh = 0;
@@ -337,6 +339,7 @@ __device__ __forceinline__ void met_stage(const float *q, const int32_t *L, int 
 __global__ void __cluster_dims__(kMetCluster, 1, 1) __launch_bounds__(kMetThreads)
     metrics_kernel(const float *q, const int32_t *L, int B, int gamma, int conditional, double *bce, double *bce_base,
                    double *auroc, int32_t *n_pos, int32_t *n_neg) {
+    griddep_wait();
     const int j = blockIdx.x / kMetCluster, rank = blockIdx.x % kMetCluster;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ float s_pos[kMetPos], s_neg[kMetNeg];
@@ -465,23 +468,21 @@ cudaError_t launch_perm_diag(const float *q, const int32_t *L, int B, int gamma,
         if (e != cudaSuccess) return e;
     }
     if (n_rep > 0) {
-        perm_build_kernel<<<n_rep * gamma, kPermThreads, smem, stream>>>(L, B, gamma, signal == SDD_SIG_CONDITIONAL,
-                                                                        seed, pi);
-        e = cudaGetLastError();
+        e = launch_dependent(perm_build_kernel, dim3(n_rep * gamma), dim3(kPermThreads), smem, stream, L, B, gamma,
+                             signal == SDD_SIG_CONDITIONAL ? 1 : 0, seed, pi);
         if (e != cudaSuccess) return e;
     }
     const int per = (B + kPrefixThreads - 1) / kPrefixThreads;
-    perm_prefix_kernel<<<static_cast<unsigned>(per) * static_cast<unsigned>(n_rep + 1), kPrefixThreads, 0, stream>>>(
-        q, pi, B, gamma, n_rep, signal, eta_loc, log_eta_c, sums);
-    return cudaGetLastError();
+    return launch_dependent(perm_prefix_kernel,
+                            dim3(static_cast<unsigned>(per) * static_cast<unsigned>(n_rep + 1)), dim3(kPrefixThreads), 0,
+                            stream, q, pi, B, gamma, n_rep, signal, eta_loc, log_eta_c, sums);
 }
 
 cudaError_t launch_position_metrics(const float *q, const int32_t *L, int B, int gamma, int conditional, double *bce,
                                     double *bce_base, double *auroc, int32_t *n_pos, int32_t *n_neg,
                                     cudaStream_t stream) {
-    metrics_kernel<<<gamma * kMetCluster, kMetThreads, 0, stream>>>(q, L, B, gamma, conditional, bce, bce_base, auroc,
-                                                                    n_pos, n_neg);
-    return cudaGetLastError();
+    return launch_dependent(metrics_kernel, dim3(gamma * kMetCluster), dim3(kMetThreads), 0, stream, q, L, B, gamma,
+                            conditional, bce, bce_base, auroc, n_pos, n_neg);
 }
 
 }  // namespace sdd

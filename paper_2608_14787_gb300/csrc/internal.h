@@ -401,25 +401,18 @@ __device__ __forceinline__ int64_t fast_div(int64_t n, const FastDiv &f) {
     return static_cast<int64_t>(f.pow2 ? (u >> f.s) : (__umul64hi(u, f.M) >> f.s));
 }
 
-// make_fastdiv on the device (a 128-bit division, once per warp).
-__device__ __forceinline__ FastDiv make_fastdiv_dev(uint64_t d) {
-    FastDiv f{0, 63u - static_cast<uint32_t>(__clzll(static_cast<long long>(d))), 0};
-    if ((d & (d - 1)) == 0) {
-        f.pow2 = 1;
-        return f;
-    }
-    const unsigned __int128 num = static_cast<unsigned __int128>(1) << (64 + f.s);
-    f.M = static_cast<uint64_t>((num + d - 1) / d);
-    return f;
-}
-
 // The launch's partition: from the parameters, or -- with a device block
-// count -- computed on the device the way the host computes it.
+// count -- computed on the device the way the host computes it; the divisions
+// by C and W are then plain 64-bit ones (a magic number for each would take a
+// 128-bit division a warp).
 struct PartView {
     int64_t nb, rows0, rows, T, T0, C;
     int32_t W;
-    FastDiv divC, divW;
 };
+__device__ __forceinline__ int64_t div_part(int64_t n, int64_t d, const FastDiv &f, const ScanParams &p) {
+    if (p.nb_dev) return static_cast<int64_t>(static_cast<uint64_t>(n) / static_cast<uint64_t>(d));
+    return fast_div(n, f);
+}
 
 __device__ __forceinline__ PartView part_view(const ScanParams &p) {
     PartView v;
@@ -431,8 +424,6 @@ __device__ __forceinline__ PartView part_view(const ScanParams &p) {
         v.T0 = p.T0;
         v.C = p.C;
         v.W = p.W;
-        v.divC = p.divC;
-        v.divW = p.divW;
         return v;
     }
     v.nb = min(max(static_cast<int64_t>(*p.nb_dev), static_cast<int64_t>(0)), static_cast<int64_t>(p.grp[0].nb));
@@ -442,8 +433,6 @@ __device__ __forceinline__ PartView part_view(const ScanParams &p) {
     v.T0 = v.rows0 * p.RV;
     v.C = v.rows0 * p.P[0] + (v.rows - v.rows0) * p.P[1];
     v.W = scan_warps(p.W, v.T, v.rows);
-    v.divC = make_fastdiv_dev(static_cast<uint64_t>(v.C > 0 ? v.C : 1));
-    v.divW = make_fastdiv_dev(static_cast<uint64_t>(v.W));
     return v;
 }
 
@@ -460,7 +449,7 @@ __device__ __forceinline__ PartView part_view(const ScanParams &p) {
 template <bool SHARES>
 __device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartView &v, int64_t w, int64_t &row,
                                               int32_t &kv) {
-    const int64_t c = fast_div((SHARES && p.units ? share_start(w) : w) * v.C, v.divW);
+    const int64_t c = div_part((SHARES && p.units ? share_start(w) : w) * v.C, v.W, p.divW, p);
     const int64_t c0 = v.rows0 * p.P[0];   // the cost of group 0
     const int g = (c <= c0) ? 0 : 1;
     const int64_t cg = g ? c - c0 : c;
@@ -480,8 +469,8 @@ __device__ __forceinline__ int64_t part_owner(const ScanParams &p, const PartVie
     const int64_t r = fast_div(u, p.divRV);
     const int64_t k = u - r * p.RV;
     const int64_t cost = (g ? pv.rows0 * p.P[0] : 0) + r * p.P[g] + (k > 0 ? p.R + k * p.wt[g] : 0);
-    if (p.units) return share_warp(fast_div((cost + 1) * p.units - 1, pv.divC));
-    return fast_div((cost + 1) * pv.W - 1, pv.divC);
+    if (p.units) return share_warp(fast_div((cost + 1) * p.units - 1, p.divC));
+    return div_part((cost + 1) * pv.W - 1, pv.C, p.divC, p);
 }
 
 }  // namespace sdd

@@ -1049,6 +1049,7 @@ __global__ void scorer_features_kernel(const float *maxprob, const float *entrop
                                        const float *top5, int64_t M, int gamma, float gen, uint16_t *f) {
     const int64_t w = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
+    griddep_wait();
     if (w >= M) return;
     float v[8];
 #pragma unroll
@@ -1075,9 +1076,8 @@ cudaError_t launch_scorer_features(const float *maxprob, const float *entropy, c
                                    int64_t M, int gamma, float gen, uint16_t *f, cudaStream_t stream) {
     if (M == 0) return cudaSuccess;
     const int64_t threads = M * 32;
-    scorer_features_kernel<<<static_cast<unsigned>((threads + 255) / 256), 256, 0, stream>>>(
-        maxprob, entropy, margin, top5, M, gamma, gen, f);
-    return cudaGetLastError();
+    return launch_dependent(scorer_features_kernel, dim3(static_cast<unsigned>((threads + 255) / 256)), dim3(256), 0,
+                            stream, maxprob, entropy, margin, top5, M, gamma, gen, f);
 }
 
 }  // namespace sdd

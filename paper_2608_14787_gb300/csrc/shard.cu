@@ -239,6 +239,7 @@ __global__ void __launch_bounds__(kShardThreads, kShardMinCtas) shard_partials_k
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t r = blockIdx.x;
     const int64_t nd = static_cast<int64_t>(sp.B) * sp.gamma;
+    griddep_wait();
     const bool drafter = r < nd;
     const char *row;
     int tok = -1;
@@ -391,8 +392,7 @@ cudaError_t launch_shard_partials(const ShardParams &sp, cudaStream_t stream) {
     const bool bf = sp.dtype == SDD_BF16, cand = sp.kcap > 0;
     void (*const k)(ShardParams) = bf ? (cand ? shard_partials_kernel<SDD_BF16, true> : shard_partials_kernel<SDD_BF16, false>)
                                       : (cand ? shard_partials_kernel<SDD_F32, true> : shard_partials_kernel<SDD_F32, false>);
-    k<<<static_cast<unsigned>(rows), kShardThreads, 0, stream>>>(sp);
-    return cudaGetLastError();
+    return launch_dependent(k, dim3(static_cast<unsigned>(rows)), dim3(kShardThreads), 0, stream, sp);
 }
 
 }  // namespace sdd
