@@ -1149,8 +1149,12 @@ sdd_status_t sdd_block_decide(const sdd_block_args *a, sdd_stream_t stream) {
 }
 
 sdd_status_t sdd_block(const sdd_block_args *a, sdd_stream_t stream) {
-    SDD_TRY(sdd_block_scan(a, stream));
-    return sdd_block_decide(a, stream);
+    ScanParams p;
+    bool empty = false;
+    SDD_TRY(block_params(a, p, &empty));
+    if (empty) return SDD_OK;
+    SDD_TRY(run_scan(p, reinterpret_cast<cudaStream_t>(stream)));
+    return run_decide(p, reinterpret_cast<cudaStream_t>(stream));
 }
 
 // Rounds of at most this many bytes of logits run in the pipelined kernel;

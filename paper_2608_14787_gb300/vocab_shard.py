@@ -133,13 +133,15 @@ def run_local(ranks, slices_d, slices_t, x, *, seed=0, round_=0):
     for r in ranks:
         r.decide(all_rec, S)
     if ranks[0].sampling:
-        all_mass = torch.stack([r.mass for r in ranks])
+        all_mass = torch.cat([r.mass for r in ranks])   # [S, B, 2]
         for s, r in enumerate(ranks):
             r.draw(all_mass, S, s)
-        for name in ("tokens_strict", "commit_tokens"):
-            top = torch.stack([getattr(r, name) for r in ranks]).amax(dim=0)
-            for r in ranks:
-                getattr(r, name).copy_(top)
+        # tokens_strict and commit_tokens of all ranks: the element-wise maximum
+        top = ranks[0].rnd._tokens
+        for r in ranks[1:]:
+            torch.maximum(top, r.rnd._tokens, out=top)
+        for r in ranks[1:]:
+            r.rnd._tokens.copy_(top)
     return ranks
 
 
