@@ -296,12 +296,12 @@ __device__ __forceinline__ float fkey_inv(uint32_t k) {
 // (~14 instructions a tile; with the tile numbers in registers of their own
 // the update took 81, as nearly every tile has a lane that inserts).  fp32:
 // the keys in ck, the tiles' numbers in ct.
-template <int DT>
-__device__ __forceinline__ void group_update(float cm, uint32_t tile, uint32_t (&ck)[5], uint32_t (&ct)[5]) {
+template <int DT, int N>
+__device__ __forceinline__ void group_update(float cm, uint32_t tile, uint32_t (&ck)[N], uint32_t (&ct)[N]) {
     if (DT == SDD_BF16) {
         uint32_t key = (fkey(cm) & 0xFFFF0000u) | (tile & 0xFFFFu);
 #pragma unroll
-        for (int j = 0; j < 5; ++j) {
+        for (int j = 0; j < N; ++j) {
             const uint32_t lo = min(ck[j], key);
             ck[j] = max(ck[j], key);
             key = lo;
@@ -309,9 +309,9 @@ __device__ __forceinline__ void group_update(float cm, uint32_t tile, uint32_t (
         return;
     }
     uint32_t key = fkey(cm);
-    if (key <= ck[4]) return;
+    if (key <= ck[N - 1]) return;
 #pragma unroll
-    for (int j = 0; j < 5; ++j)
+    for (int j = 0; j < N; ++j)
         if (key > ck[j]) {
             const uint32_t tk = ck[j], tt = ct[j];
             ck[j] = key;

@@ -2,6 +2,8 @@
 // tensor-parallel LM head: each rank holds one contiguous vocabulary slice
 // [v0, v1) of every drafter and target row).
 //
+//  * shard_stream_kernel -- rows streamed through per-warp rings by clusters of
+//    two CTAs (below); every call but those that stream_plan leaves to the next.
 //  * shard_partials_kernel -- one CTA per row of the slice.  Each thread
 //    streams its 16-byte vectors (ascending), keeping the online-softmax state
 //    of its entries relative to an integer reference in log2 units (a new
@@ -17,6 +19,10 @@
 // The records of all slices are merged, and every rule of the round runs, in
 // decide_kernel (rules.cuh: merge_row_shards); the draw that follows the
 // exchange of the slices' draw-row masses is shard_draw_kernel (decide.cu).
+#include <algorithm>
+#include <atomic>
+
+#include "scan.cuh"
 #include "rules.cuh"
 
 namespace sdd {
@@ -47,12 +53,10 @@ __device__ __forceinline__ int cand_index(uint64_t key) {
 }
 
 __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const uint64_t o = __shfl_xor_sync(0xFFFFFFFFu, v, off);
-        v = (o > v) ? o : v;
-    }
-    return v;
+    const uint32_t hi = static_cast<uint32_t>(v >> 32);
+    const uint32_t mh = __reduce_max_sync(0xFFFFFFFFu, hi);
+    const uint32_t ml = __reduce_max_sync(0xFFFFFFFFu, hi == mh ? static_cast<uint32_t>(v) : 0u);
+    return (static_cast<uint64_t>(mh) << 32) | ml;
 }
 
 // The rare paths of the per-element work, kept out of line so that the
@@ -384,12 +388,543 @@ __global__ void __launch_bounds__(kShardThreads, kShardMinCtas) shard_partials_k
     }
 }
 
+// ---------------------------------------------------------------------------
+// The streaming form: rows of the slice by clusters of two CTAs, one CTA per
+// SM.  A cluster takes whole rows (as even a cost as whole rows allow: a
+// drafter row 10, a target row 9), its 32 warps an equal run of their vectors
+// each, streamed through the rings of the one-GPU pass (scan.cuh:
+// process_tile).  A warp's piece of a row leaves its state and, for target
+// rows of a round with the top-k rule, its kcap highest entries in the shared
+// memory of the CTA that holds the row's first vector (the row that crosses
+// the cluster's middle over distributed shared memory); after one cluster
+// barrier each CTA merges its rows' pieces, a warp a row, into the records.
+//
+// Candidates: each lane keeps its kCandList largest tile maxima
+// (group_update).  With T the kcap-th largest of all lanes' maxima, the piece's
+// kcap highest entries are at least T and lie in the groups whose maximum is
+// at least T: the warp re-reads those (about kcap of them), keeps the entries
+// of at least T and ranks them by (value, index).  When more groups or entries
+// reach T than there is room for, or a lane's whole list does (it may have
+// dropped one), the piece is read again with the exact per-vector list
+// (piece_candidates): ties in their hundreds, or short pieces.
+//
+// Bound by HBM and, at the end, by the last pieces' chain of selection and
+// merge.  GB300, half of a 151,936 vocabulary, 16 x 32 positions, bf16 (158
+// MB): 36.5 us with the top-k rule (k <= 10), 29.5 us without (5.35 TB/s),
+// against 52.9 and 37.2 us with one CTA per row and register loads.
+// ---------------------------------------------------------------------------
+constexpr int kCandList = 7;      // tile maxima a lane keeps
+constexpr int kCandGroups = 32;   // groups a piece re-reads at most
+constexpr int kCandKeys = 64;     // entries it ranks at most
+constexpr int kCostSliceDrafter = 10, kCostSliceTarget = 9;
+
+// A piece's slot: its partial, then its candidate keys, descending (0: none).
+constexpr int kSlotBytes = static_cast<int>(sizeof(Partial)) + SDD_SHARD_KMAX * 8;
+
+struct StreamParams {
+    ShardParams sp;
+    int32_t rows, nd;        // all rows, drafter rows
+    int32_t slots;           // piece slots of a CTA
+    uint32_t wait_polls;
+};
+
+__device__ __forceinline__ uint32_t slice_cta_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// A shared-memory address of this CTA in the cluster's CTA `rank`.
+__device__ __forceinline__ uint32_t slice_map(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_slice_v4(uint32_t addr, uint4 v) {
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void st_slice_u64(uint32_t addr, uint64_t v) {
+    asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+
+// The first row of cluster c of G: the first whose preceding rows cost at
+// least c / G of the whole.
+__device__ __forceinline__ int slice_row(const StreamParams &p, int c, int G) {
+    const int64_t cd = static_cast<int64_t>(p.nd) * kCostSliceDrafter;
+    const int64_t ct = cd + static_cast<int64_t>(p.rows - p.nd) * kCostSliceTarget;
+    const int64_t x = ct * c / G;
+    if (x <= cd) return static_cast<int>((x + kCostSliceDrafter - 1) / kCostSliceDrafter);
+    return p.nd + static_cast<int>((x - cd + kCostSliceTarget - 1) / kCostSliceTarget);
+}
+
+__device__ __forceinline__ const char *slice_row_base(const StreamParams &p, int r) {
+    return r < p.nd ? p.sp.zd + r * p.sp.stride_bytes : p.sp.zt + (r - p.nd) * p.sp.stride_bytes;
+}
+
+// The kcap highest entries of vectors [kb, ke) of a row, exactly, by one warp:
+// a list of the kcap highest vectors held one key per lane (larger maximum
+// first, then lower index; a later vector that ties the last one ranks after
+// it), then the kcap highest of their entries.  Lane k returns the k-th key.
+template <int DT>
+__device__ __noinline__ uint64_t piece_candidates(const char *row, int kb, int ke, int Vs, int v0, int kc) {
+    constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
+    const int lane = threadIdx.x & 31;
+    uint64_t lk = 0ull;
+    float thr = -INFINITY;
+    for (int b = kb; b < ke; b += 32) {
+        const int vec = b + lane;
+        float vm = -INFINITY;
+        if (vec < ke) {
+            uint4 w = __ldg(reinterpret_cast<const uint4 *>(row) + vec);
+            if ((vec + 1) * EPV > Vs) mask_tail<DT>(w, Vs - vec * EPV);
+            w = clamp_vec<DT>(w);
+#pragma unroll
+            for (int e = 0; e < EPV; ++e) vm = fmaxf(vm, vec_elem<DT>(w, e));
+        }
+        unsigned pend = __ballot_sync(0xFFFFFFFFu, vm > thr);
+        const uint64_t mine = cand_key(vm, vec);
+        while (pend) {
+            const int src = __ffs(pend) - 1;
+            pend &= pend - 1;
+            lk = warp_list_insert(lk, __shfl_sync(0xFFFFFFFFu, mine, src), kc, lane);
+        }
+        const uint64_t last = __shfl_sync(0xFFFFFFFFu, lk, kc - 1);
+        thr = (last != 0ull) ? cand_value(last) : -INFINITY;
+    }
+    uint64_t key[8];
+    const int vec = (lane < kc && lk != 0ull) ? cand_index(lk) : -1;
+    uint4 w = make_uint4(0, 0, 0, 0);
+    if (vec >= 0) w = clamp_vec<DT>(__ldg(reinterpret_cast<const uint4 *>(row) + vec));
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        key[e] = 0ull;
+        if (e < EPV && vec >= 0 && vec * EPV + e < Vs) {
+            const float x = vec_elem<DT>(w, e);
+            if (!isnan(x)) key[e] = cand_key(x, v0 + vec * EPV + e);
+        }
+    }
+    uint64_t out = 0ull;
+    for (int k = 0; k < kc; ++k) {
+        uint64_t mine = 0ull;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) mine = key[e] > mine ? key[e] : mine;
+        const uint64_t best = warp_max_u64(mine);
+        if (lane == k) out = best;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) key[e] = (key[e] == best) ? 0ull : key[e];   // (unique keys)
+    }
+    return out;
+}
+
+// The same from the lanes' lists of tile maxima; s_key: kCandKeys keys of
+// scratch for this warp.
+template <int DT>
+__device__ __forceinline__ uint64_t group_candidates(const char *row, int kb, int ke, int Vs, int v0, int kc,
+                                                     uint32_t (&ck)[kCandList], uint32_t (&ct)[kCandList],
+                                                     uint64_t *s_key) {
+    constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
+    const int lane = threadIdx.x & 31;
+    int first = -1, groups = 0, popped = 0;   // lane g < groups: group g's first vector
+    uint32_t T = 0u;                          // the kcap-th maximum's key (its upper half for bf16)
+    bool fits = true;
+#pragma unroll 1
+    for (;;) {
+        const uint32_t m = __reduce_max_sync(0xFFFFFFFFu, ck[0]);
+        const uint32_t mv = (DT == SDD_BF16) ? (m & 0xFFFF0000u) : m;
+        if (m == 0u || (groups >= kc && mv < T)) break;
+        if (groups == kCandGroups) {
+            fits = false;
+            break;
+        }
+        if (groups < kc) T = mv;
+        const int owner = __ffs(__ballot_sync(0xFFFFFFFFu, ck[0] == m)) - 1;
+        const uint32_t tile = (DT == SDD_BF16) ? (m & 0xFFFFu) : __shfl_sync(0xFFFFFFFFu, ct[0], owner);
+        if (lane == groups) first = kb + static_cast<int>(tile) * kTileVec + owner;
+        ++groups;
+        if (lane == owner) {
+            ++popped;
+#pragma unroll
+            for (int j = 0; j + 1 < kCandList; ++j) {
+                ck[j] = ck[j + 1];
+                if (DT != SDD_BF16) ct[j] = ct[j + 1];
+            }
+            ck[kCandList - 1] = 0u;
+        }
+    }
+    // a piece of fewer groups than kcap: every entry counts
+    if (groups < kc || __any_sync(0xFFFFFFFFu, popped == kCandList)) fits = false;
+    int n = 0;
+    if (fits) {
+        const float thr = fkey_inv(DT == SDD_BF16 && !(T & 0x80000000u) ? (T | 0xFFFFu) : T);
+        for (int u0 = 0; u0 < 8 * groups; u0 += 128) {
+            uint4 w[4];
+            int vec[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                const int u = u0 + 32 * h + lane;
+                const int f = __shfl_sync(0xFFFFFFFFu, first, (u >> 3) & 31);
+                const int v = f + 32 * (u & 7);
+                vec[h] = (u < 8 * groups && v < ke) ? v : -1;
+                w[h] = (vec[h] >= 0) ? __ldg(reinterpret_cast<const uint4 *>(row) + vec[h]) : make_uint4(0, 0, 0, 0);
+            }
+            // the lane's entries of at least T, a bit each; then a place for each
+            uint32_t in = 0u;
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                w[h] = clamp_vec<DT>(w[h]);
+#pragma unroll
+                for (int e = 0; e < EPV; ++e)
+                    if (vec[h] >= 0 && vec[h] * EPV + e < Vs && vec_elem<DT>(w[h], e) >= thr)
+                        in |= 1u << (h * EPV + e);
+            }
+            const int mine = __popc(in);
+            int incl = mine;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const int t = __shfl_up_sync(0xFFFFFFFFu, incl, off);
+                if (lane >= off) incl += t;
+            }
+            int at = n + incl - mine;
+            n += __shfl_sync(0xFFFFFFFFu, incl, 31);
+            while (in) {
+                const int bit = __ffs(in) - 1, h = bit / EPV, e = bit % EPV;
+                in &= in - 1;
+                const uint4 c = (h < 2) ? (h == 0 ? w[0] : w[1]) : (h == 2 ? w[2] : w[3]);
+                const int v = (h < 2) ? (h == 0 ? vec[0] : vec[1]) : (h == 2 ? vec[2] : vec[3]);
+                if (at < kCandKeys) s_key[at] = cand_key(vec_elem_sel<DT>(c, e), v0 + v * EPV + e);
+                ++at;
+            }
+        }
+        if (n > kCandKeys) fits = false;
+    }
+    if (!fits) return piece_candidates<DT>(row, kb, ke, Vs, v0, kc);
+    __syncwarp();
+    // every key's rank among the n (they are unique); the kcap highest go back in order
+    const uint64_t a = (lane < n) ? s_key[lane] : 0ull, b = (lane + 32 < n) ? s_key[lane + 32] : 0ull;
+    int ra = 0, rb = 0;
+    for (int t = 0; t < n; ++t) {
+        const uint64_t o = s_key[t];
+        ra += o > a ? 1 : 0;
+        rb += o > b ? 1 : 0;
+    }
+    __syncwarp();
+    if (a != 0ull && ra < kc) s_key[ra] = a;
+    if (b != 0ull && rb < kc) s_key[rb] = b;
+    __syncwarp();
+    const uint64_t out = (lane < kc && lane < n) ? s_key[lane] : 0ull;
+    __syncwarp();   // (the scratch serves the warp's next piece)
+    return out;
+}
+
+template <int DT, bool CAND>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+    shard_stream_kernel(const __grid_constant__ StreamParams p) {
+    extern __shared__ __align__(128) unsigned char smem[];
+    constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
+    constexpr int CW = 2 * kWarpsPerCta;   // the cluster's warps
+    const ShardParams &sp = p.sp;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rank = static_cast<int>(slice_cta_rank());
+    unsigned char *ring = smem + warp * (kStages * kTileBytes);
+    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kWarpsPerCta * kStages * kTileBytes) + warp * kStages;
+    unsigned char *slots = smem + kScanSmem;
+    uint64_t *s_key = reinterpret_cast<uint64_t *>(slots + p.slots * kSlotBytes) + warp * kCandKeys;
+    if (lane == 0) {
+#pragma unroll
+        for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
+        fence_mbar_init();
+    }
+    __syncwarp();
+    // (the peer has started before anything is written to its shared memory)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    griddep_wait();
+
+    // the cluster's rows [ra, rb), this warp's vectors [v0, v1) of them
+    const int cl = static_cast<int>(blockIdx.x) >> 1, G = static_cast<int>(gridDim.x) >> 1;
+    const int bnd = slice_row(p, cl + (lane & 1), G);
+    const int ra = __shfl_sync(0xFFFFFFFFu, bnd, 0), rb = __shfl_sync(0xFFFFFFFFu, bnd, 1);
+    const int RV = sp.RVs, tail = sp.Vs % EPV;
+    const int64_t Tc = static_cast<int64_t>(rb - ra) * RV;
+    const int gw = rank * kWarpsPerCta + warp;
+    const int64_t v0 = Tc * gw / CW, v1 = Tc * (gw + 1) / CW;
+    // CTA 0 owns the rows that start before the cluster's middle: the first n0
+    const int n0 = static_cast<int>((Tc * kWarpsPerCta / CW + RV - 1) / RV);
+
+    struct Cur {
+        int64_t v;
+        int l, k;   // row of the cluster, vector in it
+    };
+    Cur pc{v0, static_cast<int>(v0 / RV), 0};
+    pc.k = static_cast<int>(v0 - static_cast<int64_t>(pc.l) * RV);
+    Cur cc = pc;
+    const char *prow = slice_row_base(p, ra + pc.l);
+    const uint64_t pol = l2_evict_first_policy();
+    uint32_t pending = 0, phase = 0;
+    auto issue = [&](int slot) {
+        const int n = static_cast<int>(min(static_cast<int64_t>(min(kTileVec, RV - pc.k)), v1 - pc.v));
+        if (lane == 0) {
+            mbar_arrive_expect_tx(&bars[slot], static_cast<uint32_t>(n) * 16u);
+            bulk_g2s(ring + slot * kTileBytes, prow + static_cast<int64_t>(pc.k) * 16, static_cast<uint32_t>(n) * 16u,
+                     &bars[slot], pol);
+        }
+        pending |= 1u << slot;
+        pc.v += n;
+        pc.k += n;
+        if (pc.k == RV && pc.v < v1) {
+            pc.k = 0;
+            pc.l += 1;
+            prow = slice_row_base(p, ra + pc.l);
+        }
+    };
+    for (int s = 0; s < kStages && pc.v < v1; ++s) issue(s);
+
+    SoftState st = soft_identity();
+    uint32_t ck[kCandList], ct[kCandList];
+    int kb = 0, slot = 0;
+    float s_hi = 0.f, s_lo = 0.f;
+    bool in_piece = false, ent = false, timed_out = false;
+    const char *crow = nullptr;
+    while (cc.v < v1) {
+        const int n = static_cast<int>(min(static_cast<int64_t>(min(kTileVec, RV - cc.k)), v1 - cc.v));
+        if (!in_piece) {
+            st = soft_identity();
+            s_hi = s_lo = 0.f;
+#pragma unroll
+            for (int k = 0; k < kCandList; ++k) ck[k] = ct[k] = 0u;
+            kb = cc.k;
+            ent = ra + cc.l < p.nd;
+            crow = slice_row_base(p, ra + cc.l);
+            in_piece = true;
+        }
+        if (!__any_sync(0xFFFFFFFFu, mbar_wait_bounded(&bars[slot], (phase >> slot) & 1u, p.wait_polls))) {
+            timed_out = true;
+            break;
+        }
+        uint4 *tile = reinterpret_cast<uint4 *>(ring + slot * kTileBytes);
+        const bool row_end = cc.k + n == RV;
+        const bool pad = n < kTileVec || (row_end && tail);
+        if (pad) pad_tile<DT>(tile, n, lane, row_end, tail);
+        const float cm = ent ? process_tile<DT, true>(tile, cc.k, lane, st, s_hi, s_lo)
+                             : process_tile<DT, false>(tile, cc.k, lane, st, s_hi, s_lo);
+        if (CAND && !ent) group_update<DT>(cm, static_cast<uint32_t>(cc.k - kb) / kTileVec, ck, ct);
+        __syncwarp();
+        phase ^= 1u << slot;
+        pending &= ~(1u << slot);
+        if (pad) fence_proxy_async_smem();   // generic writes of pad_tile
+        if (pc.v < v1) issue(slot);
+        slot = (slot + 1 == kStages) ? 0 : slot + 1;
+        cc.v += n;
+        cc.k += n;
+        if (row_end || cc.v == v1) {
+            // the piece's end, as in the one-GPU pass (scan_warp)
+            const float M = fkey_inv(__reduce_max_sync(0xFFFFFFFFu, fkey(st.m)));
+            const bool holds = st.m == M && st.amax != INT32_MAX;
+            const int va = (holds ? st.amax : 0) + lane;
+            uint4 aw[kVPL];
+#pragma unroll
+            for (int i = 0; i < kVPL; ++i)
+                aw[i] = (holds && va + 32 * i < RV) ? __ldg(reinterpret_cast<const uint4 *>(crow) + va + 32 * i)
+                                                    : make_uint4(0, 0, 0, 0);
+            const float rM = ceilf(M * kLog2e);
+            const float sc = pow2f_int(st.r - rM);
+            float t2 = sc * fmaf((st.m - M) * kLog2e, s_hi + s_lo, st.t2);
+            float sh = s_hi * sc, sl = s_lo * sc;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                float h, e;
+                two_sum(sh, __shfl_xor_sync(0xFFFFFFFFu, sh, off), h, e);
+                fast_two_sum(h, e + (sl + __shfl_xor_sync(0xFFFFFFFFu, sl, off)), sh, sl);
+                t2 += __shfl_xor_sync(0xFFFFFFFFu, t2, off);
+            }
+            int idx = INT32_MAX;
+#pragma unroll
+            for (int i = kVPL - 1; i >= 0; --i) {
+                const uint4 c = clamp_vec<DT>(aw[i]);
+#pragma unroll
+                for (int e = EPV - 1; e >= 0; --e)
+                    if ((va + 32 * i) * EPV + e < sp.Vs && vec_elem<DT>(c, e) == M) idx = (va + 32 * i) * EPV + e;
+            }
+            idx = __reduce_min_sync(0xFFFFFFFFu, holds ? idx : INT32_MAX);
+            uint64_t key = 0ull;
+            if (CAND && !ent) key = group_candidates<DT>(crow, kb, cc.k, sp.Vs, sp.v0, sp.kcap, ck, ct, s_key);
+            const int own = cc.l >= n0 ? 1 : 0;
+            const int at = own ? (cc.l - n0) + (gw - kWarpsPerCta) : cc.l + gw;
+            const uint32_t dst = slice_map(smem_addr(slots + at * kSlotBytes), static_cast<uint32_t>(own));
+            if (lane < 2) {
+                Partial pt;
+                pt.m = M;
+                pt.r = rM;
+                pt.t2 = t2;
+                pt.sh = sh;
+                pt.sl = sl;
+                pt.amax = idx;
+                pt.rank = 0;
+                pt.g = 0.f;
+                const uint4 *q = reinterpret_cast<const uint4 *>(&pt);
+                st_slice_v4(dst + 16 * lane, lane == 0 ? q[0] : q[1]);
+            }
+            if (CAND && !ent && lane < SDD_SHARD_KMAX)
+                st_slice_u64(dst + static_cast<uint32_t>(sizeof(Partial)) + 8 * lane, key);
+            in_piece = false;
+            if (row_end) {
+                cc.k = 0;
+                cc.l += 1;
+            }
+        }
+    }
+    if (timed_out) {
+        if (lane == 0) status_or(sp.status, SDD_DEV_TIMEOUT);
+        for (int s = 0; s < kStages; ++s)
+            if (pending & (1u << s)) (void)mbar_wait_bounded(&bars[s], (phase >> s) & 1u, kWaitPolls);
+    }
+    // the records of this CTA's rows, a warp a row; the drafted token and its
+    // logit (two dependent loads) of the warp's first row ahead of the barrier
+    const int l0 = rank ? n0 : 0, l1 = rank ? rb - ra : min(n0, rb - ra);
+    bool tok_out = false, in_slice = false;
+    float g = qnan();
+    auto token = [&](int l) {
+        const int r = ra + l;
+        int tok = -1;
+        bool has_tok = true;
+        if (r < p.nd) {
+            tok = __ldg(sp.tokens + r);
+        } else {
+            const int rr = r - p.nd, b = rr / (sp.gamma + 1), j = rr - b * (sp.gamma + 1);
+            has_tok = j < sp.gamma;
+            if (has_tok) tok = __ldg(sp.tokens + static_cast<int64_t>(b) * sp.gamma + j);
+        }
+        tok_out = has_tok && (tok < 0 || tok >= sp.V);
+        in_slice = has_tok && !tok_out && tok >= sp.v0 && tok < sp.v0 + sp.Vs;
+        g = in_slice ? fmax_nan(logit_at<DT>(slice_row_base(p, r), tok - sp.v0), clamp_floor()) : qnan();
+    };
+    if (l0 + warp < l1) token(l0 + warp);
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    for (int l = l0 + warp; l < l1; l += kWarpsPerCta) {
+        const int r = ra + l;
+        const bool drafter = r < p.nd;
+        if (l > l0 + warp) token(l);
+        // the warps that hold its first and last vector
+        const int64_t f = static_cast<int64_t>(l) * RV;
+        const int fw = static_cast<int>(((f + 1) * CW - 1) / Tc), lw = static_cast<int>(((f + RV) * CW - 1) / Tc);
+        const int at = (rank ? (l - n0) - kWarpsPerCta : l) + fw + lane;
+        const bool on = fw + lane <= lw;
+        SoftState a = soft_identity();
+        const unsigned char *piece = slots + at * kSlotBytes;
+        if (on) {
+            const Partial pt = *reinterpret_cast<const Partial *>(piece);
+            a.m = pt.m;
+            a.r = pt.r;
+            a.t2 = pt.t2;
+            a.sh = pt.sh;
+            a.sl = pt.sl;
+            a.amax = pt.amax;
+        }
+        for (int off = 1; off <= lw - fw; off <<= 1) a = soft_merge(a, soft_shfl_down(a, off));   // (lane 0: the row)
+        const uint64_t *list = reinterpret_cast<const uint64_t *>(piece + sizeof(Partial));
+        const int kc = (CAND && !drafter) ? sp.kcap : 0;
+        int head = 0, nc = 0;
+        uint64_t mine = (on && kc > 0) ? list[0] : 0ull, top = 0ull;   // lane k: the row's k-th key
+        for (int k = 0; k < kc; ++k) {
+            const uint64_t best = warp_max_u64(mine);
+            if (best == 0ull) break;
+            ++nc;
+            if (lane == k) top = best;
+            if (mine == best) mine = (++head < kc) ? list[head] : 0ull;   // (unique keys)
+        }
+        sdd_shard_partial *rec = sp.out + r;
+        if (lane == 0) {
+            rec->m = a.m;
+            rec->r = a.r;
+            rec->t2 = a.t2;
+            rec->sh = a.sh;
+            rec->sl = a.sl;
+            rec->amax = (a.amax == INT32_MAX) ? INT32_MAX : sp.v0 + a.amax;
+            rec->g = g;
+            rec->info = (in_slice ? 1 : 0) | (tok_out ? 2 : 0) | (nc << 8);
+        }
+        if (lane < SDD_SHARD_KMAX) {
+            rec->cz[lane] = (top != 0ull) ? cand_value(top) : -INFINITY;
+            rec->cv[lane] = (top != 0ull) ? cand_index(top) : INT32_MAX;
+        }
+    }
+}
+
+}  // namespace
+
+namespace {
+
+// [bf16][candidates]
+void (*const kStream[2][2])(StreamParams) = {{shard_stream_kernel<SDD_F32, false>, shard_stream_kernel<SDD_F32, true>},
+                                             {shard_stream_kernel<SDD_BF16, false>, shard_stream_kernel<SDD_BF16, true>}};
+
+size_t stream_smem(int slots) {
+    return static_cast<size_t>(kScanSmem) + static_cast<size_t>(slots) * kSlotBytes +
+           static_cast<size_t>(kWarpsPerCta) * kCandKeys * sizeof(uint64_t);
+}
+
+// The streaming form's launch facts on the current device.
+struct StreamDev {
+    int clusters, smem;   // clusters of two one-CTA SMs; shared memory of a CTA
+};
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_stream_ready[kMaxDevices];
+StreamDev g_stream_dev[kMaxDevices];
+
+cudaError_t stream_device(StreamDev &out) {
+    int dev = 0, sms = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (!g_stream_ready[dev].load(std::memory_order_acquire)) {
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        for (const auto &row : kStream)
+            for (auto k : row)
+                if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+        if (e != cudaSuccess) return e;
+        g_stream_dev[dev] = StreamDev{sms / 2, optin};
+        g_stream_ready[dev].store(1, std::memory_order_release);
+    }
+    out = g_stream_dev[dev];
+    return cudaSuccess;
+}
+
+// The clusters of the streaming form for `rows` rows of a slice, and a CTA's
+// piece slots; 0 where one CTA per row takes the call: slices of under two
+// tiles a row, whose pieces would be mostly their ends, and batches whose
+// clusters' pieces exceed the shared memory (~900 rows a cluster).  GB300, one
+// CTA per row / streaming, bf16 halves with k = 10: 1 x 32 positions of 75,968
+// entries 35.0 / 11.8 us, 8 x 32 41.6 / 24.0, 64 x 64 315 / 207; 16 x 32 of
+// 4,500 entries 18.0 / 15.8, 1 x 32 13.6 / 11.5.
+int stream_plan(const ShardParams &sp, int64_t rows, const StreamDev &dev, int32_t &slots) {
+    slots = 0;
+    if (dev.clusters < 1 || rows >= (int64_t(1) << 27)) return 0;
+    const int64_t most = (rows + dev.clusters - 1) / dev.clusters;   // rows of a cluster
+    if (sp.RVs < 2 * kTileVec) return 0;
+    // a cluster's rows by cost: at most one ninth more, and a row for the rounding
+    slots = static_cast<int32_t>((most * 10 / 9 + 2) / 2 + 2 + 2 * kWarpsPerCta);
+    return stream_smem(slots) <= static_cast<size_t>(dev.smem) ? dev.clusters : 0;
+}
+
 }  // namespace
 
 cudaError_t launch_shard_partials(const ShardParams &sp, cudaStream_t stream) {
     const int64_t rows = static_cast<int64_t>(sp.B) * (2 * sp.gamma + 1);
     if (rows == 0) return cudaSuccess;
     const bool bf = sp.dtype == SDD_BF16, cand = sp.kcap > 0;
+    StreamDev dev;
+    cudaError_t e = stream_device(dev);
+    if (e != cudaSuccess) return e;
+    StreamParams p;
+    const int clusters = stream_plan(sp, rows, dev, p.slots);
+    if (clusters > 0) {
+        p.sp = sp;
+        p.rows = static_cast<int32_t>(rows);
+        p.nd = sp.B * sp.gamma;
+        p.wait_polls = kWaitPolls;
+        return launch_dependent(kStream[bf][cand], dim3(2 * clusters), dim3(kThreads), stream_smem(p.slots), stream, p);
+    }
     void (*const k)(ShardParams) = bf ? (cand ? shard_partials_kernel<SDD_BF16, true> : shard_partials_kernel<SDD_BF16, false>)
                                       : (cand ? shard_partials_kernel<SDD_F32, true> : shard_partials_kernel<SDD_F32, false>);
     return launch_dependent(k, dim3(static_cast<unsigned>(rows)), dim3(kShardThreads), 0, stream, sp);
