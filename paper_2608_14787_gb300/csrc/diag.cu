@@ -339,6 +339,9 @@ __device__ __forceinline__ void met_stage(const float *q, const int32_t *L, int 
 __global__ void __cluster_dims__(kMetCluster, 1, 1) __launch_bounds__(kMetThreads)
     metrics_kernel(const float *q, const int32_t *L, int B, int gamma, int conditional, double *bce, double *bce_base,
                    double *auroc, int32_t *n_pos, int32_t *n_neg) {
+    // (CTA 0 has started before the others write to its shared memory: the wait
+    // for this arrival is ahead of those writes)
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     griddep_wait();
     const int j = blockIdx.x / kMetCluster, rank = blockIdx.x % kMetCluster;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -409,6 +412,7 @@ __global__ void __cluster_dims__(kMetCluster, 1, 1) __launch_bounds__(kMetThread
     }
     if (lane == 0) s_w[warp] = a;
     __syncthreads();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (tid == 0) {
 #pragma unroll
         for (int w = 1; w < kMetThreads / 32; ++w) {
@@ -426,6 +430,7 @@ __global__ void __cluster_dims__(kMetCluster, 1, 1) __launch_bounds__(kMetThread
         st_cluster_u64(dst + 24, a.gt);
         st_cluster_u64(dst + 32, a.eq);
     }
+    __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (rank == 0 && lane == 0 && warp < 3) {
         // (a warp for each result: their fp64 chains run side by side)
