@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(kThreads, 1) pipe_kernel(const __grid_constant
     }
     constexpr int kTeamWarps = TEAM / 32, kStreamWarps = kWarpsPerCta - kTeamWarps;
     const int warp = threadIdx.x >> 5;
-    if (pp.has_next) scan_warp<DTN, false, kPipeStages, TEAM == kPipeTeam>(pp.next, smem, warp - kTeamWarps, kStreamWarps);
+    if (pp.has_next) scan_warp<DTN, false, kRowsMixed, kPipeStages, TEAM == kPipeTeam>(pp.next, smem, warp - kTeamWarps, kStreamWarps);
 }
 
 using PipeKernel = void (*)(PipeParams);

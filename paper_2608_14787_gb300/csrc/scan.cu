@@ -9,32 +9,38 @@ namespace sdd {
 namespace {
 
 // FEAT: also the five largest logits of every drafter row piece (extended
-// features); the kernel without it is unchanged.
-template <int DT, bool FEAT>
+// features).  KIND: a call over rows of one kind leaves the other's code out.
+template <int DT, bool FEAT, int KIND>
 __global__ void __launch_bounds__(kThreads, 1) scan_kernel(const __grid_constant__ ScanParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     // launched as a programmatic dependent of whatever precedes it in the
     // stream: nothing is read or written before that work has completed
     griddep_wait();
-    scan_warp<DT, FEAT>(p, smem, threadIdx.x >> 5, blockDim.x >> 5);
+    scan_warp<DT, FEAT, KIND>(p, smem, threadIdx.x >> 5, blockDim.x >> 5);
 }
+
+// [bf16][mixed rows, drafter rows, target rows, drafter rows with the extended features]
+void (*const kScanKernels[2][4])(ScanParams) = {
+    {scan_kernel<SDD_F32, false, kRowsMixed>, scan_kernel<SDD_F32, false, kRowsDrafter>,
+     scan_kernel<SDD_F32, false, kRowsTarget>, scan_kernel<SDD_F32, true, kRowsDrafter>},
+    {scan_kernel<SDD_BF16, false, kRowsMixed>, scan_kernel<SDD_BF16, false, kRowsDrafter>,
+     scan_kernel<SDD_BF16, false, kRowsTarget>, scan_kernel<SDD_BF16, true, kRowsDrafter>}};
 
 }  // namespace
 
 int scan_max_ctas_per_sm() {
     int n = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, scan_kernel<SDD_BF16, false>, kThreads, kScanSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, scan_kernel<SDD_BF16, false, kRowsMixed>, kThreads, kScanSmem);
     return n;
 }
 
 // Opt both instantiations in to their dynamic shared memory on the current device.
 cudaError_t scan_prepare_device() {
-    void (*const kernels[])(ScanParams) = {scan_kernel<SDD_BF16, false>, scan_kernel<SDD_F32, false>,
-                                           scan_kernel<SDD_BF16, true>, scan_kernel<SDD_F32, true>};
-    for (auto k : kernels) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
-        if (e != cudaSuccess) return e;
-    }
+    for (const auto &row : kScanKernels)
+        for (auto k : row) {
+            const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kScanSmem);
+            if (e != cudaSuccess) return e;
+        }
     return cudaSuccess;
 }
 
@@ -52,8 +58,8 @@ void set_scan_wait_hooks(uint32_t polls, int drop_copy) {
 
 cudaError_t launch_scan(const ScanParams &p, cudaStream_t stream) {
     const bool bf = p.dtype == SDD_BF16, feat = p.feat != nullptr;
-    void (*const k)(ScanParams) = feat ? (bf ? scan_kernel<SDD_BF16, true> : scan_kernel<SDD_F32, true>)
-                                       : (bf ? scan_kernel<SDD_BF16, false> : scan_kernel<SDD_F32, false>);
+    const int kind = feat ? 3 : p.n_groups > 1 ? kRowsMixed : p.grp[0].kind == 0 ? kRowsDrafter : kRowsTarget;
+    void (*const k)(ScanParams) = kScanKernels[bf][kind];
     ScanParams q = p;
     const uint32_t polls = g_wait_polls.load(std::memory_order_relaxed);
     q.wait_polls = polls ? polls : kWaitPolls;

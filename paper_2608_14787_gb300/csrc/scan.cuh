@@ -417,6 +417,11 @@ struct RowWindow {
     uint32_t flags;     // kRowDrafter, kRowBadTok
 };
 constexpr uint32_t kRowDrafter = 1, kRowBadTok = 2;
+// The kinds of rows in a call (scan_warp).  With one kind known, the streaming
+// loop keeps one form of process_tile (119-121 registers for drafter rows
+// instead of 124-128): GB300, confidence of 16 x 32 rows 32.7 -> 31.2 us, with
+// the extended features 38.2 -> 35.7; of 128 x 32 187 -> 181 and 207 -> 188.
+constexpr int kRowsMixed = 0, kRowsDrafter = 1, kRowsTarget = 2;
 
 // Rows first + lane up to `last`; the token logits are loaded by window_logits.
 __device__ __forceinline__ void window_rows(const ScanParams &p, const PartView &pv, int64_t first, int64_t last,
@@ -460,10 +465,12 @@ __device__ __forceinline__ const char *shfl_ptr(const char *ptr, int src) {
 // ring_bytes(STAGES, n_rings): one ring of STAGES tiles per streaming warp,
 // then their barriers; this warp's is ring w.  FEAT: also the five largest logits of
 // every drafter row piece (extended features); without it the code is
-// unchanged.  SHARES: the warps may have unequal shares (the pipelined round).
-template <int DT, bool FEAT, int STAGES = kStages, bool SHARES = false>
+// unchanged.  KIND: the call's rows are all of one kind (the other kind's code
+// is left out).  SHARES: the warps may have unequal shares (the pipelined round).
+template <int DT, bool FEAT, int KIND = kRowsMixed, int STAGES = kStages, bool SHARES = false>
 __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *smem, int w, int n_rings) {
     constexpr int kStages = STAGES;
+    static_assert(!FEAT || KIND == kRowsDrafter, "the extended features are of drafter rows");
     const int lane = threadIdx.x & 31;
     const PartView pv = part_view(p);
     // the call's warps spread evenly over the CTAs (a call too small for every
@@ -538,6 +545,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
     uint32_t ck[5];        // FEAT: the lane's five largest tile maxima of the piece (keys) ...
     uint32_t ct[5];        // ... fp32: their tiles' numbers in the piece (drafter rows)
     int kb = 0;            // FEAT: the piece's first vector in the row
+    uint32_t ftile = 0u;   // FEAT: the tile's number in the piece
     float s_hi = 0.f, s_lo = 0.f;   // the lane's exp-sum as an fp32 pair
     bool in_piece = false, fresh = false;   // fresh: the piece's token has not been fetched yet
     bool ent = false;      // warp-uniform: drafter row (entropy accumulator, clamped entries)
@@ -560,6 +568,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
                     ct[k] = 0u;
                 }
                 kb = cc.k;
+                ftile = 0u;
             }
             s_hi = 0.f;
             s_lo = 0.f;
@@ -569,7 +578,8 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
             }
             const int at = static_cast<int>(cc.r - win.first);
             crow = shfl_ptr(win.base, at);
-            ent = (__shfl_sync(0xFFFFFFFFu, win.flags, at) & kRowDrafter) != 0;
+            ent = (KIND == kRowsMixed) ? (__shfl_sync(0xFFFFFFFFu, win.flags, at) & kRowDrafter) != 0
+                                       : KIND == kRowsDrafter;
             rank_on = false;
             wrank = 0;
             fresh = true;
@@ -583,9 +593,10 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
         uint4 *tile = reinterpret_cast<uint4 *>(ring + slot * kTileBytes);
         const bool row_end = (cc.k + n == p.RV);
         if (n < kTileVec || (row_end && tail)) pad_tile<DT>(tile, n, lane, row_end, tail);
-        const float cm = ent ? process_tile<DT, true>(tile, cc.k, lane, st, s_hi, s_lo)
+        const float cm = (KIND == kRowsDrafter || (KIND == kRowsMixed && ent))
+                             ? process_tile<DT, true>(tile, cc.k, lane, st, s_hi, s_lo)
                              : process_tile<DT, false>(tile, cc.k, lane, st, s_hi, s_lo);
-        if (FEAT && ent) group_update<DT>(cm, static_cast<uint32_t>(cc.k - kb) / kTileVec, ck, ct);
+        if (FEAT) group_update<DT>(cm, ftile++, ck, ct);
         if (fresh) {
             // the token's logit is first needed here: its load had the first
             // tile's copy and arithmetic to arrive
@@ -593,10 +604,10 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
             tok = __shfl_sync(0xFFFFFFFFu, win.tok, at);
             g = __shfl_sync(0xFFFFFFFFu, win.g, at);
             tok_bad = (__shfl_sync(0xFFFFFFFFu, win.flags, at) & kRowBadTok) != 0;
-            rank_on = !ent && tok >= 0;
+            rank_on = KIND != kRowsDrafter && !ent && tok >= 0;
             fresh = false;
         }
-        if (rank_on) {
+        if (KIND != kRowsDrafter && rank_on) {
             const bool want = cm >= g;
             if (__any_sync(0xFFFFFFFFu, want)) {
                 int c = want ? count_before<DT>(tile, n, cc.k, lane, g, tok) : 0;
@@ -630,7 +641,7 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
                                               : make_uint4(0, 0, 0, 0);
             }
             float top[5];
-            if (FEAT && ent) group_top5<DT>(crow, kb, cc.k, p.V, lane, ck, ct, top);   // (cc.k: the piece's end)
+            if (FEAT) group_top5<DT>(crow, kb, cc.k, p.V, lane, ck, ct, top);   // (cc.k: the piece's end)
             // every reference is a power of two below M's, so the rescaling is
             // exact; each step adds two lanes' double-floats the same way on
             // both, so all lanes agree
@@ -655,14 +666,12 @@ __device__ __forceinline__ void scan_warp(const ScanParams &p, unsigned char *sm
                     if (vec * EPV + e < p.V && vec_elem<DT>(c, e) == M) idx = vec * EPV + e;
             }
             idx = __reduce_min_sync(0xFFFFFFFFu, holds ? idx : INT32_MAX);
-            if (FEAT && ent) {
-                if (lane == 0) {
+            if (FEAT && lane == 0) {
                 FeatPartial fp;
 #pragma unroll
                 for (int k = 0; k < 5; ++k) fp.top[k] = top[k];
                 fp.pad[0] = fp.pad[1] = fp.pad[2] = 0.f;
                 p.feat[cc.r + gw] = fp;
-                }
             }
             if (lane == 0) {
                 Partial pt;
