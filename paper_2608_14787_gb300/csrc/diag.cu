@@ -32,11 +32,10 @@ constexpr uint32_t kPurposePerm = 3;
 // The permutation builder's threads: every phase below is a pass over the n
 // valid blocks between two barriers, so with 256 threads a 2,048-block log
 // takes 8 elements a thread and phase, and seven CTAs (28 KiB each) share an
-// SM.  Bound by issue (72 % of the slots; ~300 warp instructions per 32
-// elements, of which the ten Philox rounds are about 80).  GB300, 2,048 blocks
-// x 32 positions x 100 repetitions: 75 us; with 64 threads a CTA, buckets by a
-// counting sort, ceil(log2 n) pointer-jumping passes and the scores gathered
-// here 265 us.
+// SM.  Bound by issue (72 % of the slots), of which the ten Philox rounds are
+// about a third.  GB300, 2,048 blocks x 32 positions x 100 repetitions: 61 us;
+// with the chains followed by pointer jumping between barriers 75 us; with 64
+// threads a CTA, buckets by a counting sort and the scores gathered here 265 us.
 constexpr int kPermThreads = 256;
 
 // Logs of at most this many blocks are shuffled by the parallel construction
@@ -98,8 +97,13 @@ __global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const int32_t 
     __syncthreads();
     const int n = s_n;
     // the valid blocks in index order (the order defines the draw): block b is
-    // the (s_wpre + popcount)-th of them
+    // the (s_wpre + popcount)-th of them, or the b-th where all are valid
+    const bool all = n == B;
     auto rank_of = [&](int b, bool &valid) {
+        if (all) {
+            valid = true;
+            return b;
+        }
         const uint32_t m = s_mask[b >> 5], bit = 1u << (b & 31);
         valid = (m & bit) != 0;
         return s_wpre[b >> 5] + __popc(m & (bit - 1u));
@@ -124,20 +128,19 @@ __global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const int32_t 
         //   final[0] = P(0).
         // Each bucket is a linked list in any order (one atomic exchange per
         // step); both minima are taken by walking a bucket, whose length is
-        // about ln(n / s), and P follows the "first step above" chains to
-        // their ends by pointer jumping, until no pointer moves (the chains
-        // are about as short as the buckets).
+        // about ln(n / s), and P follows the "first step above" chains, about
+        // as short, to their ends.
         int32_t *s_head = s_rest;                                  // a bucket's first step (0: none; steps are >= 1)
         int16_t *s_list = reinterpret_cast<int16_t *>(s_head + B); // the valid blocks
         int16_t *s_kk = s_list + B;                                // k_a
         int16_t *s_link = s_kk + B;                                // the bucket's next step (0: none)
         int16_t *s_nxt = s_link + B;                               // the bucket's first step above a (0: none)
-        int16_t *s_ptr = s_nxt + B;                                // chain links, then chain ends
+        int16_t *s_ptr = s_nxt + B;                                // chain links (the slot itself at an end)
         for (int b = tid; b < B; b += kPermThreads) {
             s_head[b] = 0;
             bool valid;
             const int t = rank_of(b, valid);
-            if (valid) s_list[t] = static_cast<int16_t>(b);
+            if (valid && !all) s_list[t] = static_cast<int16_t>(b);
         }
         __syncthreads();
         for (int a = 1 + tid; a < n; a += kPermThreads) {
@@ -159,26 +162,20 @@ __global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const int32_t 
             }
         }
         __syncthreads();
-        // (in place: a pointer read during a pass is an earlier or later link
-        // of the same chain, so it never passes the chain's end)
-        for (int more = n > 1; more;) {
-            bool moved = false;
-            for (int t = tid; t < n; t += kPermThreads) {
-                const int p = s_ptr[t], pp = s_ptr[p];
-                if (pp != p) {
-                    s_ptr[t] = static_cast<int16_t>(pp);
-                    moved = true;
-                }
-            }
-            more = __syncthreads_or(moved);
-        }
         for (int b = tid; b < B; b += kPermThreads) {
             bool valid;
             const int a = rank_of(b, valid);
             int src = b;
             if (valid) {
-                const int na = (a > 0) ? s_nxt[a] : 0;
-                src = s_list[(a == 0) ? s_ptr[0] : (na > 0) ? s_ptr[na] : s_kk[a]];
+                // the slot whose first block step a takes: k_a, or the end of
+                // the chain of the bucket's next step (of slot 0 itself)
+                int u = (a > 0) ? s_nxt[a] : 0;
+                if (a > 0 && u == 0) {
+                    u = s_kk[a];
+                } else {
+                    for (int v = s_ptr[u]; v != u; v = s_ptr[u]) u = v;
+                }
+                src = all ? u : s_list[u];
             }
             row[b] = static_cast<uint16_t>(src);
         }
