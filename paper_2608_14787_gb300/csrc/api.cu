@@ -1178,7 +1178,7 @@ static sdd_status_t pipe_params(const sdd_block_args *a, ScanParams &p, bool *em
     // the decide team beside this round's streaming pass (warps 0 .. warp0-1)
     const int team_warps = (p.T * 16 <= kPipeSmallBytes ? kPipeTeamSmall : kPipeTeam) / 32;
     const int wpc = kWarpsPerCta - team_warps;
-    p.W = scan_warps(w.W_max / kWarpsPerCta * wpc, p.T, p.rows);
+    p.W = scan_warps(w.W_max / kWarpsPerCta * wpc, p.T, p.rows, kPipePieces);
     set_divisors(p, kPipeCostDrafter, kPipeCostTarget);
     p.warp0 = team_warps;
     p.wpc = wpc;

@@ -276,16 +276,17 @@ constexpr int64_t kRowStartVec = 400;
 constexpr int64_t kPiecesPerRow = 16;
 constexpr int64_t kWholeMin = 8;
 // The pieces of every row in a call cut into whole pieces, or 0.
-__host__ __device__ inline int64_t whole_pieces(int64_t W_max, int64_t T, int64_t rows) {
+__host__ __device__ inline int64_t whole_pieces(int64_t W_max, int64_t T, int64_t rows, int64_t most) {
     int64_t k = rows > 0 ? W_max / rows : 0;
-    k = k < kPiecesPerRow ? k : kPiecesPerRow;
+    k = k < most ? k : most;
     return (k >= kWholeMin && 2 * rows * k <= T) ? k : 0;
 }
-__host__ __device__ inline int32_t scan_warps(int64_t W_max, int64_t T, int64_t rows) {
-    const int64_t k = whole_pieces(W_max, T, rows);
+__host__ __device__ inline int32_t scan_warps(int64_t W_max, int64_t T, int64_t rows,
+                                              int64_t most = kPiecesPerRow) {
+    const int64_t k = whole_pieces(W_max, T, rows, most);
     if (k > 0) return static_cast<int32_t>(rows * k);
     int64_t w = W_max < T / 2 ? W_max : T / 2;
-    if (w > rows * kPiecesPerRow) w = rows * kPiecesPerRow;
+    if (w > rows * most) w = rows * most;
     return static_cast<int32_t>(w > 1 ? w : 1);
 }
 
@@ -298,6 +299,11 @@ __host__ __device__ inline int32_t scan_warps(int64_t W_max, int64_t T, int64_t 
 // block: 22.8 / 24.2 us), while at 16 blocks the two more streaming warps
 // win (61.2 against 63.5 us).
 constexpr int kPipeTeam = 64, kPipeTeamSmall = 128;
+// Pieces of a row in a pipelined pass at most: the decide team beside it is
+// narrow and bounds a small round, so fewer partials are worth longer pieces
+// (GB300, one 32 x 151,936 bf16 block a round: 8 pieces 16.2 us, 9 16.5, 12
+// 17.8, 16 20.3; one 8 x 32,000 fp32 block 13.5, 13.0, 13.0, 13.1).
+constexpr int64_t kPipePieces = 8;
 constexpr int64_t kPipeSmallBytes = int64_t(64) << 20;
 // The pipelined pass's cost weights (drafter, target vector), as kCostDrafter
 // and kCostTarget for the streaming kernel: on fourteen warps beside the
