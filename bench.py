@@ -5,7 +5,7 @@ confidence statistics of every drafter row, the prefix skip schedule, strict
 (shadow) verification of every block with residual / bonus resampling,
 lenience and top-k acceptance on the same target read, agreement counters and
 the committed tokens.  Rounds over independent batches are pipelined
-(``sdd_block_pipelined``): each launch streams one round's logits and, on four
+(``sdd_block_pipelined``): each launch streams one round's logits and, on the first
 warps of every CTA, finishes the round before; K steps are K launches and one
 closing decide.  The same rounds run unpipelined (``sdd_block_scan`` then
 ``sdd_block_decide``) are reported beside them.
@@ -47,10 +47,10 @@ NEAR = 1e-6
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch on the c3
 # workload, from one ncu capture of the kernel as it stands; reported as the
 # "traffic" of that workload's rooflines only: the streaming kernel
-# (318,294,528 B + 3,656,960 B) and the pipelined round's kernel
-# (328,386,304 B + 3,987,968 B, three rotating input sets).
-SCAN_TRAFFIC_C3 = 321_951_488
-PIPE_TRAFFIC_C3 = 332_374_272
+# (318,332,160 B + 2,773,504 B) and the pipelined round's kernel
+# (328,103,680 B + 2,805,760 B).
+SCAN_TRAFFIC_C3 = 321_105_664
+PIPE_TRAFFIC_C3 = 330_909_440
 
 
 def _peaks():
@@ -388,16 +388,16 @@ def run_gpu(args):
     esz = 2 if wl.dtype == torch.bfloat16 else 4
     scan_bytes = (2 * gamma + 1) * V * esz * B          # every logit read once
     draw_bytes = 2 * V * esz * B                         # the decide's two draw rows per block
-    # (the library runs rounds of at most 512 MiB of logits in the pipelined
+    # (the library runs rounds of at most 1 GiB of logits in the pipelined
     # kernel, larger ones as its streaming and decide kernels; rows padded to
     # 16 bytes)
-    pipelined_kernel = (2 * gamma + 1) * B * (-(-V * esz // 16) * 16) <= (512 << 20)
+    pipelined_kernel = (2 * gamma + 1) * B * (-(-V * esz // 16) * 16) <= (1 << 30)
     stream = torch.cuda.current_stream()
     props = torch.cuda.get_device_properties(dev)
     bus = getattr(props, "pci_bus_id", None)
 
     # A step is one round over one batch.  Rounds over independent batches are
-    # pipelined (sdd_block_pipelined): launch i streams round i and, on four
+    # pipelined (sdd_block_pipelined): launch i streams round i and, on a few
     # warps of each CTA, finishes round i - 1; a last call finishes the last
     # round.  K steps = K launches + that last call, all inside the region.
     def pstep(i):
@@ -572,7 +572,7 @@ def run_gpu(args):
                        "launch": ("pipelined rounds (sdd_block_pipelined): K calls each streaming one round "
                                   "and finishing the one before, + one closing decide, "
                                   + ("in one launch per call (pipe_kernel), " if pipelined_kernel else
-                                     "as the decide and streaming kernels (a round above 512 MiB), ")
+                                     "as the decide and streaming kernels (a round above 1 GiB), ")
                                   + (f"as replays of a CUDA graph of {args.graph} calls" if args.graph
                                      else "queued behind a device spin"))},
             "achieved_gbs_step": ws * scan_bytes / (ms_per_step / 1e3) / 1e9,

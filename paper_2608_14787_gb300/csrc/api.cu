@@ -1157,18 +1157,8 @@ sdd_status_t sdd_block(const sdd_block_args *a, sdd_stream_t stream) {
     return run_decide(p, reinterpret_cast<cudaStream_t>(stream));
 }
 
-// Rounds of at most this many bytes of logits run in the pipelined kernel;
-// larger ones stream on all sixteen warps of each CTA (sdd_block_scan) and are
-// decided by the decide kernel in the next call.  Measured on GB300 (rows of
-// 32 positions over V = 151,936 bf16, blocks/s pipelined kernel / two
-// kernels): B = 16 (316 MB) 257 k / 232 k, B = 24 (474 MB) 274.5 k / 257.4 k,
-// B = 32 (632 MB) 254.9 k / 272.4 k, B = 40 (790 MB) 256.5 k / 282.4 k: the
-// decide kernel's fixed tail matters less as the round grows, while fourteen
-// streaming warps and the decide work beside them trail sixteen warps alone.
-constexpr int64_t kPipeMaxBytes = int64_t(512) << 20;
-
 // A pipelined round's launch parameters: sdd_block's, streamed by warps
-// kPipeWarps..15 of each CTA when the round is at most kPipeMaxBytes (the same
+// behind the decide team's when the round is at most kPipeMaxBytes (the same
 // when the round is streamed and when it is decided).
 static sdd_status_t pipe_params(const sdd_block_args *a, ScanParams &p, bool *empty) {
     SDD_TRY(block_params(a, p, empty));
@@ -1176,14 +1166,16 @@ static sdd_status_t pipe_params(const sdd_block_args *a, ScanParams &p, bool *em
     Work w;
     SDD_TRY(get_work(a->workspace, a->workspace_bytes, a->B, a->gamma, w));
     // the decide team beside this round's streaming pass (warps 0 .. warp0-1)
-    const int team_warps = (p.T * 16 <= kPipeSmallBytes ? kPipeTeamSmall : kPipeTeam) / 32;
+    const int64_t bytes = p.T * 16;
+    const bool wide = bytes <= kPipeSmallBytes || bytes > kPipeMidBytes;
+    const int team_warps = (wide ? kPipeTeamWide : kPipeTeam) / 32;
     const int wpc = kWarpsPerCta - team_warps;
     p.W = scan_warps(w.W_max / kWarpsPerCta * wpc, p.T, p.rows, kPipePieces);
     set_divisors(p, kPipeCostDrafter, kPipeCostTarget);
     p.warp0 = team_warps;
     p.wpc = wpc;
     if (wpc == kShareWarps && p.W == p.ctas * wpc && p.whole == 0) {
-        p.units = p.ctas * kShareCta;   // (C units < 2^53: a round here is at most kPipeMaxBytes)
+        p.units = p.ctas * kShareCta;   // (C units < 2^53: a round here is at most kPipeMidBytes)
         p.divW = make_fastdiv(static_cast<uint64_t>(p.units));
     }
     return SDD_OK;

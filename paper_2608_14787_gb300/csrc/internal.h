@@ -291,20 +291,26 @@ __host__ __device__ inline int32_t scan_warps(int64_t W_max, int64_t T, int64_t 
 }
 
 // The pipelined round (sdd_block_pipelined): the first warps of every CTA (a
-// team of 64 threads, or 128 after a round of at most kPipeSmallBytes of
-// logits) run the previous round's decide work while the others stream.  A
-// round that small is latency-bound: its decide items are few and each takes
-// longer than its streaming pass (GB300, one 32 x 151,936 bf16 block: 23.8
-// us per round with a 128-thread team, 27.9 us with 64; one 8 x 32,000 fp32
-// block: 22.8 / 24.2 us), while at 16 blocks the two more streaming warps
-// win (61.2 against 63.5 us).
-constexpr int kPipeTeam = 64, kPipeTeamSmall = 128;
+// team of 64 or 128 threads, by the size of the round that streams) run the
+// previous round's decide work while the others stream.  In a small round the
+// decide items are longer than the pass beside them, and in a large one again
+// (fewer draw segments to a block, each longer); between them the two more
+// streaming warps win.  Above kPipeMaxBytes the decide kernel's fixed tail
+// matters less than sixteen streaming warps.  GB300, us a round of B blocks of
+// 32 positions over V = 151,936 bf16 (19.75 MB each), team of 128 / 64 / the
+// two kernels in turn: B = 4 22.7 / 25.8 / 30.5, 8 33.4 / 37.0 / 42.1, 10 39.4
+// / 40.2 / 47.2, 12 45.3 / 43.8 / 53.0, 16 57.4 / 54.5 / 64.2, 24 81.5 / 77.5 /
+// 88.1, 27 - / 100.2 / -, 28 94.5 / 101.3 / 101.2, 32 107.5 / 117.5 / 112.6, 48 158.6 / 157.7 /
+// 161.8, 56 186.4 / 246.6 / 188.8, 64 211.8 / 254.8 / 212.0, 80 371 / 659 / 262.
+constexpr int kPipeTeam = 64, kPipeTeamWide = 128;
+constexpr int64_t kPipeSmallBytes = int64_t(200) << 20;   // at most: the wide team
+constexpr int64_t kPipeMidBytes = int64_t(480) << 20;     // at most: the narrow team
+constexpr int64_t kPipeMaxBytes = int64_t(1) << 30;       // at most: the wide team; above: two kernels
 // Pieces of a row in a pipelined pass at most: the decide team beside it is
 // narrow and bounds a small round, so fewer partials are worth longer pieces
 // (GB300, one 32 x 151,936 bf16 block a round: 8 pieces 16.2 us, 9 16.5, 12
 // 17.8, 16 20.3; one 8 x 32,000 fp32 block 13.5, 13.0, 13.0, 13.1).
 constexpr int64_t kPipePieces = 8;
-constexpr int64_t kPipeSmallBytes = int64_t(64) << 20;
 // The pipelined pass's cost weights (drafter, target vector), as kCostDrafter
 // and kCostTarget for the streaming kernel: on fourteen warps beside the
 // decide work the drafter rows' entropy work weighs more (GB300, 16-block

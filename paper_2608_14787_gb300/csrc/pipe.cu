@@ -7,16 +7,13 @@
 // streaming pass it leaves the memory system idle for most of its ~12 us.
 // Rounds over independent batches need not wait for one another, so here the
 // decide work of round n-1 runs beside the streaming pass of round n: in every
-// CTA, the first warps (a team of kPipeTeam = 64 threads; kPipeTeamSmall =
-// 128 when round n is a small, latency-bound one) do one (block, draw
-// segment) item of round n-1's decide work (decide_cta, its barrier over the
-// team only) while the other warps stream round n, the rows divided among
-// them.  Measured on GB300 (16 blocks of 32 positions, V = 151,936 bf16, back
-// to back): 61.2 us per round against 69.0 us for the streaming and decide
-// kernels in turn.  A team of eight decide warps beside eight streaming warps
-// (which then streamed a share cut to its decide time) gave 71-75 us, four
-// decide warps beside twelve 63.5-64.0 us; with two, a decide item takes ~42
-// us under the concurrent stream, still before the streaming warps end.
+// CTA, the first warps (a team of kPipeTeam = 64 threads or kPipeTeamWide = 128,
+// by the size of round n) do one (block, draw segment) item of round n-1's
+// decide work (decide_cta, its barrier over the team only) while the other
+// warps stream round n, the rows divided among them.  Measured on GB300 (16
+// blocks of 32 positions, V = 151,936 bf16, back to back): 54.5 us per round
+// against 64.1 us for the streaming and decide kernels in turn (a team of 128:
+// 57.4); the decide items end after 28-50 us, the streaming warps after 43-57.
 // Round n-1's partials were written by the previous launch on the stream,
 // which has completed when this grid passes griddepcontrol.wait.
 #include <algorithm>
@@ -77,12 +74,12 @@ __global__ void __launch_bounds__(kThreads, 1) pipe_kernel(const __grid_constant
 }
 
 using PipeKernel = void (*)(PipeParams);
-// [next is bf16][prev is bf16][team: kPipeTeam, kPipeTeamSmall]
+// [next is bf16][prev is bf16][team: kPipeTeam, kPipeTeamWide]
 const PipeKernel kPipeKernels[2][2][2] = {
-    {{pipe_kernel<SDD_F32, SDD_F32, kPipeTeam>, pipe_kernel<SDD_F32, SDD_F32, kPipeTeamSmall>},
-     {pipe_kernel<SDD_F32, SDD_BF16, kPipeTeam>, pipe_kernel<SDD_F32, SDD_BF16, kPipeTeamSmall>}},
-    {{pipe_kernel<SDD_BF16, SDD_F32, kPipeTeam>, pipe_kernel<SDD_BF16, SDD_F32, kPipeTeamSmall>},
-     {pipe_kernel<SDD_BF16, SDD_BF16, kPipeTeam>, pipe_kernel<SDD_BF16, SDD_BF16, kPipeTeamSmall>}}};
+    {{pipe_kernel<SDD_F32, SDD_F32, kPipeTeam>, pipe_kernel<SDD_F32, SDD_F32, kPipeTeamWide>},
+     {pipe_kernel<SDD_F32, SDD_BF16, kPipeTeam>, pipe_kernel<SDD_F32, SDD_BF16, kPipeTeamWide>}},
+    {{pipe_kernel<SDD_BF16, SDD_F32, kPipeTeam>, pipe_kernel<SDD_BF16, SDD_F32, kPipeTeamWide>},
+     {pipe_kernel<SDD_BF16, SDD_BF16, kPipeTeam>, pipe_kernel<SDD_BF16, SDD_BF16, kPipeTeamWide>}}};
 
 // The dynamic shared memory a pipelined launch may use on this device (the
 // per-block opt-in limit less the kernels' static shared memory).
@@ -115,21 +112,21 @@ cudaError_t pipe_prepare_device() {
 }
 
 // next: streamed on warps next->warp0..15 (next->warp0 = the decide team's
-// warps: kPipeTeam / 32 or kPipeTeamSmall / 32); grid: next's streaming grid;
+// warps: kPipeTeam / 32 or kPipeTeamWide / 32); grid: next's streaming grid;
 // prev (or null): decided by the team, prev->dec.nseg / seg_vec its blocks'
 // draw segments over that grid for that team (one item per CTA while they
 // fit).
 cudaError_t launch_pipe(const ScanParams *next, const ScanParams *prev, int grid, cudaStream_t stream) {
     const int team = 32 * next->warp0;
-    const int ti = (team == kPipeTeamSmall) ? 1 : 0;
-    if (team != kPipeTeam && team != kPipeTeamSmall) return cudaErrorInvalidValue;
+    const int ti = (team == kPipeTeamWide) ? 1 : 0;
+    if (team != kPipeTeam && team != kPipeTeamWide) return cudaErrorInvalidValue;
     PipeParams pp;
     std::memset(&pp, 0, sizeof pp);
     pp.next = *next;
     pp.has_next = 1;
     pp.next.wait_polls = kWaitPolls;
     pp.next.spread = (next->W + grid - 1) / std::max(grid, 1);
-    size_t smem = static_cast<size_t>(ti ? pipe_rings(kPipeTeamSmall) : pipe_rings(kPipeTeam));
+    size_t smem = static_cast<size_t>(ti ? pipe_rings(kPipeTeamWide) : pipe_rings(kPipeTeam));
     if (prev) {
         pp.prev = *prev;
         pp.has_prev = 1;

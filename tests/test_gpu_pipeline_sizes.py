@@ -1,0 +1,39 @@
+"""The pipelined call at the sizes where its form changes (a decide team of 128
+threads up to 200 MiB of logits and from 480 MiB to 1 GiB, of 64 between, two
+kernels above): chains whose rounds lie on both sides of each line, each
+round's outputs against the same round unpipelined (decisions equal; statistics
+within the rounding that another cut of the rows can make)."""
+import pytest
+import torch
+
+import paper_2608_14787_gb300 as sdd
+from paper_2608_14787_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+WHOLE = ("argmax", "K", "D_out", "L_strict", "tokens_strict", "n_strict", "commit_tokens", "commit_n", "L_topk", "tokens_topk")
+
+
+@pytest.mark.parametrize("sizes", [(10, 11, 10), (25, 26, 25), (54, 55, 3, 54)])
+def test_sizes(sizes):
+    gamma, V = 32, 151936       # 19.75 MB a block: 200 MiB lie between 10 and 11, 480 MiB between 25 and 26, 1 GiB at 54
+    pairs = []
+    for i, B in enumerate(sizes):
+        blk = synth.make_block("c3", device="cuda", B=B, round_=20 + i)
+        two = []
+        for _ in range(2):
+            r = sdd.BlockRound(B, gamma, V, ks=(2,))
+            r.set_inputs(blk.z_d, blk.z_t, blk.x, seed=i, round_=i)
+            two.append(r)
+        pairs.append((two, blk))
+    prev = None
+    for two, _ in pairs:
+        sdd.block_pipelined(two[0], prev)
+        prev = two[0]
+    sdd.block_pipelined(None, prev)
+    for (a, b), _ in pairs:
+        b.run()
+        for n in WHOLE:
+            assert torch.equal(getattr(a, n), getattr(b, n)), n
+        for n in ("q", "maxprob", "entropy"):
+            torch.testing.assert_close(getattr(a, n), getattr(b, n), rtol=2e-6, atol=1e-7)
+        assert int(a.status.item()) == 0
