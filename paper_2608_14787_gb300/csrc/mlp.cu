@@ -14,7 +14,7 @@
 // 128 x 64, B tile 256 x 64, K-major, 128-byte swizzle) filled by 2D TMA, one
 // thread issues tcgen05.mma.kind::f16 (M = 128, N = 256, K = 16) into a
 // 256-column TMEM accumulator; the partial accumulators meet through an L2
-// workspace (stores, one cluster barrier, bulk copies) and CTA q finishes
+// workspace (stores, one cluster barrier, loads) and CTA q finishes
 // output columns [64 q, 64 q + 64) with the fused epilogue.
 // Layers 2-3 of the deep scorer (mlp_tail_kernel): a cluster of four CTAs per
 // tile, each computing 64 output columns of both layers, a2 through the
@@ -227,7 +227,13 @@ __device__ __forceinline__ void mlp_mainloop(unsigned char *smem, uint64_t *full
 // partial to the workspace (L2; distributed shared memory moves these 96 KiB
 // per CTA several times slower), a cluster barrier orders the stores before
 // the loads, and each CTA sums the S partials of its columns in rank order
-// (its own from TMEM) and runs the epilogue.
+// (its own from TMEM) and runs the epilogue.  A thread's loads of the other
+// partials (48 with S = 4, a warp's each 128 contiguous bytes) are in flight
+// together, straight to registers: GB300, 4,096 x 3,584, 13.85 us per call
+// against 14.47 with the partials brought into the idle ring by bulk copies
+// (one more round trip and pass through shared memory; 14.2-14.3 with that
+// form's tighter epilogue).  What bounds it: the main loop's bytes (5.7 us of
+// it, 31 MB), then the chain of the exchange and the GELUs.
 //
 // The A operand is the concatenation [A1 | A2] along K: slices below p.Ka come
 // from tmA, the rest from tmA2 (the scalar features of the deep scorer).
@@ -245,8 +251,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kMlpStages * kStageBytes);
     uint64_t *empty = full + kMlpStages;
     uint64_t *done = empty + kMlpStages;
-    uint64_t *xfer = done + 1;   // the other CTAs' partials of this CTA's columns have landed
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 2);
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
     __shared__ int s_abort;
     __shared__ float s_b1[kMlpN], s_w2[kMlpN];   // epilogue constants, widened once per CTA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -262,7 +267,6 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
             mbar_init(&empty[s], 1);
         }
         mbar_init(done, 1);
-        mbar_init(xfer, 1);
         fence_mbar_init();
         s_abort = 0;
     }
@@ -292,7 +296,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     // column block [q W, (q + 1) W) (W = 256 / S) of all 128 rows: its own
     // partial of the block stays in its TMEM, every other column of its
     // partial goes to ws[tile][q][column][row] (a warp's 32 rows of one column
-    // are 128 contiguous bytes), from where the owner of the column copies it.
+    // are 128 contiguous bytes), from where the owner of the column loads it.
     // Warp w reads TMEM lanes 32 (w % 4) .. + 31 (tile rows); the four warps
     // of a lane quarter share the columns in 16-column chunks.
     constexpr int W = kMlpN / S;
@@ -316,23 +320,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
 #pragma unroll
             for (int j = 0; j < 16; ++j) __stcg(mine + (c + j) * kMlpBM + row, __uint_as_float(v[j]));
         }
-        fence_proxy_async_global();   // the stores, before the bulk copies of the other CTAs read them
         cluster_sync();               // every partial of the tile is in the workspace (release / acquire)
-        if (tid == 0) {
-            // the S - 1 other partials of this CTA's columns (W x 128 fp32, contiguous
-            // in the column-major workspace) into slots of the idle stage ring
-            constexpr uint32_t kBlock = W * kMlpBM * sizeof(float);
-            mbar_arrive_expect_tx(xfer, (S - 1) * kBlock);
-            for (int r = 0; r < S; ++r)
-                if (r != static_cast<int>(rank))
-                    bulk_load(smem_addr(smem + (r - (r > static_cast<int>(rank) ? 1 : 0)) * kBlock),
-                              ws_tile + (static_cast<int64_t>(r) * kMlpN + static_cast<int>(rank) * W) * kMlpBM, kBlock,
-                              smem_addr(xfer));
-        }
     }
-    const bool okx = (S == 1) || __all_sync(0xFFFFFFFFu, mbar_wait_bounded(xfer, 0u, kWaitPolls));
-    if (!okx) s_abort = 1;
-    const float *recv = reinterpret_cast<const float *>(smem);   // [S - 1 other CTAs][W columns][128 rows]
 
     // epilogue: z = the partials summed in rank order, then bias and GELU;
     // this warp's columns [rank W + part W / 4, + W / 4) of its 32 rows
@@ -341,17 +330,23 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
 #pragma unroll 1
     for (int c = static_cast<int>(rank) * W + part * (W / 4); c < static_cast<int>(rank) * W + (part + 1) * (W / 4);
          c += 16) {
+        float rem[S][16];   // the other CTAs' partials: all loads in flight together
+#pragma unroll
+        for (int r = 0; r < S; ++r)
+            if (r != static_cast<int>(rank)) {
+                const float *src = ws_tile + (static_cast<int64_t>(r) * kMlpN + c) * kMlpBM + row;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) rem[r][j] = __ldcg(src + j * kMlpBM);
+            }
         uint32_t own[16];
         tmem_ld16_or0(ok, tbase + c, own);
         float g[16];   // the partials' sum, then the activations
 #pragma unroll
-        for (int r = 0; r < S; ++r) {
-            const bool mine = r == static_cast<int>(rank);
-            const float *src = recv + ((r - (r > static_cast<int>(rank) ? 1 : 0)) * W + c - static_cast<int>(rank) * W) *
-                                          kMlpBM + row;
+        for (int j = 0; j < 16; ++j) {
+            g[j] = 0.f;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float x = mine ? __uint_as_float(own[j]) : src[j * kMlpBM];
+            for (int r = 0; r < S; ++r) {
+                const float x = (r == static_cast<int>(rank)) ? __uint_as_float(own[j]) : rem[r][j];
                 g[j] = (r == 0) ? x : g[j] + x;
             }
         }
@@ -399,7 +394,6 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && s_abort) status_or(p.status, SDD_DEV_TIMEOUT);
-    if (S > 1 && tid == 0 && !okx) (void)mbar_wait_bounded(xfer, 0u, kWaitPolls);   // copies still in flight
     if (p.late_wait) griddep_wait();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
