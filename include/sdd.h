@@ -425,8 +425,9 @@ SDD_API sdd_status_t sdd_scorer_workspace_size(int M, size_t *bytes);
  *   s   [M] fp32 output.
  *   workspace  device scratch of sdd_scorer_workspace_size(M) bytes, 16-byte
  *       aligned (SDD_ERR_INVALID_ARGUMENT if smaller).
- * One launch: 128-position tiles, K split over a cluster of up to four CTAs
- * whose partial products meet in the workspace.  Needs an sm_10x device
+ * One or two launches: whole waves of 128-position tiles, one per SM, in one;
+ * the tiles left over with K split over clusters of up to four CTAs whose
+ * partial products meet in the workspace.  Needs an sm_10x device
  * (returns SDD_ERR_UNSUPPORTED otherwise).  A bounded wait that gives up sets
  * SDD_DEV_TIMEOUT in *status (s is then undefined).
  */

@@ -862,11 +862,11 @@ cudaError_t mlp_prepare(int *sm_count) {
 // How M rows' tiles are run: `full` of them, whole waves of one tile per SM,
 // with K not split (no operand read twice, nothing exchanged), and the `rest`
 // after them with K split S ways, as far as the SMs reach (one wave again; a
-// wave with S = 4, 2, 1 takes 13.5, 18.4 and 33.7 us at K = 3584).  A rest of
+// wave with S = 4, 2, 1 takes 12.8, 17.8 and 33.6 us at K = 3584).  A rest of
 // more than half the SMs runs unsplit too (it is then part of `full`).  GB300,
 // one-layer scorer, K = 3584, against all tiles split four ways: 8,192 rows
-// 18.4 / 26.4 us, 12,000 25.2 / 43.7, 16,384 33.7 / 58.0, 20,000 43.6 / 71.9,
-// 32,768 65.8 / 111.7.
+// 17.8 / 26.4 us, 12,000 25.3 / 43.7, 16,384 33.6 / 58.0, 20,000 42.9 / 71.9,
+// 32,768 65.4 / 111.7.
 struct MlpPlan {
     int full, rest, S;
 };
