@@ -228,11 +228,13 @@ __global__ void __launch_bounds__(kPermThreads) perm_build_kernel(const int32_t 
 // last of which is the logged order.  Neighbouring threads are neighbouring blocks, so a repetition's
 // indices are read in whole lines, and a score is gathered only while the
 // block's local gate holds; the positions go in groups of kPrefixU whose
-// loads are in flight together.  Bound by the gathers' latency.  GB300, 2,048
-// x 32 x 100: 20 us; with a warp per (repetition, block), its lanes on scores
-// 4 B bytes apart, 112 us.
+// loads are in flight together, the indices of a group loaded beside the scores
+// of the one before.  Bound by the gathers' latency.  GB300, 2,048 x 32 x 100:
+// 20 us; with a warp per (repetition, block), its lanes on scores 4 B bytes
+// apart, 112 us.  The whole diagnostic of 512 blocks, groups of 2 / 4 / 8:
+// 31.0 / 31.1 / 31.7 us; with a group's indices loaded before its scores, 4: 33.0.
 constexpr int kPrefixThreads = 256;
-constexpr int kPrefixU = 4;
+constexpr int kPrefixU = 2;
 __global__ void __launch_bounds__(kPrefixThreads) perm_prefix_kernel(const float *q, const uint16_t *pi, int B,
                                                                      int gamma, int n_rep, int signal, df eta_loc,
                                                                      df log_eta_c, unsigned long long *sums) {
@@ -245,15 +247,19 @@ __global__ void __launch_bounds__(kPrefixThreads) perm_prefix_kernel(const float
         int kb = 0, best = 0;   // leading positions passing the local gate; the largest prefix meeting Eq. 3
         bool open = true;
         df S = df{0.f, 0.f};
+        int src[kPrefixU];   // the group's source blocks, loaded a group ahead
+        auto load_src = [&](int j0) {
+#pragma unroll
+            for (int u = 0; u < kPrefixU; ++u)
+                src[u] = (r < n_rep && j0 + u < gamma) ? __ldg(row + static_cast<int64_t>(j0 + u) * B) : b;
+        };
+        load_src(0);
         for (int j0 = 0; j0 < gamma && open; j0 += kPrefixU) {
             float qj[kPrefixU];
 #pragma unroll
-            for (int u = 0; u < kPrefixU; ++u) {
-                const int j = j0 + u;
-                int src = b;
-                if (r < n_rep && j < gamma) src = __ldg(row + static_cast<int64_t>(j) * B);
-                qj[u] = (j < gamma) ? __ldg(q + static_cast<int64_t>(src) * gamma + j) : qnan();
-            }
+            for (int u = 0; u < kPrefixU; ++u)
+                qj[u] = (j0 + u < gamma) ? __ldg(q + static_cast<int64_t>(src[u]) * gamma + j0 + u) : qnan();
+            load_src(j0 + kPrefixU);
 #pragma unroll
             for (int u = 0; u < kPrefixU; ++u) {
                 // (past gamma: NaN closes the gate)
