@@ -55,10 +55,6 @@ struct MlpParams {
     float *ws;              // [tiles][S][256][128] fp32: partial accumulators (column-major per source CTA)
     int32_t *status;
     int32_t tile0;          // the launch's first tile
-    // The launch follows another of the same layer over other tiles: it need
-    // not wait for that one to start, only to end (so that whatever waits for
-    // this launch has waited for both).
-    int32_t late_wait;
 };
 
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
@@ -278,8 +274,9 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     }
     // launched as a programmatic dependent: the setup above overlaps the end
     // of the work ahead in the stream; nothing is read before that completes
-    // (with late_wait the launch ahead waited for it before it let this start)
-    if (!p.late_wait) griddep_wait();
+    // (earlier grids' writes are visible only behind this grid's own wait: the
+    // launch ahead having waited for them promises nothing here)
+    griddep_wait();
     for (int n = tid; n < kMlpN; n += kMlpThreads) {
         s_b1[n] = __ldg(p.b1 + n);
         s_w2[n] = HEAD ? __uint_as_float(static_cast<uint32_t>(__ldg(p.w2 + n)) << 16) : 0.f;
@@ -394,7 +391,6 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && s_abort) status_or(p.status, SDD_DEV_TIMEOUT);
-    if (p.late_wait) griddep_wait();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
 }
@@ -905,9 +901,8 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
     p.ws = ws;
     p.status = status;
     // Tiles [t0, t0 + n) with K split S ways.
-    auto launch = [&](int t0, int n, int S, bool late) {
+    auto launch = [&](int t0, int n, int S) {
         p.tile0 = t0;
-        p.late_wait = late ? 1 : 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(n * S);
         cfg.blockDim = dim3(kMlpThreads);
@@ -929,10 +924,10 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
     };
     const MlpPlan plan = mlp_plan(M, K, sms);
     if (head && plan.full > 0) {
-        e = launch(0, plan.full, 1, false);
+        e = launch(0, plan.full, 1);
         if (e != cudaSuccess) return e;
     }
-    return plan.rest > 0 ? launch(plan.full, plan.rest, plan.S, plan.full > 0) : cudaSuccess;
+    return plan.rest > 0 ? launch(plan.full, plan.rest, plan.S) : cudaSuccess;
 }
 
 }  // namespace

@@ -42,3 +42,25 @@ def test_deep(sdd, M, Kh):
     want = torch.sigmoid(u @ w4.double() + b4)
     assert int(status.item()) == 0 and torch.equal(s, again)
     torch.testing.assert_close(s.double(), want, rtol=0, atol=3e-4)
+
+
+@pytest.mark.parametrize("M", [38 * 128 + 1, 152 * 128 + 1, 157 * 128])
+def test_hidden_states_written_just_before(sdd, M):
+    """Every launch of a call (whole waves of tiles, then the tiles left over) sees what the stream wrote just ahead."""
+    K = 256
+    W1, b1, w2, b2 = synth.make_mlp(device="cuda", hidden=K)
+    w = synth.make_scorer_deep(device="cuda", hidden=K)
+    f = synth.make_features(M, device="cuda")
+    src = [synth.make_hidden(M, device="cuda", seed=s, hidden=K) for s in (3, 4)]
+    want = [(sdd.survival_mlp(h, W1, b1, w2, float(b2)), sdd.scorer_deep(h, f, *w)) for h in src]
+    h = torch.zeros_like(src[0])
+    torch.cuda.synchronize()
+    got = []
+    for i in (0, 1, 0):
+        h.copy_(src[i])
+        s = sdd.survival_mlp(h, W1, b1, w2, float(b2))
+        h.copy_(src[1 - i])
+        got.append((s, i, 0))
+        got.append((sdd.scorer_deep(h, f, *w), 1 - i, 1))
+    for s, i, k in got:
+        assert torch.equal(s, want[i][k])
