@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(done, 0u, kWaitPolls));
     tc_fence_after();
     if (!ok) s_abort = 1;
-    griddep_launch_dependents();   // the next layer's setup and weight loads may start
+    griddep_launch_dependents();   // the next launch may set up (it still waits for this grid)
     const int quarter = warp & 3, part = warp >> 2;
     const int row = quarter * 32 + lane;
     const uint32_t tbase = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
@@ -457,11 +457,6 @@ __global__ void __launch_bounds__(kTailThreads, PAIR ? 2 : 1) mlp_tail_kernel(co
     const uint32_t rank = cluster_rank();
     const int m0 = (p.tile0 + static_cast<int>(blockIdx.x) / kTailCluster) * kMlpBM;
     const int n0 = static_cast<int>(rank) * kTailN;
-    for (int n = tid; n < kTailN; n += kTailThreads) {
-        s_b2[n] = __ldg(p.b2 + n0 + n);
-        s_b3[n] = __ldg(p.b3 + n0 + n);
-        s_w4[n] = __uint_as_float(static_cast<uint32_t>(__ldg(p.w4 + n0 + n)) << 16);
-    }
     if (tid == 0) {
         for (int i = 0; i < 6; ++i) mbar_init(&bar[i], 1);
         fence_mbar_init();
@@ -473,31 +468,35 @@ __global__ void __launch_bounds__(kTailThreads, PAIR ? 2 : 1) mlp_tail_kernel(co
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-
     auto load_w3 = [&] {
         mbar_arrive_expect_tx(fullW3, kTailW);
         for (int c = 0; c < kTailSlices; ++c)
             tma_load_2d(smem_addr(bufW3 + c * kTailWSlice), &tmW3, c * kMlpBK, n0, smem_addr(fullW3));
     };
-    if (tid == 0) {
-        // the weights do not depend on the first layer: loaded while it finishes
-        mbar_arrive_expect_tx(fullW2, kTailW);
-        for (int c = 0; c < kTailSlices; ++c)
-            tma_load_2d(smem_addr(bufW2 + c * kTailWSlice), &tmW2, c * kMlpBK, n0, smem_addr(fullW2));
-        if (!PAIR) load_w3();
-    }
     // launched as a programmatic dependent of the first layer: a1 (and the
-    // workspace, which a2 overwrites) only once that grid has completed
+    // workspace, which a2 overwrites) only once that grid has completed, and
+    // the weights too, which a grid ahead of it may have written
     griddep_wait();
     if (tid == 0) {
         mbar_arrive_expect_tx(fullA, kTailA);
-        for (int c = 0; c < kTailSlices; ++c)
+        mbar_arrive_expect_tx(fullW2, kTailW);
+        for (int c = 0; c < kTailSlices; ++c) {
             tma_load_2d(smem_addr(bufA + c * kTailASlice), &tmAct, c * kMlpBK, m0, smem_addr(fullA));
-    } else if (warp == 1 && lane == 0) {
+            tma_load_2d(smem_addr(bufW2 + c * kTailWSlice), &tmW2, c * kMlpBK, n0, smem_addr(fullW2));
+        }
+        if (!PAIR) load_w3();
+    }
+    for (int n = tid; n < kTailN; n += kTailThreads) {
+        s_b2[n] = __ldg(p.b2 + n0 + n);
+        s_b3[n] = __ldg(p.b3 + n0 + n);
+        s_w4[n] = __uint_as_float(static_cast<uint32_t>(__ldg(p.w4 + n0 + n)) << 16);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 1 && lane == 0) {
         const bool okA = mbar_wait_bounded(fullA, 0u, kWaitPolls), okB = mbar_wait_bounded(fullW2, 0u, kWaitPolls);
         if (okA && okB) {
             tc_fence_after();

@@ -64,3 +64,23 @@ def test_hidden_states_written_just_before(sdd, M):
         got.append((sdd.scorer_deep(h, f, *w), 1 - i, 1))
     for s, i, k in got:
         assert torch.equal(s, want[i][k])
+
+
+@pytest.mark.parametrize("M", [128, 38 * 128 + 1, 152 * 128 + 1])
+def test_weights_written_just_before(sdd, M):
+    """Every layer's launch sees weights and biases that the stream wrote just ahead of the call."""
+    K = 256
+    h, f = synth.make_hidden(M, device="cuda", seed=3, hidden=K), synth.make_features(M, device="cuda")
+    src = [synth.make_scorer_deep(device="cuda", hidden=K, seed=s) for s in (1, 2)]
+    want = [sdd.scorer_deep(h, f, *w) for w in src]
+    w = [t.clone() if torch.is_tensor(t) else t for t in src[0]]
+    torch.cuda.synchronize()
+    got = []
+    for i in (1, 0, 1):
+        for dst, new in zip(w, src[i]):
+            if torch.is_tensor(dst):
+                dst.copy_(new)
+        w[-1] = src[i][-1]
+        got.append((sdd.scorer_deep(h, f, *w), i))
+    for s, i in got:
+        assert torch.equal(s, want[i])
