@@ -21,7 +21,8 @@
 // workspace and back by TMA.
 // Larger batches (mlp_plan): whole waves of one tile per SM run unsplit
 // (mlp_kernel with S = 1; the deep scorer all layers in one CTA,
-// mlp_deep_kernel), the tiles left over as above with S = 4 or 2.
+// mlp_deep_kernel), the tiles left over as above with S = 4 or 2.  However its
+// tile is run, a row's sum over K is taken in the same chains (kMlpChains).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -37,12 +38,24 @@ constexpr int kMlpN = 256;           // hidden units = UMMA N
 constexpr int kMlpBM = 128;          // rows per CTA = UMMA M
 constexpr int kMlpBK = 64;           // K per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kMlpStages = 4;
-constexpr int kMlpThreads = 512;     // warp 0 lane 0: TMA producer; warp 1 lane 0: MMA issuer; all: epilogue
+// Warps 0-15: epilogue.  The TMA producer is lane 0 of warp kRole, the MMA
+// issuer lane 0 of the next: epilogue warps, or warps of their own where the
+// epilogue warps read finished chains (kMlpChains) beside the main loop.
+constexpr int kMlpThreads = 512, kMlpThreadsChains = kMlpThreads + 64;
 constexpr uint32_t kATileBytes = kMlpBM * kMlpBK * 2;   // 16 KiB
 constexpr uint32_t kBTileBytes = kMlpN * kMlpBK * 2;    // 32 KiB
 constexpr uint32_t kStageBytes = kATileBytes + kBTileBytes;
 constexpr int kMlpSmem = kMlpStages * kStageBytes + 1024 + 256;   // + alignment slack + barriers
 constexpr uint32_t kTmemCols = 256;
+// A tile's sum over K is taken in up to this many chains (quarters of K), each
+// accumulated by the tensor cores from zero, added in fp32 in their order: a
+// CTA of S splits takes kMlpChains / S of them.  The tensor cores' fp32
+// accumulation loses about in proportion to a chain's length: error of the
+// scores against 64 bits (2-norm), K = 3584: one chain 3.9e-7, two 1.9e-7, four
+// 0.98e-7; K = 2048: 2.2e-7, 1.1e-7, 0.66e-7.  Four against one chain cost
+// (S = 1) 28.0 against 27.4 us at 12,000 rows, 33.1 / 32.9 at 16,384, 35.4 /
+// 35.4 at 19,456, and two against one (S = 2) 20.4 / 20.1 at 8,192.
+constexpr int kMlpChains = 4;
 
 struct MlpParams {
     int32_t M, K;
@@ -111,6 +124,15 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
         : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
+// 16 consecutive fp32 columns into this thread's TMEM lane.
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const float *v) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+        "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "f"(v[8]), "f"(v[9]),
+        "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]), "f"(v[15])
+        : "memory");
+}
 // 16 columns of this thread's TMEM lane, or zeros when the accumulator is not valid.
 __device__ __forceinline__ void tmem_ld16_or0(bool ok, uint32_t taddr, uint32_t (&v)[16]) {
     if (ok) {
@@ -162,14 +184,18 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 __device__ __forceinline__ float gelu_erf(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 
 // The first layer's main loop over K slices [kt0, kt0 + nk) of the tile at row
-// m0: warp 0 lane 0 fills the ring, warp 1 lane 0 issues the products into the
-// 256 TMEM columns at tmem; `done` completes with the accumulator.  The ring
-// is idle when both lanes have left (once `done` has completed).
+// m0, in C chains (chain c: slices [c nk / C, (c + 1) nk / C), into the 256 TMEM
+// columns at tmem + 256 (c & 1)).  Warp ROLE lane 0 fills the ring, the next
+// warp's lane 0 issues the products; done[c] completes with chain c, and chain
+// c >= 2 starts once drained[c - 2] says that its columns have been read.  The
+// ring is idle when both lanes have left (once the last chain has completed).
+template <int ROLE>
 __device__ __forceinline__ void mlp_mainloop(unsigned char *smem, uint64_t *full, uint64_t *empty, uint64_t *done,
-                                             const CUtensorMap *tmA, const CUtensorMap *tmA2, const CUtensorMap *tmB,
-                                             int Ka, int m0, int kt0, int nk, uint32_t tmem, int *s_abort) {
+                                             uint64_t *drained, const CUtensorMap *tmA, const CUtensorMap *tmA2,
+                                             const CUtensorMap *tmB, int Ka, int m0, int kt0, int nk, int C,
+                                             uint32_t tmem, int *s_abort) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp == 0 && lane == 0) {
+    if (warp == ROLE && lane == 0) {
         // TMA producer: stage s holds K slice kt0 + t of the A tile (rows
         // m0..m0+127) and of the B tile (all 256 hidden units)
         int t = 0;
@@ -195,25 +221,72 @@ __device__ __forceinline__ void mlp_mainloop(unsigned char *smem, uint64_t *full
             const int last = ((t - 1 - s) / kMlpStages) * kMlpStages + s;
             (void)mbar_wait_bounded(&full[s], static_cast<uint32_t>(last / kMlpStages) & 1u, kWaitPolls);
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == ROLE + 1 && lane == 0) {
         // MMA issuer: four K = 16 steps per stage, the 128-byte rows advanced
         // by 32 bytes per step
-        for (int t = 0; t < nk; ++t) {
-            const int s = t % kMlpStages;
-            const uint32_t ph = static_cast<uint32_t>(t / kMlpStages) & 1u;
-            if (!mbar_wait_bounded(&full[s], ph, kWaitPolls)) {
-                *s_abort = 1;
-                break;
+        bool ok = true;
+        int t = 0;
+        for (int c = 0; c < C; ++c) {
+            const int first = t, end = (c + 1) * nk / C;
+            const uint32_t d = tmem + (c & 1) * kTmemCols;
+            if (ok && c >= 2) {
+                ok = mbar_wait_bounded(&drained[c - 2], 0u, kWaitPolls);
+                tc_fence_after();
             }
-            tc_fence_after();
-            const uint32_t a = smem_addr(smem + s * kStageBytes), b = a + kATileBytes;
+            for (; ok && t < end; ++t) {
+                const int s = t % kMlpStages;
+                const uint32_t ph = static_cast<uint32_t>(t / kMlpStages) & 1u;
+                if (!mbar_wait_bounded(&full[s], ph, kWaitPolls)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t a = smem_addr(smem + s * kStageBytes), b = a + kATileBytes;
 #pragma unroll
-            for (int kk = 0; kk < kMlpBK / 16; ++kk)
-                umma_f16(tmem, umma_desc_sw128(a + kk * 32), umma_desc_sw128(b + kk * 32), (t | kk) != 0 ? 1u : 0u);
-            umma_commit(smem_addr(&empty[s]));   // the stage is free once these MMAs have read it
+                for (int kk = 0; kk < kMlpBK / 16; ++kk)
+                    umma_f16(d, umma_desc_sw128(a + kk * 32), umma_desc_sw128(b + kk * 32),
+                             (t != first || kk != 0) ? 1u : 0u);
+                umma_commit(smem_addr(&empty[s]));   // the stage is free once these MMAs have read it
+            }
+            umma_commit(smem_addr(&done[c]));        // the chain is complete (at once when nothing was issued)
         }
-        umma_commit(smem_addr(done));            // the accumulator is complete
+        if (!ok) *s_abort = 1;
     }
+}
+
+// The chains of a CTA that takes the whole of K, added in order by the epilogue
+// warps while the later ones run: warp w its 32 TMEM lanes (tlane) and columns
+// [64 (w / 4), + 64), the sum left in the first 256 columns.  Every warp of the
+// CTA calls it; epi: the epilogue warps.  False when a wait gave up.
+__device__ __forceinline__ bool mlp_drain(uint64_t *done, uint64_t *drained, int C, bool epi, uint32_t tlane, int part) {
+    bool ok = true;
+    float acc[64];
+#pragma unroll
+    for (int j = 0; j < 64; ++j) acc[j] = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < C && ok; ++c) {
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&done[c], 0u, kWaitPolls));
+        tc_fence_after();
+        if (!ok || !epi || C == 1) continue;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint32_t v[16];
+            tmem_ld16(tlane + (c & 1) * kTmemCols + part * 64 + 16 * q, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) acc[16 * q + j] += __uint_as_float(v[j]);
+        }
+        if (c + 2 < C) {   // a later chain takes these columns
+            tc_fence_before();
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) mbar_arrive(&drained[c]);
+        }
+    }
+    if (ok && epi && C > 1) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tmem_st16(tlane + part * 64 + 16 * q, acc + 16 * q);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+    }
+    return ok;
 }
 
 // Grid: (M tiles x S) CTAs in clusters of S along x (S = 1, 2 or 4 splits of
@@ -236,8 +309,11 @@ __device__ __forceinline__ void mlp_mainloop(unsigned char *smem, uint64_t *full
 // HEAD: the epilogue fuses GELU, the w2 dot product and the sigmoid (one
 // float per row); otherwise it writes the layer's activations GELU(z + b1)
 // as bf16 rows of p.act for the next layer.
+// The CTA's K is taken in 4 / S chains (as its slices allow): S = 2 adds its two
+// where it reads them, S = 1 its four beside the main loop (mlp_drain).
+__host__ __device__ constexpr int mlp_threads(int S) { return S == 1 ? kMlpThreadsChains : kMlpThreads; }
 template <int S, bool HEAD>
-__global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(mlp_threads(S), 1) mlp_kernel(const __grid_constant__ CUtensorMap tmA,
                                                             const __grid_constant__ CUtensorMap tmA2,
                                                             const __grid_constant__ CUtensorMap tmB,
                                                             const __grid_constant__ MlpParams p) {
@@ -246,8 +322,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
                                                             ~static_cast<uintptr_t>(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kMlpStages * kStageBytes);
     uint64_t *empty = full + kMlpStages;
-    uint64_t *done = empty + kMlpStages;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(done + 1);
+    uint64_t *done = empty + kMlpStages;      // a barrier a chain
+    uint64_t *drained = done + kMlpChains;    // [kMlpChains - 2]
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drained + kMlpChains - 2);
+    constexpr int kRole = S == 1 ? kMlpThreads / 32 : 0;
+    constexpr uint32_t kCols = S < kMlpChains ? 2 * kTmemCols : kTmemCols;
     __shared__ int s_abort;
     __shared__ float s_b1[kMlpN], s_w2[kMlpN];   // epilogue constants, widened once per CTA
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -256,19 +335,17 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     const int slices = p.K / kMlpBK;
     const int kt0 = static_cast<int>(rank) * slices / S;                // K slices of this CTA
     const int nk = (static_cast<int>(rank) + 1) * slices / S - kt0;
+    const int C = min(kMlpChains / S, nk);
 
     if (tid == 0) {
-        for (int s = 0; s < kMlpStages; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        mbar_init(done, 1);
+        for (int i = 0; i < 2 * kMlpStages + kMlpChains; ++i) mbar_init(&full[i], 1);
+        for (int i = 0; i < kMlpChains - 2; ++i) mbar_init(&drained[i], kMlpThreads / 32);
         fence_mbar_init();
         s_abort = 0;
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
-                     "r"(kTmemCols)
+                     "r"(kCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -277,7 +354,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     // (earlier grids' writes are visible only behind this grid's own wait: the
     // launch ahead having waited for them promises nothing here)
     griddep_wait();
-    for (int n = tid; n < kMlpN; n += kMlpThreads) {
+    for (int n = tid; n < kMlpN; n += mlp_threads(S)) {
         s_b1[n] = __ldg(p.b1 + n);
         s_w2[n] = HEAD ? __uint_as_float(static_cast<uint32_t>(__ldg(p.w2 + n)) << 16) : 0.f;
     }
@@ -286,7 +363,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    mlp_mainloop(smem, full, empty, done, &tmA, &tmA2, &tmB, p.Ka, m0, kt0, nk, tmem, &s_abort);
+    mlp_mainloop<kRole>(smem, full, empty, done, drained, &tmA, &tmA2, &tmB, p.Ka, m0, kt0, nk, C, tmem, &s_abort);
     __syncwarp();
 
     // Exchange through the workspace.  CTA q of the cluster finishes the
@@ -297,13 +374,29 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     // Warp w reads TMEM lanes 32 (w % 4) .. + 31 (tile rows); the four warps
     // of a lane quarter share the columns in 16-column chunks.
     constexpr int W = kMlpN / S;
-    const bool ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(done, 0u, kWaitPolls));
-    tc_fence_after();
-    if (!ok) s_abort = 1;
-    griddep_launch_dependents();   // the next launch may set up (it still waits for this grid)
-    const int quarter = warp & 3, part = warp >> 2;
+    const int quarter = warp & 3, part = warp >> 2;   // (part 4: the producer's and the issuer's warps of S = 1)
+    const bool epi = warp < kMlpThreads / 32;
     const int row = quarter * 32 + lane;
     const uint32_t tbase = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
+    bool ok;
+    if (S == 1) {
+        ok = mlp_drain(done, drained, C, epi, tbase, part);
+    } else {   // (the last chain's products end after the first's)
+        ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&done[C - 1], 0u, kWaitPolls));
+        tc_fence_after();
+    }
+    // 16 columns of this CTA's sum
+    auto own16 = [&](int c, uint32_t (&v)[16]) {
+        tmem_ld16_or0(ok, tbase + c, v);
+        if (S == 2 && C == 2) {
+            uint32_t w[16];
+            tmem_ld16_or0(ok, tbase + kTmemCols + c, w);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(__uint_as_float(v[j]) + __uint_as_float(w[j]));
+        }
+    };
+    if (!ok) s_abort = 1;
+    griddep_launch_dependents();   // the next launch may set up (it still waits for this grid)
     float *ws_tile = p.ws + static_cast<int64_t>(blockIdx.x / S) * S * kMlpN * kMlpBM;
     if (S > 1) {
         float *mine = ws_tile + static_cast<int64_t>(rank) * kMlpN * kMlpBM;
@@ -313,7 +406,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
             if (c / W == static_cast<int>(rank)) continue;
             if ((idx++ & 3) != part) continue;
             uint32_t v[16];
-            tmem_ld16_or0(ok, tbase + c, v);
+            own16(c, v);
 #pragma unroll
             for (int j = 0; j < 16; ++j) __stcg(mine + (c + j) * kMlpBM + row, __uint_as_float(v[j]));
         }
@@ -323,10 +416,10 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     // epilogue: z = the partials summed in rank order, then bias and GELU;
     // this warp's columns [rank W + part W / 4, + W / 4) of its 32 rows
     const int grow = m0 + row;
-    float t2 = 0.f;   // HEAD: this thread's part of the w2 dot product
+    float t2 = 0.f;   // HEAD: this thread's part of the w2 dot product, a sum of 16 columns at a time
 #pragma unroll 1
-    for (int c = static_cast<int>(rank) * W + part * (W / 4); c < static_cast<int>(rank) * W + (part + 1) * (W / 4);
-         c += 16) {
+    for (int c = static_cast<int>(rank) * W + part * (W / 4);
+         epi && c < static_cast<int>(rank) * W + (part + 1) * (W / 4); c += 16) {
         float rem[S][16];   // the other CTAs' partials: all loads in flight together
 #pragma unroll
         for (int r = 0; r < S; ++r)
@@ -336,7 +429,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
                 for (int j = 0; j < 16; ++j) rem[r][j] = __ldcg(src + j * kMlpBM);
             }
         uint32_t own[16];
-        tmem_ld16_or0(ok, tbase + c, own);
+        own16(c, own);
         float g[16];   // the partials' sum, then the activations
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
@@ -347,12 +440,14 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
                 g[j] = (r == 0) ? x : g[j] + x;
             }
         }
+        float t = 0.f;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             const int n = c + j;
             g[j] = gelu_erf(g[j] + s_b1[n]);
-            if (HEAD) t2 = fmaf(s_w2[n], g[j], t2);
+            if (HEAD) t = fmaf(s_w2[n], g[j], t);
         }
+        t2 += t;
         if (!HEAD && ok && grow < p.M) {
             // 16 bf16 activations (round to nearest even) in two 16-byte stores
             uint32_t w[8];
@@ -368,7 +463,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
         // the S column blocks in rank order (CTA 0 of the cluster finishes)
         __shared__ float s_part[3][kMlpBM];
         __shared__ float s_head[S][kMlpBM];
-        if (part > 0) s_part[part - 1][row] = t2;
+        if (epi && part > 0) s_part[part - 1][row] = t2;
         __syncthreads();
         if (part == 0) {
             const float t = ((t2 + s_part[0][row]) + s_part[1][row]) + s_part[2][row];
@@ -392,7 +487,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_kernel(const __grid_consta
     __syncthreads();
     if (tid == 0 && s_abort) status_or(p.status, SDD_DEV_TIMEOUT);
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
 }
 
 // ---------------------------------------------------------------------------
@@ -599,19 +694,21 @@ __global__ void __launch_bounds__(kTailThreads, PAIR ? 2 : 1) mlp_tail_kernel(co
 
 // ---------------------------------------------------------------------------
 // The deep scorer of one 128-row tile in one CTA (whole waves of tiles): the
-// first layer with K not split, then layers 2 and 3 and the head without a1,
-// a2 or partial sums leaving the SM.  After the main loop the ring's 192 KiB
+// first layer with K in kMlpChains chains, then layers 2 and 3 and the head
+// without a2 or partial sums leaving the SM; every sum in the order of the
+// split form, so that a row's score does not depend on the batch.  After the main loop the ring's 192 KiB
 // hold the activations (64 KiB, written by the epilogues in the operands'
 // swizzled layout) and one 256 x 256 weight matrix (128 KiB: W2 as soon as the
 // main loop's products have read the ring, W3 once layer 2's have read W2,
 // each under the epilogue before it).  TMEM columns 0-255 hold z1, 256-511 z2,
-// 0-255 z3.  a1 is also written to p.act.
+// 0-255 z3 (and the main loop's chains all of them in turn).  a1 is also written to
+// p.act.
 //
 // Bound by the main loop's operands (2.9 MB into each SM, ~22 us) and then by
-// the issue of 3 x 32 K erf-form GELUs an SM.  GB300, K = 3584 + 256: 50.9 us
+// the issue of 3 x 32 K erf-form GELUs an SM.  GB300, K = 3584 + 256: 51.7 us
 // for 128 tiles (16,384 rows) against 93.8 us with K split four ways, clusters
 // of four and a second launch for the tail (61.4 us with K not split and the
-// tail in a second launch); 20,000 rows 69.3 against 116 us.
+// tail in a second launch); 20,000 rows 71.7 against 116 us.
 // ---------------------------------------------------------------------------
 struct DeepParams {
     int32_t M, K, Ka, tile0;
@@ -631,7 +728,7 @@ __device__ __forceinline__ unsigned char *act_chunk(unsigned char *buf, int row,
     return buf + (c8 >> 3) * kTailASlice + row * 128 + (((c8 & 7) ^ (row & 7)) << 4);
 }
 
-__global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_constant__ CUtensorMap tmA,
+__global__ void __launch_bounds__(kMlpThreadsChains, 1) mlp_deep_kernel(const __grid_constant__ CUtensorMap tmA,
                                                                  const __grid_constant__ CUtensorMap tmA2,
                                                                  const __grid_constant__ CUtensorMap tmB,
                                                                  const __grid_constant__ CUtensorMap tmW2,
@@ -643,9 +740,10 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
     unsigned char *bufA = smem, *bufW = smem + kTailA;
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kMlpStages * kStageBytes);
     uint64_t *empty = full + kMlpStages;
-    uint64_t *done = empty + kMlpStages;   // z1, then z2, z3
-    uint64_t *fullW = done + 3;            // W2, W3
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(fullW + 2);
+    uint64_t *done = empty + kMlpStages;   // z1's chains, then z2, z3
+    uint64_t *fullW = done + kMlpChains + 2;   // W2, W3
+    uint64_t *drained = fullW + 2;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drained + kMlpChains - 2);
     __shared__ int s_abort;
     __shared__ float s_b[3][kMlpN], s_w4[kMlpN];
     __shared__ float s_part[3][kMlpBM];
@@ -653,7 +751,8 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
     const int m0 = (p.tile0 + static_cast<int>(blockIdx.x)) * kMlpBM;
 
     if (tid == 0) {
-        for (int i = 0; i < 2 * kMlpStages + 5; ++i) mbar_init(&full[i], 1);
+        for (int i = 0; i < 2 * kMlpStages + kMlpChains + 4; ++i) mbar_init(&full[i], 1);
+        for (int i = 0; i < kMlpChains - 2; ++i) mbar_init(&drained[i], kMlpThreads / 32);
         fence_mbar_init();
         s_abort = 0;
     }
@@ -664,7 +763,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     griddep_wait();
-    for (int n = tid; n < kMlpN; n += kMlpThreads) {
+    for (int n = tid; n < kMlpN; n += kMlpThreadsChains) {
         s_b[0][n] = __ldg(p.b1 + n);
         s_b[1][n] = __ldg(p.b2 + n);
         s_b[2][n] = __ldg(p.b3 + n);
@@ -674,11 +773,13 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    mlp_mainloop(smem, full, empty, done, &tmA, &tmA2, &tmB, p.Ka, m0, 0, p.K / kMlpBK, tmem, &s_abort);
+    const int nk = p.K / kMlpBK, C = min(kMlpChains, nk);
+    mlp_mainloop<kMlpThreads / 32>(smem, full, empty, done, drained, &tmA, &tmA2, &tmB, p.Ka, m0, 0, nk, C, tmem, &s_abort);
     __syncwarp();
 
     // warp w: TMEM lanes 32 (w % 4) .. + 31 (tile rows), columns 64 (w / 4) .. + 63
     const int quarter = warp & 3, part = warp >> 2;
+    const bool epi = warp < kMlpThreads / 32;
     const int row = quarter * 32 + lane, grow = m0 + row;
     const uint32_t tlane = tmem + (static_cast<uint32_t>(quarter * 32) << 16);
     bool ok = true;
@@ -687,8 +788,12 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
 #pragma unroll 1
     for (int layer = 0; layer < 3; ++layer) {
         // z of this layer is complete, and its products have read their operands
-        ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&done[layer], 0u, kWaitPolls)) && ok;
-        tc_fence_after();
+        if (layer == 0) {
+            ok = mlp_drain(done, drained, C, epi, tlane, part);
+        } else {
+            ok = __all_sync(0xFFFFFFFFu, mbar_wait_bounded(&done[kMlpChains + layer - 1], 0u, kWaitPolls)) && ok;
+            tc_fence_after();
+        }
         if (!ok) s_abort = 1;
         if (layer == 0) {
             // (every warp: a CTA's threads have all passed the main loop)
@@ -705,15 +810,17 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
         const uint32_t z = tlane + (layer == 1 ? kTmemCols : 0u) + part * 64;
         const float *bias = s_b[layer];
 #pragma unroll 1
-        for (int c = 0; c < 64; c += 16) {
+        for (int c = 0; epi && c < 64; c += 16) {
             uint32_t v[16];
             tmem_ld16_or0(ok, z + c, v);
             float g[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) g[j] = gelu_erf(__uint_as_float(v[j]) + bias[part * 64 + c + j]);
             if (layer == 2) {
+                float d = 0.f;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) t = fmaf(s_w4[part * 64 + c + j], g[j], t);
+                for (int j = 0; j < 16; ++j) d = fmaf(s_w4[part * 64 + c + j], g[j], d);
+                t += d;   // (16 columns at a time, as the tail kernel's warps)
                 continue;
             }
             uint32_t w[8];
@@ -746,11 +853,11 @@ __global__ void __launch_bounds__(kMlpThreads, 1) mlp_deep_kernel(const __grid_c
             } else {
                 s_abort = 1;
             }
-            umma_commit(smem_addr(&done[layer + 1]));   // (arrives at once when nothing was issued)
+            umma_commit(smem_addr(&done[kMlpChains + layer]));   // (arrives at once when nothing was issued)
         }
         __syncwarp();
     }
-    if (part > 0) s_part[part - 1][row] = t;
+    if (epi && part > 0) s_part[part - 1][row] = t;
     tc_fence_before();
     __syncthreads();
     if (part == 0 && ok && grow < p.M) {
@@ -857,11 +964,11 @@ cudaError_t mlp_prepare(int *sm_count) {
 // How M rows' tiles are run: `full` of them, whole waves of one tile per SM,
 // with K not split (no operand read twice, nothing exchanged), and the `rest`
 // after them with K split S ways, as far as the SMs reach (one wave again; a
-// wave with S = 4, 2, 1 takes 12.8, 17.8 and 33.6 us at K = 3584).  A rest of
+// wave with S = 4, 2, 1 takes 13.7, 20.3 and 35.4 us at K = 3584).  A rest of
 // more than half the SMs runs unsplit too (it is then part of `full`).  GB300,
-// one-layer scorer, K = 3584, against all tiles split four ways: 8,192 rows
-// 17.8 / 26.4 us, 12,000 25.3 / 43.7, 16,384 33.6 / 58.0, 20,000 42.9 / 71.9,
-// 32,768 65.4 / 111.7.
+// one-layer scorer, K = 3584, three inputs in turn, against all tiles split four
+// ways: 8,192 rows 20.3 / 28.9 us, 12,000 28.2 / 43.7, 16,384 33.3 / 58.0,
+// 20,000 44.9 / 71.9, 32,768 64.4 / 111.9.
 struct MlpPlan {
     int full, rest, S;
 };
@@ -904,7 +1011,7 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
         p.tile0 = t0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(n * S);
-        cfg.blockDim = dim3(kMlpThreads);
+        cfg.blockDim = dim3(mlp_threads(S));
         cfg.dynamicSmemBytes = kMlpSmem;
         cfg.stream = stream;
         cudaLaunchAttribute attr[2];
@@ -978,7 +1085,7 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
         d.status = status;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(plan.full);
-        cfg.blockDim = dim3(kMlpThreads);
+        cfg.blockDim = dim3(kMlpThreadsChains);
         cfg.dynamicSmemBytes = kMlpSmem;
         cfg.stream = stream;
         cudaLaunchAttribute attr[1];

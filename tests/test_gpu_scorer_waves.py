@@ -1,7 +1,9 @@
 """The scorers where their launch changes shape: batches just inside and past
 one CTA per SM (38 tiles of 128 rows on 152 SMs) and of several waves with a
 ragged last tile, and K whose slices of 64 do not divide by four (and under
-four of them), against fp64.  Tolerances as derived in the scorers' own tests."""
+four of them), against fp64.  One layer: fp32 sums of K products in four
+chains are off by 2e-7 at the most (K = 3,520); 1e-6 allowed.  Deep: as derived
+in the scorer's own test (bf16 activations)."""
 import pytest
 import torch
 
@@ -24,7 +26,25 @@ def test_mlp(sdd, M, K):
     again = sdd.survival_mlp(h, W1, b1, w2, float(b2), status=status)
     want = torch.sigmoid(_gelu(h.double() @ W1.double().T + b1.double()) @ w2.double() + b2.double())
     assert int(status.item()) == 0 and torch.equal(s, again)
-    torch.testing.assert_close(s.double(), want, rtol=0, atol=5e-5)
+    torch.testing.assert_close(s.double(), want, rtol=0, atol=1e-6)
+
+
+@pytest.mark.parametrize("K", [256, 448, 2048, 3584])
+@pytest.mark.parametrize("M", [64 * 128, 12000, 152 * 128, 20001])
+def test_mlp_error_does_not_grow_with_the_batch(sdd, M, K):
+    """However a batch's tiles are run, a tile's K is summed in chains as short as a small batch's (four).  One CTA a
+    tile (and the tiles left over) add the same sums in the same order as 2,048 rows at a time do; two CTAs a tile add
+    them pairwise, so there the errors against fp64 are compared, which differ by their last rounding (a single chain's
+    is four times as large at K = 3,584, and a tenth larger at K = 256)."""
+    W1, b1, w2, b2 = synth.make_mlp(device="cuda", hidden=K)
+    h = synth.make_hidden(M, device="cuda", seed=3, hidden=K)
+    s = sdd.survival_mlp(h, W1, b1, w2, float(b2))
+    small = torch.cat([sdd.survival_mlp(c, W1, b1, w2, float(b2)) for c in h.split(2048)])
+    if M > 76 * 128:
+        assert torch.equal(s, small)
+    else:
+        want = torch.sigmoid(_gelu(h.double() @ W1.double().T + b1.double()) @ w2.double() + b2.double())
+        assert float((s - want).norm()) <= 1.1 * float((small - want).norm())
 
 
 @pytest.mark.parametrize("M,Kh", [(38 * 128, 256), (38 * 128 + 1, 256), (12345, 192), (20001, 64), (20001, 704)])
@@ -42,6 +62,24 @@ def test_deep(sdd, M, Kh):
     want = torch.sigmoid(u @ w4.double() + b4)
     assert int(status.item()) == 0 and torch.equal(s, again)
     torch.testing.assert_close(s.double(), want, rtol=0, atol=3e-4)
+
+
+@pytest.mark.parametrize("Kh", [64, 704, 3584])
+@pytest.mark.parametrize("M", [64 * 128, 12000, 152 * 128, 20001])
+def test_deep_rows_do_not_depend_on_the_batch(sdd, M, Kh):
+    """One CTA a tile and the split form sum alike: activations of the first layer and scores of a batch are those of
+    its rows 2,048 at a time, except between 38 and 76 tiles, where two splits add the chains pairwise."""
+    w = synth.make_scorer_deep(device="cuda", hidden=Kh)
+    h, f = synth.make_hidden(M, device="cuda", seed=5, hidden=Kh), synth.make_features(M, device="cuda")
+    act = [torch.empty(n, 256, dtype=torch.bfloat16, device="cuda") for n in (M, M)]
+    s = sdd.scorer_deep(h, f, *w, act=act[0])
+    small = torch.cat([sdd.scorer_deep(h[i:i + 2048], f[i:i + 2048], *w, act=act[1][i:i + 2048])
+                       for i in range(0, M, 2048)])
+    if M > 76 * 128:
+        assert torch.equal(act[0], act[1]) and torch.equal(s, small)
+    else:
+        assert float((act[0] != act[1]).float().mean()) < 1e-3
+        torch.testing.assert_close(s, small, rtol=0, atol=1e-4)   # a bf16 step of a few activations
 
 
 @pytest.mark.parametrize("M", [38 * 128 + 1, 152 * 128 + 1, 157 * 128])
