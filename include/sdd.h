@@ -356,7 +356,8 @@ SDD_API sdd_status_t sdd_commit(const int32_t *K, const int32_t *draft_tokens, c
 /*
  * sdd_test_wait_hooks -- failure-detection test hooks (the paper has no
  * counterpart: they test the library's bounded device waits).  They apply to
- * the streaming kernel of every call this process enqueues afterwards, from
+ * the streaming kernel of every call this process enqueues afterwards (the
+ * sharded records' streaming form among them; the pipelined rounds' not), from
  * any thread, until changed:
  *   polls      the number of polls after which a wait for a tile copy gives
  *              up (each poll may suspend the warp briefly); 0 restores the

@@ -199,9 +199,11 @@ struct ScheduleParams {
 
 // The streaming kernel: p.W warps over min(p.W, p.ctas) CTAs.
 cudaError_t launch_scan(const ScanParams &p, cudaStream_t stream);
-// Failure-detection test hooks of the streaming kernel, read at each launch:
-// the ring waits' poll limit (0 = kWaitPolls) and the dropped first copy.
+// Failure-detection test hooks of the streaming kernel and of the sharded
+// records' streaming form, read at each launch: the ring waits' poll limit (0 =
+// kWaitPolls) and the dropped first copy.
 void set_scan_wait_hooks(uint32_t polls, int drop_copy);
+void get_scan_wait_hooks(uint32_t &polls, int32_t &drop_copy);
 // The decide kernel over (listed blocks, p.dec.nseg) CTAs, launched as a
 // programmatic dependent of the streaming kernel.
 cudaError_t launch_decide(const ScanParams &p, cudaStream_t stream);

@@ -55,16 +55,19 @@ void set_scan_wait_hooks(uint32_t polls, int drop_copy) {
     g_wait_polls.store(polls, std::memory_order_relaxed);
     g_drop_copy.store(drop_copy ? 1 : 0, std::memory_order_relaxed);
 }
+void get_scan_wait_hooks(uint32_t &polls, int32_t &drop_copy) {
+    const uint32_t n = g_wait_polls.load(std::memory_order_relaxed);
+    polls = n ? n : kWaitPolls;
+    drop_copy = g_drop_copy.load(std::memory_order_relaxed);
+}
 
 cudaError_t launch_scan(const ScanParams &p, cudaStream_t stream) {
     const bool bf = p.dtype == SDD_BF16, feat = p.feat != nullptr;
     const int kind = feat ? 3 : p.n_groups > 1 ? kRowsMixed : p.grp[0].kind == 0 ? kRowsDrafter : kRowsTarget;
     void (*const k)(ScanParams) = kScanKernels[bf][kind];
     ScanParams q = p;
-    const uint32_t polls = g_wait_polls.load(std::memory_order_relaxed);
-    q.wait_polls = polls ? polls : kWaitPolls;
+    get_scan_wait_hooks(q.wait_polls, q.drop_copy);
     q.spread = (p.W + std::min(p.W, p.ctas) - 1) / std::min(p.W, p.ctas);
-    q.drop_copy = g_drop_copy.load(std::memory_order_relaxed);
     return launch_dependent(k, dim3(std::min(p.W, p.ctas)), dim3(32 * q.spread), ring_bytes(kStages, q.spread), stream,
                             q);
 }

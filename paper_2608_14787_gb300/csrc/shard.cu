@@ -426,6 +426,7 @@ struct StreamParams {
     int32_t rows, nd;        // all rows, drafter rows
     int32_t slots;           // piece slots of a CTA
     uint32_t wait_polls;
+    int32_t drop_copy;       // failure-detection test hook: the first warp never issues its first copy
 };
 
 __device__ __forceinline__ uint32_t slice_cta_rank() {
@@ -660,14 +661,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     const char *prow = slice_row_base(p, ra + pc.l);
     const uint64_t pol = l2_evict_first_policy();
     uint32_t pending = 0, phase = 0;
+    bool drop = p.drop_copy != 0 && cl == 0 && gw == 0;
     auto issue = [&](int slot) {
         const int n = static_cast<int>(min(static_cast<int64_t>(min(kTileVec, RV - pc.k)), v1 - pc.v));
-        if (lane == 0) {
-            mbar_arrive_expect_tx(&bars[slot], static_cast<uint32_t>(n) * 16u);
-            bulk_g2s(ring + slot * kTileBytes, prow + static_cast<int64_t>(pc.k) * 16, static_cast<uint32_t>(n) * 16u,
-                     &bars[slot], pol);
+        if (drop) {   // (test hook: nothing completes this slot's barrier, and nothing is in flight for the drain)
+            drop = false;
+        } else {
+            if (lane == 0) {
+                mbar_arrive_expect_tx(&bars[slot], static_cast<uint32_t>(n) * 16u);
+                bulk_g2s(ring + slot * kTileBytes, prow + static_cast<int64_t>(pc.k) * 16,
+                         static_cast<uint32_t>(n) * 16u, &bars[slot], pol);
+            }
+            pending |= 1u << slot;
         }
-        pending |= 1u << slot;
         pc.v += n;
         pc.k += n;
         if (pc.k == RV && pc.v < v1) {
@@ -772,6 +778,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             }
         }
     }
+    // (a warp that gave up leaves its pieces' slots as they were, so the rows'
+    // records are undefined; it meets the cluster's barrier below all the same)
     if (timed_out) {
         if (lane == 0) status_or(sp.status, SDD_DEV_TIMEOUT);
         for (int s = 0; s < kStages; ++s)
@@ -922,7 +930,7 @@ cudaError_t launch_shard_partials(const ShardParams &sp, cudaStream_t stream) {
         p.sp = sp;
         p.rows = static_cast<int32_t>(rows);
         p.nd = sp.B * sp.gamma;
-        p.wait_polls = kWaitPolls;
+        get_scan_wait_hooks(p.wait_polls, p.drop_copy);
         return launch_dependent(kStream[bf][cand], dim3(2 * clusters), dim3(kThreads), stream_smem(p.slots), stream, p);
     }
     void (*const k)(ShardParams) = bf ? (cand ? shard_partials_kernel<SDD_BF16, true> : shard_partials_kernel<SDD_BF16, false>)

@@ -1,5 +1,5 @@
 """Failure detection of the bounded device waits: the streaming kernel's wait
-for a tile copy is made to run out (the test hook keeps the first warp's first
+(and that of the sharded records' streaming form) for a tile copy is made to run out (the test hook keeps the first warp's first
 copy from ever being issued, so nothing completes its barrier), with a short
 poll limit.  The call must return, report SDD_DEV_TIMEOUT in its device status
 word without trapping, and leave the context, the workspace and the next calls
@@ -52,6 +52,35 @@ def test_ring_wait_runs_out_and_recovers(sdd, orc, polls):
     rnd.run()
     torch.cuda.synchronize()
     assert int(rnd.status.item()) == 0
+
+
+@pytest.mark.parametrize("k", [0, 10])
+@pytest.mark.parametrize("polls", [64, 4096])
+def test_sharded_records_wait_runs_out_and_recover(sdd, polls, k):
+    """One warp of the sharded records' streaming form gives up; both CTAs of its cluster still meet at their barrier,
+    the call returns with its status, and the next one writes the records that it wrote before."""
+    from paper_2608_14787_gb300 import vocab_shard
+    blk = synth.make_block("c3", device="cuda", B=5, gamma=7, V=20_000)
+    r = vocab_shard.ShardRound(5, 7, 20_000, 0, 20_000, ks=(k,) if k else ())
+    r.set_inputs(blk.z_d, blk.z_t, blk.x)
+    want = r.partials().clone()
+    torch.cuda.synchronize()
+    assert int(r.status.item()) == 0
+    try:
+        sdd.test_wait_hooks(polls, drop_copy=True)
+        t0 = time.perf_counter()
+        r.partials()
+        torch.cuda.synchronize()
+        dt = time.perf_counter() - t0
+    finally:
+        sdd.test_wait_hooks(0, drop_copy=False)
+    assert dt < 30.0
+    code, bits = sdd.status_from_device(r.status, clear=True)
+    assert code == sdd.binding.SDD_ERR_DEVICE and bits == sdd.DEV_TIMEOUT
+    r.partials().zero_()
+    got = r.partials()
+    torch.cuda.synchronize()
+    assert int(r.status.item()) == 0 and torch.equal(got.view(torch.uint8), want.view(torch.uint8))
 
 
 def test_short_limit_without_a_dropped_copy_is_harmless(sdd, orc):
