@@ -163,13 +163,6 @@ __device__ __forceinline__ void fence_proxy_async_global() {
     asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-// Untiled global -> shared bulk copy (16-byte aligned, size a multiple of 16).
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float a) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
 }
@@ -308,7 +301,8 @@ __device__ __forceinline__ bool mlp_drain(uint64_t *done, uint64_t *drained, int
 // from tmA, the rest from tmA2 (the scalar features of the deep scorer).
 // HEAD: the epilogue fuses GELU, the w2 dot product and the sigmoid (one
 // float per row); otherwise it writes the layer's activations GELU(z + b1)
-// as bf16 rows of p.act for the next layer.
+// as bf16 rows of p.act for the next layer (S > 1: whole tiles of the deep
+// scorer are mlp_deep_kernel's).
 // The CTA's K is taken in 4 / S chains (as its slices allow): S = 2 adds its two
 // where it reads them, S = 1 its four beside the main loop (mlp_drain).
 __host__ __device__ constexpr int mlp_threads(int S) { return S == 1 ? kMlpThreadsChains : kMlpThreads; }
@@ -942,8 +936,8 @@ cudaError_t mlp_prepare(int *sm_count) {
         *sm_count = g_sms[dev].load(std::memory_order_relaxed);
         return cudaSuccess;
     }
-    for (auto fn : {mlp_kernel<1, true>, mlp_kernel<2, true>, mlp_kernel<4, true>, mlp_kernel<1, false>,
-                    mlp_kernel<2, false>, mlp_kernel<4, false>}) {
+    for (auto fn : {mlp_kernel<1, true>, mlp_kernel<2, true>, mlp_kernel<4, true>, mlp_kernel<2, false>,
+                    mlp_kernel<4, false>}) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
         if (e != cudaSuccess) return e;
     }
@@ -1023,9 +1017,10 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
         attr[1].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 2;
+        // (a plan's rest has S = 4 or 2)
         const auto kernel = S == 4   ? (head ? mlp_kernel<4, true> : mlp_kernel<4, false>)
                             : S == 2 ? (head ? mlp_kernel<2, true> : mlp_kernel<2, false>)
-                                     : (head ? mlp_kernel<1, true> : mlp_kernel<1, false>);
+                                     : mlp_kernel<1, true>;
         return cudaLaunchKernelEx(&cfg, kernel, tmA, tmA2, tmB, p);
     };
     const MlpPlan plan = mlp_plan(M, K, sms);
