@@ -1174,10 +1174,7 @@ static sdd_status_t pipe_params(const sdd_block_args *a, ScanParams &p, bool *em
     set_divisors(p, kPipeCostDrafter, kPipeCostTarget);
     p.warp0 = team_warps;
     p.wpc = wpc;
-    if (wpc == kShareWarps && p.W == p.ctas * wpc && p.whole == 0) {
-        p.units = p.ctas * kShareCta;   // (C units < 2^53: a round here is at most kPipeMidBytes)
-        p.divW = make_fastdiv(static_cast<uint64_t>(p.units));
-    }
+    if (wpc == kShareWarps && p.W == p.ctas * wpc && p.whole == 0) set_shares(p);
     return SDD_OK;
 }
 

@@ -146,7 +146,7 @@ struct ScanParams {
     int32_t W;               // active warps
     int32_t units;           // the pipelined pass's weighted warps: the total of their shares (0: equal shares)
     int32_t whole;           // every row is cut into this many pieces (0: cut by cost, or a device block count)
-    int32_t pieces;          // pieces of a row at most (warps that stream parts of it)
+    int32_t pieces;          // about the most pieces of a row (an estimate: the decide team's groups follow from it)
     int32_t ctas;            // CTAs of a full streaming grid (one per SM)
     int64_t rows0;           // rows of group 0
     int64_t rows;            // rows of all groups
@@ -380,6 +380,44 @@ inline void set_divisors(ScanParams &p, int32_t cost_drafter = kCostDrafter, int
     p.wpc = kWarpsPerCta;
 }
 
+// Unequal shares for the p.ctas * kShareWarps warps of a full pipelined pass,
+// after set_divisors (C * units < 2^53: such a round is at most kPipeMidBytes).
+inline void set_shares(ScanParams &p) {
+    p.units = p.ctas * kShareCta;
+    p.divW = make_fastdiv(static_cast<uint64_t>(p.units));
+}
+
+// The sharded records' streaming form (shard.cu): the cut of a slice's rows, nd
+// drafter rows first, over G clusters of kSliceWarps warps in two CTAs.
+constexpr int kSliceWarps = 2 * kWarpsPerCta;
+constexpr int kCostSliceDrafter = 10, kCostSliceTarget = 9;
+// The first row of cluster c: the first whose preceding rows cost at least c / G
+// of the whole.
+__host__ __device__ inline int slice_row(int nd, int rows, int c, int G) {
+    const int64_t cd = static_cast<int64_t>(nd) * kCostSliceDrafter;
+    const int64_t ct = cd + static_cast<int64_t>(rows - nd) * kCostSliceTarget;
+    const int64_t x = ct * c / G;
+    if (x <= cd) return static_cast<int>((x + kCostSliceDrafter - 1) / kCostSliceDrafter);
+    return nd + static_cast<int>((x - cd + kCostSliceTarget - 1) / kCostSliceTarget);
+}
+// Of a cluster's Tc vectors: warp w's first, and the warp that holds vector v.
+__host__ __device__ inline int64_t slice_start(int64_t Tc, int w) { return Tc * w / kSliceWarps; }
+__host__ __device__ inline int slice_owner(int64_t Tc, int64_t v) {
+    return static_cast<int>(((v + 1) * kSliceWarps - 1) / Tc);
+}
+// The rows that CTA 0 merges: those that start before the cluster's middle.
+__host__ __device__ inline int slice_half(int64_t Tc, int RV) {
+    return static_cast<int>((slice_start(Tc, kWarpsPerCta) + RV - 1) / RV);
+}
+// The slot, in the CTA that merges row l (of the cluster), of warp w's piece of it.
+__host__ __device__ inline int slice_slot(int l, int n0, int w) { return l >= n0 ? l - n0 + w - kWarpsPerCta : l + w; }
+// Slots of a CTA for `rows` rows in all: a cluster's rows by cost are at most one
+// ninth more than its even part, and a row for the rounding.
+__host__ __device__ inline int slice_slots(int64_t rows, int clusters) {
+    const int64_t most = (rows + clusters - 1) / clusters;
+    return static_cast<int>((most * 10 / 9 + 2) / 2 + 2 + kSliceWarps);
+}
+
 // Offline diagnostics (diag.cu).  pi: [n_rep, gamma, B] 16-bit scratch;
 // sums: [n_rep + 1] feasible-prefix sums (the last: the logged order).
 cudaError_t launch_perm_diag(const float *q, const int32_t *L, int B, int gamma, int signal, df eta_loc,
@@ -410,9 +448,14 @@ cudaError_t decide_prepare_device();
 cudaError_t pipe_prepare_device();
 void set_last_error(const char *msg);  // message returned by sdd_last_error()
 
-__device__ __forceinline__ int64_t fast_div(int64_t n, const FastDiv &f) {
+__host__ __device__ __forceinline__ int64_t fast_div(int64_t n, const FastDiv &f) {
     const uint64_t u = static_cast<uint64_t>(n);
-    return static_cast<int64_t>(f.pow2 ? (u >> f.s) : (__umul64hi(u, f.M) >> f.s));
+#ifdef __CUDA_ARCH__
+    const uint64_t hi = __umul64hi(u, f.M);
+#else
+    const uint64_t hi = static_cast<uint64_t>((static_cast<unsigned __int128>(u) * f.M) >> 64);
+#endif
+    return static_cast<int64_t>((f.pow2 ? u : hi) >> f.s);
 }
 
 // The launch's partition: from the parameters, or -- with a device block
@@ -423,7 +466,7 @@ struct PartView {
     int64_t nb, rows0, rows, T, T0, C;
     int32_t W;
 };
-__device__ __forceinline__ int64_t div_part(int64_t n, int64_t d, const FastDiv &f, const ScanParams &p) {
+__host__ __device__ __forceinline__ int64_t div_part(int64_t n, int64_t d, const FastDiv &f, const ScanParams &p) {
     if (p.nb_dev) return static_cast<int64_t>(static_cast<uint64_t>(n) / static_cast<uint64_t>(d));
     return fast_div(n, f);
 }
@@ -461,7 +504,7 @@ __device__ __forceinline__ PartView part_view(const ScanParams &p) {
 // Also the row r (of both groups) that holds start(w) and its vector k there.
 // SHARES: the launch's warps may have shares (p.units; W is then the units').
 template <bool SHARES>
-__device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartView &v, int64_t w, int64_t &row,
+__host__ __device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartView &v, int64_t w, int64_t &row,
                                               int32_t &kv) {
     const int64_t c = div_part((SHARES && p.units ? share_start(w) : w) * v.C, v.W, p.divW, p);
     const int64_t c0 = v.rows0 * p.P[0];   // the cost of group 0
@@ -477,7 +520,7 @@ __device__ __forceinline__ int64_t part_start(const ScanParams &p, const PartVie
     return (g ? v.T0 : 0) + r * p.RV + k;
 }
 // The warp owning vector v.
-__device__ __forceinline__ int64_t part_owner(const ScanParams &p, const PartView &pv, int64_t v) {
+__host__ __device__ __forceinline__ int64_t part_owner(const ScanParams &p, const PartView &pv, int64_t v) {
     const int g = (v < pv.T0) ? 0 : 1;
     const int64_t u = g ? v - pv.T0 : v;
     const int64_t r = fast_div(u, p.divRV);

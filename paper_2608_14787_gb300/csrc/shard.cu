@@ -416,7 +416,6 @@ __global__ void __launch_bounds__(kShardThreads, kShardMinCtas) shard_partials_k
 constexpr int kCandList = 7;      // tile maxima a lane keeps
 constexpr int kCandGroups = 32;   // groups a piece re-reads at most
 constexpr int kCandKeys = 64;     // entries it ranks at most
-constexpr int kCostSliceDrafter = 10, kCostSliceTarget = 9;
 
 // A piece's slot: its partial, then its candidate keys, descending (0: none).
 constexpr int kSlotBytes = static_cast<int>(sizeof(Partial)) + SDD_SHARD_KMAX * 8;
@@ -446,16 +445,6 @@ __device__ __forceinline__ void st_slice_v4(uint32_t addr, uint4 v) {
 }
 __device__ __forceinline__ void st_slice_u64(uint32_t addr, uint64_t v) {
     asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
-}
-
-// The first row of cluster c of G: the first whose preceding rows cost at
-// least c / G of the whole.
-__device__ __forceinline__ int slice_row(const StreamParams &p, int c, int G) {
-    const int64_t cd = static_cast<int64_t>(p.nd) * kCostSliceDrafter;
-    const int64_t ct = cd + static_cast<int64_t>(p.rows - p.nd) * kCostSliceTarget;
-    const int64_t x = ct * c / G;
-    if (x <= cd) return static_cast<int>((x + kCostSliceDrafter - 1) / kCostSliceDrafter);
-    return p.nd + static_cast<int>((x - cd + kCostSliceTarget - 1) / kCostSliceTarget);
 }
 
 __device__ __forceinline__ const char *slice_row_base(const StreamParams &p, int r) {
@@ -622,7 +611,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     shard_stream_kernel(const __grid_constant__ StreamParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int EPV = (DT == SDD_BF16) ? 8 : 4;
-    constexpr int CW = 2 * kWarpsPerCta;   // the cluster's warps
     const ShardParams &sp = p.sp;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int rank = static_cast<int>(slice_cta_rank());
@@ -642,14 +630,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
     // the cluster's rows [ra, rb), this warp's vectors [v0, v1) of them
     const int cl = static_cast<int>(blockIdx.x) >> 1, G = static_cast<int>(gridDim.x) >> 1;
-    const int bnd = slice_row(p, cl + (lane & 1), G);
+    const int bnd = slice_row(p.nd, p.rows, cl + (lane & 1), G);
     const int ra = __shfl_sync(0xFFFFFFFFu, bnd, 0), rb = __shfl_sync(0xFFFFFFFFu, bnd, 1);
     const int RV = sp.RVs, tail = sp.Vs % EPV;
     const int64_t Tc = static_cast<int64_t>(rb - ra) * RV;
     const int gw = rank * kWarpsPerCta + warp;
-    const int64_t v0 = Tc * gw / CW, v1 = Tc * (gw + 1) / CW;
-    // CTA 0 owns the rows that start before the cluster's middle: the first n0
-    const int n0 = static_cast<int>((Tc * kWarpsPerCta / CW + RV - 1) / RV);
+    const int64_t v0 = slice_start(Tc, gw), v1 = slice_start(Tc, gw + 1);
+    const int n0 = slice_half(Tc, RV);   // CTA 0 owns the first n0 rows
 
     struct Cur {
         int64_t v;
@@ -754,8 +741,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             uint64_t key = 0ull;
             if (CAND && !ent) key = group_candidates<DT>(crow, kb, cc.k, sp.Vs, sp.v0, sp.kcap, ck, ct, s_key);
             const int own = cc.l >= n0 ? 1 : 0;
-            const int at = own ? (cc.l - n0) + (gw - kWarpsPerCta) : cc.l + gw;
-            const uint32_t dst = slice_map(smem_addr(slots + at * kSlotBytes), static_cast<uint32_t>(own));
+            const uint32_t dst = slice_map(smem_addr(slots + slice_slot(cc.l, n0, gw) * kSlotBytes), static_cast<uint32_t>(own));
             if (lane < 2) {
                 Partial pt;
                 pt.m = M;
@@ -814,11 +800,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (l > l0 + warp) token(l);
         // the warps that hold its first and last vector
         const int64_t f = static_cast<int64_t>(l) * RV;
-        const int fw = static_cast<int>(((f + 1) * CW - 1) / Tc), lw = static_cast<int>(((f + RV) * CW - 1) / Tc);
-        const int at = (rank ? (l - n0) - kWarpsPerCta : l) + fw + lane;
+        const int fw = slice_owner(Tc, f), lw = slice_owner(Tc, f + RV - 1);
         const bool on = fw + lane <= lw;
         SoftState a = soft_identity();
-        const unsigned char *piece = slots + at * kSlotBytes;
+        const unsigned char *piece = slots + slice_slot(l, n0, fw + lane) * kSlotBytes;
         if (on) {
             const Partial pt = *reinterpret_cast<const Partial *>(piece);
             a.m = pt.m;
@@ -908,10 +893,8 @@ cudaError_t stream_device(StreamDev &out) {
 int stream_plan(const ShardParams &sp, int64_t rows, const StreamDev &dev, int32_t &slots) {
     slots = 0;
     if (dev.clusters < 1 || rows >= (int64_t(1) << 27)) return 0;
-    const int64_t most = (rows + dev.clusters - 1) / dev.clusters;   // rows of a cluster
     if (sp.RVs < 2 * kTileVec) return 0;
-    // a cluster's rows by cost: at most one ninth more, and a row for the rounding
-    slots = static_cast<int32_t>((most * 10 / 9 + 2) / 2 + 2 + 2 * kWarpsPerCta);
+    slots = slice_slots(rows, dev.clusters);
     return stream_smem(slots) <= static_cast<size_t>(dev.smem) ? dev.clusters : 0;
 }
 
