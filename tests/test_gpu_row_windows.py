@@ -1,7 +1,7 @@
 """Streaming warps whose ranges touch more than 32 rows (their rows' facts are
 held one row per lane and reloaded): short rows in large batches, the ranges
 starting and ending inside rows, tokens out of range and masked rows among
-them, against the oracle."""
+them, against the oracle (the tolerance as in the extended features' tests)."""
 import numpy as np
 import pytest
 import torch
@@ -27,7 +27,7 @@ def test_many_rows_per_warp(sdd, orc, B, gamma, V):
     st = orc.row_stats(synth.bf16_bits(z_d), tokens=x.cpu().numpy())
     ok = np.ones((B, gamma), bool)
     ok[3, 1] = ok[5, 2] = ok[6, 0] = False
-    np.testing.assert_allclose(rnd.q.cpu().numpy()[ok], st.q[ok], rtol=2e-3, atol=1e-7)
+    np.testing.assert_allclose(rnd.q.cpu().numpy()[ok], st.q[ok], rtol=4e-6)
     assert np.isnan(rnd.q.cpu().numpy()[~ok]).all()
     np.testing.assert_array_equal(rnd.argmax.cpu().numpy()[ok], st.argmax[ok])
     zt, xs = synth.bf16_bits(z_t), x.cpu().numpy()

@@ -2,7 +2,9 @@
 streaming form can go wrong: rows that do and do not divide over the clusters,
 rows crossing a cluster's middle, ragged slices, and the candidate lists under
 ties (few levels, constant rows), masked rows, candidates bunched in one lane
-or at the slice's ends, up to the largest k; both types, odd slice starts."""
+or at the slice's ends, up to the largest k; both types, even and odd slice
+starts; rows with NaN and infinities through the whole round, and the most rows
+that its shared memory holds."""
 import numpy as np
 import pytest
 import torch
@@ -45,7 +47,7 @@ def test_records(B, gamma, w, k, kind, dtype):
         B = max(1, 76 // (2 * gamma + 1))
     gen = torch.Generator(device="cuda")
     gen.manual_seed(B * 1000 + w + k)
-    v0, V = 24, w + 100
+    v0, V = 24 if kind in ("plain", "levels") else 23, w + 100
     zd, zt = _logits(kind, B, gamma, w, dtype, gen), _logits(kind, B, gamma + 1, w, dtype, gen)
     x = torch.randint(0, V, (B, gamma), generator=gen, device="cuda", dtype=torch.int32)
     x[0, 0] = V
@@ -81,3 +83,80 @@ def test_records(B, gamma, w, k, kind, dtype):
         order = np.argsort(-z[nd:], axis=1, kind="stable")[:, :k]
         np.testing.assert_array_equal(rec["cv"][nd:, :k], v0 + order)
         np.testing.assert_array_equal(rec["cz"][nd:, :k], np.take_along_axis(z[nd:], order, 1).astype(np.float32))
+
+
+@pytest.mark.parametrize("V", [30011, 3000])   # two slices of the streaming form; of one CTA per row
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_nonfinite_rows(V, dtype):
+    """NaN and +inf rows, drafter and target, in either slice: flagged and NaN as in the round over whole rows, every
+    decision as there, and the other rows' results those of the clean round bit for bit."""
+    B, gamma = 6, 9
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(V)
+    pad = -(-V // 8) * 8
+    zd, zt = (torch.zeros(B, n, pad, dtype=dtype, device="cuda")[..., :V] for n in (gamma, gamma + 1))
+    for z in (zd, zt):
+        z.copy_(torch.randn(*z.shape, generator=gen, device="cuda") * 2)
+    x = zt[:, :gamma].argmax(-1).to(torch.int32)
+    kw = dict(dtype=dtype, ells=(0.5,), ks=(2, 10), greedy=True, K_min=0)
+    cuts = vocab_shard.slice_bounds(V, 2)
+
+    def both():
+        full = sdd.BlockRound(B, gamma, V, **kw)
+        full.set_inputs(zd, zt, x)
+        full.run()
+        ranks = [vocab_shard.ShardRound(B, gamma, V, *c, **kw) for c in cuts]
+        vocab_shard.run_local(ranks, [vocab_shard.slice_logits(zd, *c) for c in cuts],
+                              [vocab_shard.slice_logits(zt, *c) for c in cuts], x)
+        return full, ranks[0].rnd
+
+    _, clean = both()
+    assert int(clean.status.item()) == 0
+    nan, inf = float("nan"), float("inf")
+    zd[0, 1, 5], zd[1, 0, V - 1], zd[2, 3, 700], zd[2, 3, V - 2] = nan, nan, inf, -inf
+    zt[0, 2, V - 3], zt[1, 4, 0], zt[3, gamma, 17], zt[4, 0, V // 2 + 9] = nan, inf, inf, nan
+    full, r = both()
+    assert int(r.status.item()) == int(full.status.item()) == sdd.DEV_NONFINITE
+    bad = torch.zeros(B, gamma, dtype=torch.bool, device="cuda")
+    for b, j in ((0, 1), (1, 0), (2, 3)):
+        bad[b, j] = True
+    for n in ("q", "logq", "maxprob", "entropy", "lse"):
+        got, ref = getattr(r, n), getattr(clean, n)
+        assert bool(got[bad].isnan().all()) and torch.equal(got[~bad], ref[~bad]), n
+    for n in ("L_strict", "tokens_strict", "L_lenient", "tokens_lenient", "L_topk", "tokens_topk", "K", "commit_n",
+              "commit_tokens"):
+        assert torch.equal(getattr(r, n), getattr(full, n)), n
+    for n in ("L_strict", "tokens_strict", "L_topk", "tokens_topk"):   # the untouched block
+        a, c = getattr(r, n), getattr(clean, n)
+        assert torch.equal(a[..., 5, :] if "tokens" in n else a[..., 5], c[..., 5, :] if "tokens" in n else c[..., 5]), n
+
+
+@pytest.mark.parametrize("side", [0, 1])
+def test_most_rows(side):
+    """The last batch whose pieces' slots fit the shared memory, and the first that goes to one CTA per row."""
+    prop = torch.cuda.get_device_properties(0)
+    clusters, optin = prop.multi_processor_count // 2, 227 * 1024
+    slots = (optin - 16 * 2 * 4104 - 16 * 64 * 8) // 160          # rings; candidate keys; a partial and 16 keys
+    most = next(m for m in range(2000, 0, -1) if (m * 10 // 9 + 2) // 2 + 34 <= slots)
+    gamma, w, k = 2, 4096, 3
+    B = clusters * most // (2 * gamma + 1) + side
+    assert (B * (2 * gamma + 1) > clusters * most) == bool(side)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(side)
+    zd, zt = (torch.randn(B, n, w, generator=gen, device="cuda").to(torch.bfloat16) for n in (gamma, gamma + 1))
+    x = torch.randint(0, w, (B, gamma), generator=gen, device="cuda", dtype=torch.int32)
+    r = vocab_shard.ShardRound(B, gamma, w, 0, w, ks=(k,))
+    r.set_inputs(zd, zt, x)
+    rec = np.frombuffer(r.partials().cpu().numpy().tobytes(), REC)
+    assert int(r.status.item()) == 0
+    z = torch.cat([zd.reshape(-1, w), zt.reshape(-1, w)])
+    m = z.float().amax(1)
+    np.testing.assert_array_equal(rec["m"], m.cpu().numpy())
+    first = torch.where(z == m[:, None].to(z.dtype), torch.arange(w, device="cuda", dtype=torch.int32), w).amin(1)
+    np.testing.assert_array_equal(rec["amax"], first.cpu().numpy())
+    lse = torch.cat([torch.logsumexp(c.double(), 1) for c in z.split(8192)]).cpu().numpy()
+    got = np.log(rec["sh"].astype(np.float64) + rec["sl"]) + rec["r"].astype(np.float64) * np.log(2)
+    np.testing.assert_allclose(got, lse, rtol=0, atol=1e-6)       # ex2: 2^-22 of the sum
+    np.testing.assert_array_equal(rec["g"][:B * gamma], zd.float().gather(2, x.long()[..., None]).reshape(-1).cpu().numpy())
+    nd = B * gamma
+    np.testing.assert_array_equal(rec["cz"][nd:, :k], zt.float().topk(k, -1).values.reshape(-1, k).cpu().numpy())
