@@ -190,3 +190,15 @@ def test_pipelined_arguments_rejected_on_host(lib):
     # two rounds in flight cannot share one workspace
     assert lib.sdd_block_pipelined(ctypes.byref(a), ctypes.byref(b), None) == 1
     assert b"workspace" in lib.sdd_last_error()
+
+
+def test_current_stream_without_the_private_entry(monkeypatch):
+    """A torch without the raw-handle entry: the binding asks the public one."""
+    from types import SimpleNamespace
+
+    import torch
+
+    from paper_2608_14787_gb300 import binding
+    monkeypatch.setattr(binding, "_raw_stream", None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: SimpleNamespace(cuda_stream=7))
+    assert binding._stream() == 7 and binding._stream(SimpleNamespace(cuda_stream=9)) == 9
