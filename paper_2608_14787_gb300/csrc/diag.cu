@@ -23,6 +23,8 @@
 //                       integer sums per repetition (exact, order-free).
 // metrics_kernel     -- one cluster of CTAs per position: fp64 BCE sums, integer
 //                       pair counts.
+#include <atomic>
+
 #include "rules.cuh"
 
 namespace sdd {
@@ -504,6 +506,28 @@ __global__ void __cluster_dims__(kMetCluster, 1, 1) __launch_bounds__(kMetThread
     }
 }
 
+constexpr int kMaxDevices = 64;
+std::atomic<int> g_perm_ready[kMaxDevices];
+
+// Per-device opt-in of the builder to all the dynamic shared memory that its
+// static part leaves, once: the limit of 48 KiB without it is on the two
+// together, and a limit set for one call's log would be another thread's too.
+cudaError_t perm_prepare() {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (g_perm_ready[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    cudaFuncAttributes attr;
+    e = cudaFuncGetAttributes(&attr, perm_build_kernel);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(perm_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 optin - static_cast<int>(attr.sharedSizeBytes));
+    if (e == cudaSuccess) g_perm_ready[dev].store(1, std::memory_order_release);
+    return e;
+}
+
 }  // namespace
 
 cudaError_t launch_perm_diag(const float *q, const int32_t *L, int B, int gamma, int signal, df eta_loc,
@@ -512,12 +536,9 @@ cudaError_t launch_perm_diag(const float *q, const int32_t *L, int B, int gamma,
     cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * (n_rep + 1), stream);
     if (e != cudaSuccess) return e;
     const size_t smem = perm_smem_bytes(B);
-    if (smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(perm_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-    }
     if (n_rep > 0) {
+        e = perm_prepare();
+        if (e != cudaSuccess) return e;
         e = launch_dependent(perm_build_kernel, dim3(n_rep * gamma), dim3(kPermThreads), smem, stream, L, B, gamma,
                              signal == SDD_SIG_CONDITIONAL ? 1 : 0, seed, pi);
         if (e != cudaSuccess) return e;

@@ -1,5 +1,6 @@
 """The diagnostics at the edges of their kernels' tiles: logs around a warp, the
-builder's and the prefix kernel's CTA, the parallel shuffle's limit, and the
+builder's and the prefix kernel's CTA, the parallel shuffle's limit, the largest
+log and those whose builder needs about 48 KiB of shared memory, and the
 metrics' tiles of sorted positives (1,024 of a cluster CTA's eighth of the
 log), against the oracle."""
 import numpy as np
@@ -17,7 +18,8 @@ def _log(B, gamma, seed):
     return q, L
 
 
-@pytest.mark.parametrize("B", [1, 2, 31, 32, 33, 255, 256, 257, 1025, 4095, 4096, 4097])
+@pytest.mark.parametrize("B", [1, 2, 31, 32, 33, 255, 256, 257, 1025, 3376, 3377, 3413, 3449, 3450, 4095, 4096, 4097,
+                               11323, 11324, 11450, 11564, 11565, 50000])
 @pytest.mark.parametrize("signal", [0, 2])
 def test_permutation_sizes(sdd, orc, B, signal):
     q, L = _log(B, 7, B)
