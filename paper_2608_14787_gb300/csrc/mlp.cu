@@ -8,7 +8,7 @@
 //
 // and the scalar-feature block f of the deep scorer's input.
 //
-// Up to a quarter of the SMs' worth of 128-row tiles (a decode round's batch):
+// As many 128-row tiles as clusters of four fit the SMs (a decode round's batch):
 // first layer (mlp_kernel): a cluster of S = 4 CTAs per 128-row tile splits K;
 // each CTA streams its K quarter through a four-stage ring of 48 KiB (A tile
 // 128 x 64, B tile 256 x 64, K-major, 128-byte swizzle) filled by 2D TMA, one
@@ -507,8 +507,8 @@ constexpr int kTailSlices = kMlpN / kMlpBK;                // 4
 constexpr uint32_t kTailA = kTailSlices * kTailASlice;     // 64 KiB
 constexpr uint32_t kTailW = kTailSlices * kTailWSlice;     // 32 KiB
 // PAIR: W3 takes W2's place, so that two CTAs share an SM (launches of more
-// CTAs than SMs: one's round trips run under the other's epilogue); otherwise
-// both are loaded ahead.
+// clusters than fit at one CTA per SM: one's round trips run under the other's
+// epilogue); otherwise both are loaded ahead.
 constexpr int tail_smem(bool pair) { return static_cast<int>(kTailA + (pair ? 1 : 2) * kTailW) + 1024 + 256; }
 constexpr uint32_t kTailTmemCols = 128;
 constexpr int kTailThreads = 512;   // 16 warps: four per TMEM lane quarter, 16 columns each
@@ -924,16 +924,37 @@ struct MapCache {
 MapCache g_maps;
 constexpr int kMaxDevices = 64;
 std::atomic<int> g_attr_ready[kMaxDevices];
-std::atomic<int> g_sms[kMaxDevices];
+// What fits a device at once: CTAs of the first layer's kernels one per SM, and
+// clusters of 4 and of 2 of them (a GPC's SMs are not a multiple of four: 36
+// clusters of 4 on 152 SMs, 76 of 2).
+struct MlpDev {
+    int sms, c4, c2;
+};
+MlpDev g_dev[kMaxDevices];
+
+cudaError_t max_clusters(int *n, void (*kernel)(CUtensorMap, CUtensorMap, CUtensorMap, MlpParams), int S) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(S);
+    cfg.blockDim = dim3(mlp_threads(S));
+    cfg.dynamicSmemBytes = kMlpSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = S;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(n, kernel, &cfg);
+}
 
 // Per-device opt-in of every kernel here to its dynamic shared memory.
-cudaError_t mlp_prepare(int *sm_count) {
+cudaError_t mlp_prepare(MlpDev *out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
     if (g_attr_ready[dev].load(std::memory_order_acquire)) {
-        *sm_count = g_sms[dev].load(std::memory_order_relaxed);
+        *out = g_dev[dev];
         return cudaSuccess;
     }
     for (auto fn : {mlp_kernel<1, true>, mlp_kernel<2, true>, mlp_kernel<4, true>, mlp_kernel<2, false>,
@@ -941,35 +962,43 @@ cudaError_t mlp_prepare(int *sm_count) {
         e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
         if (e != cudaSuccess) return e;
     }
-    int sms = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    MlpDev d = {};
+    e = cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = max_clusters(&d.c4, mlp_kernel<4, true>, 4);
+    if (e == cudaSuccess) e = max_clusters(&d.c2, mlp_kernel<2, true>, 2);
     if (e != cudaSuccess) return e;
-    g_sms[dev].store(sms, std::memory_order_relaxed);
     e = cudaFuncSetAttribute(mlp_tail_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem(false));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(mlp_tail_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, tail_smem(true));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(mlp_deep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmem);
     if (e != cudaSuccess) return e;
-    g_attr_ready[dev].store(1, std::memory_order_release);
-    *sm_count = sms;
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!g_attr_ready[dev].load(std::memory_order_acquire)) {
+        g_dev[dev] = d;
+        g_attr_ready[dev].store(1, std::memory_order_release);
+    }
+    *out = d;
     return cudaSuccess;
 }
 
 // How M rows' tiles are run: `full` of them, whole waves of one tile per SM,
 // with K not split (no operand read twice, nothing exchanged), and the `rest`
-// after them with K split S ways, as far as the SMs reach (one wave again; a
-// wave with S = 4, 2, 1 takes 13.7, 20.3 and 35.4 us at K = 3584).  A rest of
-// more than half the SMs runs unsplit too (it is then part of `full`).  GB300,
+// after them with K split S ways, as far as their clusters all fit at once (one
+// wave again: 13.9 us with S = 4 at 32 tiles of K = 3584, 14.6 at 36, and 25.4 at
+// 37, whose last cluster waits for another; 18.2 with S = 2 there, 22.4 at 76; a
+// full wave with S = 1 35.4).  A larger rest runs unsplit too (it is then part of
+// `full`).  GB300,
 // one-layer scorer, K = 3584, three inputs in turn, against all tiles split four
 // ways: 8,192 rows 20.3 / 28.9 us, 12,000 28.2 / 43.7, 16,384 33.3 / 58.0,
 // 20,000 44.9 / 71.9, 32,768 64.4 / 111.9.
 struct MlpPlan {
     int full, rest, S;
 };
-MlpPlan mlp_plan(int M, int K, int sms) {
+MlpPlan mlp_plan(int M, int K, const MlpDev &dev) {
     const int tiles = (M + kMlpBM - 1) / kMlpBM, nk = K / kMlpBK;
-    MlpPlan q{tiles / sms * sms, tiles % sms, 1};
-    if (q.rest > 0) q.S = (4 * q.rest <= sms && nk >= 4) ? 4 : (2 * q.rest <= sms && nk >= 2) ? 2 : 1;
+    MlpPlan q{tiles / dev.sms * dev.sms, tiles % dev.sms, 1};
+    if (q.rest > 0) q.S = (q.rest <= dev.c4 && nk >= 4) ? 4 : (q.rest <= dev.c2 && nk >= 2) ? 2 : 1;
     if (q.S == 1) q = MlpPlan{tiles, 0, 1};
     return q;
 }
@@ -986,8 +1015,8 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
         *why = "cuTensorMapEncodeTiled failed";
         return cudaErrorInvalidValue;
     }
-    int sms = 0;
-    cudaError_t e = mlp_prepare(&sms);
+    MlpDev dev;
+    cudaError_t e = mlp_prepare(&dev);
     if (e != cudaSuccess) return e;
     MlpParams p;
     p.M = M;
@@ -1023,7 +1052,7 @@ cudaError_t launch_layer1(const void *a1, int Ka, const void *a2, int M, int K, 
                                      : mlp_kernel<1, true>;
         return cudaLaunchKernelEx(&cfg, kernel, tmA, tmA2, tmB, p);
     };
-    const MlpPlan plan = mlp_plan(M, K, sms);
+    const MlpPlan plan = mlp_plan(M, K, dev);
     if (head && plan.full > 0) {
         e = launch(0, plan.full, 1);
         if (e != cudaSuccess) return e;
@@ -1052,11 +1081,11 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
                                const char **why) {
     *why = nullptr;
     if (M == 0) return cudaSuccess;
-    int sms = 0;
-    cudaError_t e = mlp_prepare(&sms);
+    MlpDev dev;
+    cudaError_t e = mlp_prepare(&dev);
     if (e != cudaSuccess) return e;
     const int K = Kh + kMlpN;
-    const MlpPlan plan = mlp_plan(M, K, sms);
+    const MlpPlan plan = mlp_plan(M, K, dev);
     if (plan.full > 0) {
         CUtensorMap tmA, tmA2, tmB, tmW2, tmW3;
         if (!g_maps.get(&tmA, h, M, Kh, kMlpBM) || !g_maps.get(&tmA2, f, M, kMlpN, kMlpBM) ||
@@ -1101,7 +1130,7 @@ cudaError_t launch_scorer_deep(const void *h, int Kh, const void *f, int M, cons
         *why = "cuTensorMapEncodeTiled failed";
         return cudaErrorInvalidValue;
     }
-    const bool pair = plan.rest * kTailCluster > sms;
+    const bool pair = plan.rest > dev.c4;   // (more clusters of 4 than fit one CTA per SM)
     TailParams p;
     p.M = M;
     p.tile0 = plan.full;

@@ -1,6 +1,6 @@
 """The scorers where their launch changes shape: batches just inside and past
-one CTA per SM (38 tiles of 128 rows on 152 SMs) and of several waves with a
-ragged last tile, and K whose slices of 64 do not divide by four (and under
+one CTA per SM (36 tiles of 128 rows as clusters of four on 152 SMs, 76 as
+clusters of two) and of several waves with a ragged last tile, and K whose slices of 64 do not divide by four (and under
 four of them), against fp64.  One layer: fp32 sums of K products in four
 chains are off by 2e-7 at the most (K = 3,520); 1e-6 allowed.  Deep: as derived
 in the scorer's own test (bf16 activations)."""
@@ -16,7 +16,7 @@ def _gelu(z):
     return 0.5 * z * (1 + torch.erf(z / 2 ** 0.5))
 
 
-@pytest.mark.parametrize("M,K", [(38 * 128, 512), (38 * 128 + 1, 512), (76 * 128 - 5, 448), (20001, 320), (700, 192),
+@pytest.mark.parametrize("M,K", [(36 * 128, 512), (36 * 128 + 1, 512), (38 * 128, 512), (38 * 128 + 1, 512), (76 * 128 - 5, 448), (20001, 320), (700, 192),
                                  (20001, 64), (300, 3520)])
 def test_mlp(sdd, M, K):
     W1, b1, w2, b2 = synth.make_mlp(device="cuda", hidden=K)
@@ -47,7 +47,7 @@ def test_mlp_error_does_not_grow_with_the_batch(sdd, M, K):
         assert float((s - want).norm()) <= 1.1 * float((small - want).norm())
 
 
-@pytest.mark.parametrize("M,Kh", [(38 * 128, 256), (38 * 128 + 1, 256), (12345, 192), (20001, 64), (20001, 704)])
+@pytest.mark.parametrize("M,Kh", [(36 * 128, 256), (37 * 128, 256), (38 * 128, 256), (38 * 128 + 1, 256), (12345, 192), (20001, 64), (20001, 704)])
 def test_deep(sdd, M, Kh):
     w = synth.make_scorer_deep(device="cuda", hidden=Kh)
     W1, b1, W2, b2, W3, b3, w4, b4 = w
@@ -68,7 +68,7 @@ def test_deep(sdd, M, Kh):
 @pytest.mark.parametrize("M", [64 * 128, 12000, 152 * 128, 20001])
 def test_deep_rows_do_not_depend_on_the_batch(sdd, M, Kh):
     """One CTA a tile and the split form sum alike: activations of the first layer and scores of a batch are those of
-    its rows 2,048 at a time, except between 38 and 76 tiles, where two splits add the chains pairwise."""
+    its rows 2,048 at a time, except between 36 and 76 tiles, where two splits add the chains pairwise."""
     w = synth.make_scorer_deep(device="cuda", hidden=Kh)
     h, f = synth.make_hidden(M, device="cuda", seed=5, hidden=Kh), synth.make_features(M, device="cuda")
     act = [torch.empty(n, 256, dtype=torch.bfloat16, device="cuda") for n in (M, M)]
@@ -122,3 +122,32 @@ def test_weights_written_just_before(sdd, M):
         got.append((sdd.scorer_deep(h, f, *w), i))
     for s, i in got:
         assert torch.equal(s, want[i])
+
+
+def _us(fn, n=20):
+    for _ in range(3):
+        fn()
+    ts = []
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda._sleep(1000000)
+        a.record()
+        for _ in range(n):
+            fn()
+        b.record()
+        torch.cuda.synchronize()
+        ts.append(a.elapsed_time(b) * 1e3 / n)
+    return min(ts)
+
+
+@pytest.mark.parametrize("K", [256, 448])
+def test_split_tiles_fit_one_wave(sdd, K):
+    """38 tiles of a short K (clusters of four that do not all fit at once took 1.6 times as long as 39 tiles, which run
+    as clusters of two)."""
+    W1, b1, w2, b2 = synth.make_mlp(device="cuda", hidden=K)
+    b2, us = float(b2), []
+    for tiles in (38, 39):
+        h = synth.make_hidden(tiles * 128, device="cuda", hidden=K)
+        ws, out = sdd.scorer_workspace(tiles * 128, "cuda"), torch.empty(tiles * 128, device="cuda")
+        us.append(_us(lambda: sdd.survival_mlp(h, W1, b1, w2, b2, workspace=ws, out=out)))
+    assert us[0] <= 1.2 * us[1], us
