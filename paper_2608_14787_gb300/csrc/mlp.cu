@@ -47,7 +47,7 @@ constexpr uint32_t kBTileBytes = kMlpN * kMlpBK * 2;    // 32 KiB
 constexpr uint32_t kStageBytes = kATileBytes + kBTileBytes;
 constexpr int kMlpSmem = kMlpStages * kStageBytes + 1024 + 256;   // + alignment slack + barriers
 constexpr uint32_t kTmemCols = 256;
-// A tile's sum over K is taken in up to this many chains (quarters of K), each
+// A tile's sum over K is taken in this many chains (quarters of K), each
 // accumulated by the tensor cores from zero, added in fp32 in their order: a
 // CTA of S splits takes kMlpChains / S of them.  The tensor cores' fp32
 // accumulation loses about in proportion to a chain's length: error of the
@@ -55,7 +55,12 @@ constexpr uint32_t kTmemCols = 256;
 // 0.98e-7; K = 2048: 2.2e-7, 1.1e-7, 0.66e-7.  Four against one chain cost
 // (S = 1) 28.0 against 27.4 us at 12,000 rows, 33.1 / 32.9 at 16,384, 35.4 /
 // 35.4 at 19,456, and two against one (S = 2) 20.4 / 20.1 at 8,192.
+// Under eight slices of K two chains or one, as measured there (K = 448: one
+// chain 0.64e-7 and 10.0 us at 19,456 rows, four 0.48e-7 and 11.1).
 constexpr int kMlpChains = 4;
+__host__ __device__ constexpr int mlp_chains(int slices) {
+    return slices >= 2 * kMlpChains ? kMlpChains : (slices >= kMlpChains && slices % 2 == 0) ? 2 : 1;
+}
 
 struct MlpParams {
     int32_t M, K;
@@ -329,7 +334,7 @@ __global__ void __launch_bounds__(mlp_threads(S), 1) mlp_kernel(const __grid_con
     const int slices = p.K / kMlpBK;
     const int kt0 = static_cast<int>(rank) * slices / S;                // K slices of this CTA
     const int nk = (static_cast<int>(rank) + 1) * slices / S - kt0;
-    const int C = min(kMlpChains / S, nk);
+    const int C = max(mlp_chains(slices) / S, 1);
 
     if (tid == 0) {
         for (int i = 0; i < 2 * kMlpStages + kMlpChains; ++i) mbar_init(&full[i], 1);
@@ -767,7 +772,7 @@ __global__ void __launch_bounds__(kMlpThreadsChains, 1) mlp_deep_kernel(const __
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
-    const int nk = p.K / kMlpBK, C = min(kMlpChains, nk);
+    const int nk = p.K / kMlpBK, C = mlp_chains(nk);
     mlp_mainloop<kMlpThreads / 32>(smem, full, empty, done, drained, &tmA, &tmA2, &tmB, p.Ka, m0, 0, nk, C, tmem, &s_abort);
     __syncwarp();
 
@@ -988,7 +993,9 @@ cudaError_t mlp_prepare(MlpDev *out) {
 // wave again: 13.9 us with S = 4 at 32 tiles of K = 3584, 14.6 at 36, and 25.4 at
 // 37, whose last cluster waits for another; 18.2 with S = 2 there, 22.4 at 76; a
 // full wave with S = 1 35.4).  A larger rest runs unsplit too (it is then part of
-// `full`).  GB300,
+// `full`), and so do, of fewer than eight slices of K, a rest that two splits
+// would take (K = 448, 47 tiles: 9.4 us against 9.9) and one behind whole waves
+// (196 tiles: 18.3 against 20.0).  GB300,
 // one-layer scorer, K = 3584, three inputs in turn, against all tiles split four
 // ways: 8,192 rows 20.3 / 28.9 us, 12,000 28.2 / 43.7, 16,384 33.3 / 58.0,
 // 20,000 44.9 / 71.9, 32,768 64.4 / 111.9.
@@ -999,6 +1006,7 @@ MlpPlan mlp_plan(int M, int K, const MlpDev &dev) {
     const int tiles = (M + kMlpBM - 1) / kMlpBM, nk = K / kMlpBK;
     MlpPlan q{tiles / dev.sms * dev.sms, tiles % dev.sms, 1};
     if (q.rest > 0) q.S = (q.rest <= dev.c4 && nk >= 4) ? 4 : (q.rest <= dev.c2 && nk >= 2) ? 2 : 1;
+    if (nk < 2 * kMlpChains && (q.S == 2 || q.full > 0)) q.S = 1;
     if (q.S == 1) q = MlpPlan{tiles, 0, 1};
     return q;
 }
