@@ -590,7 +590,8 @@ SDD_API sdd_status_t sdd_block_decide(const sdd_block_args *args, sdd_stream_t s
  *           call: the pipelined pass divides the rows among warps
  *           differently from sdd_block_scan.
  * Rounds of more than 1 GiB of logits, whose decide work is a small part of
- * their time, run as sdd_block_scan (in the call that names them as next) and
+ * their time, and rounds of more than 480 MiB whose draws would outlast the
+ * streaming pass (many blocks of few positions) run as sdd_block_scan (in the call that names them as next) and
  * sdd_block_decide (in the call that names them as prev) instead.
  * next and prev must use different workspaces and different output arrays.
  * Results are those of sdd_block on the same args: the same decisions and

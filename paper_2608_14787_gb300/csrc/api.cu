@@ -1158,8 +1158,9 @@ sdd_status_t sdd_block(const sdd_block_args *a, sdd_stream_t stream) {
 }
 
 // A pipelined round's launch parameters: sdd_block's, streamed by warps
-// behind the decide team's when the round is at most kPipeMaxBytes (the same
-// when the round is streamed and when it is decided).
+// behind the decide team's when the round is at most kPipeMaxBytes and its draw
+// work fits beside the pass (the same when the round is streamed and when it is
+// decided).
 static sdd_status_t pipe_params(const sdd_block_args *a, ScanParams &p, bool *empty) {
     SDD_TRY(block_params(a, p, empty));
     if (*empty || p.T * 16 > kPipeMaxBytes) return SDD_OK;
@@ -1168,6 +1169,13 @@ static sdd_status_t pipe_params(const sdd_block_args *a, ScanParams &p, bool *em
     // the decide team beside this round's streaming pass (warps 0 .. warp0-1)
     const int64_t bytes = p.T * 16;
     const bool wide = bytes <= kPipeSmallBytes || bytes > kPipeMidBytes;
+    if (bytes > kPipeMidBytes && p.dec.do_strict && !p.dec.greedy) {
+        const int nb = p.grp[0].nb;
+        int32_t nseg = 1, seg_vec = 0;
+        draw_segments(p.RV, nb, p.ctas, kPipeTeamWide, nseg, seg_vec);
+        const int64_t items = (static_cast<int64_t>(nb) * nseg + p.ctas - 1) / p.ctas;   // of a CTA
+        if (items * seg_vec * (16 / esize(a->dtype)) * kPipeDrawBytes > bytes) return SDD_OK;
+    }
     const int team_warps = (wide ? kPipeTeamWide : kPipeTeam) / 32;
     const int wpc = kWarpsPerCta - team_warps;
     p.W = scan_warps(w.W_max / kWarpsPerCta * wpc, p.T, p.rows, kPipePieces);

@@ -308,6 +308,16 @@ constexpr int kPipeTeam = 64, kPipeTeamWide = 128;
 constexpr int64_t kPipeSmallBytes = int64_t(200) << 20;   // at most: the wide team
 constexpr int64_t kPipeMidBytes = int64_t(480) << 20;     // at most: the narrow team
 constexpr int64_t kPipeMaxBytes = int64_t(1) << 30;       // at most: the wide team; above: two kernels
+// Above kPipeMidBytes a round with a sampling draw goes to the two kernels too
+// when a team's draw work would outlast the pass: the entries of a draw row that
+// a CTA's items weigh (more blocks: fewer segments to each, down to a whole row),
+// times this, above the round's bytes.  GB300, us a round, pipelined / two
+// kernels, by that product over the bytes: 128 x 4 positions of 151,936 fp32 (2.7)
+// 523 / 151; 80 x 16 bf16 (2.4) 308 / 152; 64 x 8 fp32 (1.4) 178 / 130; 64 x 16
+// bf16 (1.5) 141 / 124; 200 x 32 of 32,003 bf16 (2.0) 157 / 153; 200 x 16 of 32,003
+// fp32 (0.95) 150 / 160; 56 x 32 bf16 (0.87) 187 / 188; 48 x 32 bf16 (0.68) 159 /
+// 162; 48 x 16 fp32 (0.66) 146 / 173; 33 x 32 bf16 (0.75) 111 / 115.
+constexpr int64_t kPipeDrawBytes = 12500;
 // Pieces of a row in a pipelined pass at most: the decide team beside it is
 // narrow and bounds a small round, so fewer partials are worth longer pieces
 // (GB300, one 32 x 151,936 bf16 block a round: 8 pieces 16.2 us, 9 16.5, 12

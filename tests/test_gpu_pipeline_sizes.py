@@ -1,6 +1,6 @@
 """The pipelined call at the sizes where its form changes (a decide team of 128
 threads up to 200 MiB of logits and from 480 MiB to 1 GiB, of 64 between, two
-kernels above): chains whose rounds lie on both sides of each line, each
+kernels above, and above 480 MiB where the draws would outlast the pass): chains whose rounds lie on both sides of each line, each
 round's outputs against the same round unpipelined (decisions equal; statistics
 within the rounding that another cut of the rows can make)."""
 import pytest
@@ -37,3 +37,49 @@ def test_sizes(sizes):
         for n in ("q", "maxprob", "entropy"):
             torch.testing.assert_close(getattr(a, n), getattr(b, n), rtol=2e-6, atol=1e-7)
         assert int(a.status.item()) == 0
+
+
+@pytest.mark.parametrize("B,gamma", [(128, 4), (64, 8)])
+def test_many_blocks_of_few_positions(B, gamma):
+    """Rounds whose draws would outlast the streaming pass beside them (whole fp32 draw rows to a team: 3.5 times the two
+    kernels' time) are no slower than the two kernels by more than a tenth, and decide the same; a small round follows."""
+    V = 151936
+    blks = [synth.make_block("c3", device="cuda", B=b, gamma=gamma, dtype=torch.float32, round_=i)
+            for i, b in enumerate((B, B, 3))]
+    rnds = []
+    for i, blk in enumerate(blks):
+        r = sdd.BlockRound(blk.x.shape[0], gamma, V, dtype=torch.float32, ks=(2,))
+        r.set_inputs(blk.z_d, blk.z_t, blk.x, seed=i, round_=i)
+        rnds.append(r)
+    prev = None
+    for r in rnds:
+        sdd.block_pipelined(r, prev)
+        prev = r
+    sdd.block_pipelined(None, prev)
+    got = [{n: getattr(r, n).clone() for n in WHOLE} for r in rnds]
+    for r, g in zip(rnds, got):
+        r.run()
+        assert all(torch.equal(getattr(r, n), g[n]) for n in WHOLE) and int(r.status.item()) == 0
+    state = [0]
+
+    def piped():
+        state[0] ^= 1
+        sdd.block_pipelined(rnds[state[0]], rnds[1 - state[0]])
+
+    def us(fn, n=10):
+        ts = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(1000000)
+            a.record()
+            for _ in range(n):
+                fn()
+            b.record()
+            torch.cuda.synchronize()
+            ts.append(a.elapsed_time(b) * 1e3 / n)
+        return min(ts)
+    sdd.block_pipelined(rnds[0], None)
+    two = us(lambda: rnds[0].run())
+    rnds[0].run()
+    sdd.block_pipelined(rnds[0], None)
+    assert us(piped) <= 1.1 * two
