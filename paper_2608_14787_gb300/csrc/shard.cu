@@ -885,15 +885,21 @@ cudaError_t stream_device(StreamDev &out) {
 
 // The clusters of the streaming form for `rows` rows of a slice, and a CTA's
 // piece slots; 0 where one CTA per row takes the call: slices of under two
-// tiles a row, whose pieces would be mostly their ends, and batches whose
-// clusters' pieces exceed the shared memory (~900 rows a cluster).  GB300, one
+// tiles a row, whose pieces would be mostly their ends; without candidates,
+// rows of under kRowFormVec vectors whose CTAs are all resident at once (GB300,
+// one CTA per row / streaming, 17 rows: 8,000 bf16 entries 4.0 / 7.2 us, 16,000 5.4
+// / 7.0, 24,000 6.8 / 7.0, 38,000 9.6 / 7.0; 1,040 rows 7.7 / 10.1, 10.9 / 12.1, 14.8
+// / 14.8, 21.5 / 18.9; 2,080 rows of 8,000 13.8 / 12.4; 17 rows of 12,000 fp32 entries
+// 5.9 / 6.2); and batches whose clusters' pieces exceed the shared memory (~900 rows a cluster).  GB300, one
 // CTA per row / streaming, bf16 halves with k = 10: 1 x 32 positions of 75,968
 // entries 35.0 / 11.8 us, 8 x 32 41.6 / 24.0, 64 x 64 315 / 207; 16 x 32 of
 // 4,500 entries 18.0 / 15.8, 1 x 32 13.6 / 11.5.
+constexpr int kRowFormVec = 3000;
 int stream_plan(const ShardParams &sp, int64_t rows, const StreamDev &dev, int32_t &slots) {
     slots = 0;
     if (dev.clusters < 1 || rows >= (int64_t(1) << 27)) return 0;
     if (sp.RVs < 2 * kTileVec) return 0;
+    if (sp.kcap == 0 && rows <= static_cast<int64_t>(2 * kShardMinCtas) * dev.clusters && sp.RVs < kRowFormVec) return 0;
     slots = slice_slots(rows, dev.clusters);
     return stream_smem(slots) <= static_cast<size_t>(dev.smem) ? dev.clusters : 0;
 }

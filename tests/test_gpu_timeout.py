@@ -60,8 +60,8 @@ def test_sharded_records_wait_runs_out_and_recover(sdd, polls, k):
     """One warp of the sharded records' streaming form gives up; both CTAs of its cluster still meet at their barrier,
     the call returns with its status, and the next one writes the records that it wrote before."""
     from paper_2608_14787_gb300 import vocab_shard
-    blk = synth.make_block("c3", device="cuda", B=5, gamma=7, V=20_000)
-    r = vocab_shard.ShardRound(5, 7, 20_000, 0, 20_000, ks=(k,) if k else ())
+    blk = synth.make_block("c3", device="cuda", B=5, gamma=7, V=30_000)
+    r = vocab_shard.ShardRound(5, 7, 30_000, 0, 30_000, ks=(k,) if k else ())
     r.set_inputs(blk.z_d, blk.z_t, blk.x)
     want = r.partials().clone()
     torch.cuda.synchronize()
