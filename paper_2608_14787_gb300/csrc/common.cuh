@@ -334,21 +334,29 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 }
 
 // Launch `kernel` behind the previous work of `stream` as a programmatic
-// dependent grid (host side).
+// dependent grid (host side); carveout: the part of an SM's memory preferred as
+// shared memory, in percent (negative: what the most resident CTAs need).
 template <class... Params, class... Args>
-inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                    const Args &...args) {
+inline cudaError_t launch_dependent_carveout(int carveout, void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem,
+                                             cudaStream_t stream, const Args &...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = static_cast<unsigned>(carveout);
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = carveout < 0 ? 1 : 2;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+template <class... Params, class... Args>
+inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                    const Args &...args) {
+    return launch_dependent_carveout(-1, kernel, grid, block, smem, stream, args...);
 }
 
 // ---------------------------------------------------------------------------

@@ -274,6 +274,10 @@ cudaError_t decide_prepare_device() {
     return cudaSuccess;
 }
 
+// The decide kernel's static shared memory and the driver's KiB beside it (7.8
+// KiB), rounded up; the most shared memory of an SM.
+constexpr size_t kDecStaticSmem = 8 << 10, kSmSharedBytes = 228 << 10;
+
 cudaError_t launch_decide(const ScanParams &p, cudaStream_t stream) {
     const int nb = p.grp[0].nb;
     if (nb == 0) return cudaSuccess;
@@ -290,7 +294,18 @@ cudaError_t launch_decide(const ScanParams &p, cudaStream_t stream) {
                                   : feat ? (bf ? decide_kernel<SDD_BF16, true> : decide_kernel<SDD_F32, true>)
                                          : (bf ? decide_kernel<SDD_BF16, false> : decide_kernel<SDD_F32, false>);
     if (team == kDecThreadsWhole) return launch_dependent(kDecideWhole[feat][bf], grid, dim3(team), smem, stream, p);
-    return launch_dependent(k, grid, dim3(kDecThreads), smem, stream, p);
+    // With a device block count a CTA asks for the prefixes of as many segments
+    // as there could be (64 KiB).  The grid is two CTAs an SM (dec_ctas); the
+    // fp32 kernel's registers would let three in, and the shared memory kept for
+    // three left 23 KiB of L1 to the draw, whose threads each read a run of
+    // their own (GB300, 150 of 300 blocks of 1 x 151,936 fp32: 142 us against 43,
+    // L1 hits 16 % against 44).
+    int carveout = -1;
+    if (dev_geom) {
+        const size_t two = 2 * (smem + kDecStaticSmem);
+        carveout = static_cast<int>(std::min<size_t>(100, (100 * two + kSmSharedBytes - 1) / kSmSharedBytes));
+    }
+    return launch_dependent_carveout(carveout, k, grid, dim3(kDecThreads), smem, stream, p);
 }
 
 // The blocks that go to the verifier: K[b] == 0, in ascending order, by one
