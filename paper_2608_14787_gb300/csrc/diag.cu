@@ -18,9 +18,11 @@
 //                       kPermPar blocks, in order by one thread above); it
 //                       writes, for every block, the block whose score it takes.
 // perm_prefix_kernel -- one thread per (repetition, block): the gates of Eq. 3
-//                       on the permuted scores (the schedule's own arithmetic),
-//                       position by position until the local gate fails;
-//                       integer sums per repetition (exact, order-free).
+//                       on the permuted scores, position by position until the
+//                       local gate fails (the schedule's double-floats, added
+//                       one after another where it adds them in a tree: a sum
+//                       within their rounding of its threshold, ~2^-43, may
+//                       fall on the other side); integer sums per repetition (exact, order-free).
 // metrics_kernel     -- one cluster of CTAs per position: fp64 BCE sums, integer
 //                       pair counts.
 #include <atomic>

@@ -300,10 +300,11 @@ __host__ __device__ inline int32_t scan_warps(int64_t W_max, int64_t T, int64_t 
 // streaming warps win.  Above kPipeMaxBytes the decide kernel's fixed tail
 // matters less than sixteen streaming warps.  GB300, us a round of B blocks of
 // 32 positions over V = 151,936 bf16 (19.75 MB each), team of 128 / 64 / the
-// two kernels in turn: B = 4 22.7 / 25.8 / 30.5, 8 33.4 / 37.0 / 42.1, 10 39.4
-// / 40.2 / 47.2, 12 45.3 / 43.8 / 53.0, 16 57.4 / 54.5 / 64.2, 24 81.5 / 77.5 /
-// 88.1, 27 - / 100.2 / -, 28 94.5 / 101.3 / 101.2, 32 107.5 / 117.5 / 112.6, 48 158.6 / 157.7 /
-// 161.8, 56 186.4 / 246.6 / 188.8, 64 211.8 / 254.8 / 212.0, 80 371 / 659 / 262.
+// two kernels in turn (one GPU): B = 4 22.7 / 25.9 / 30.8, 8 33.2 / 37.0 / 42.1,
+// 10 39.2 / 40.7 / 47.5, 11 42.5 / 42.4 / 50.4, 12 45.5 / 44.3 / 53.0, 14 51.5 / 49.2 /
+// 58.6, 16 57.7 / 54.8 / 64.2, 24 82.2 / 78.1 / 88.6, 28 95.5 / 102.3 / 101.4, 32 108.5 /
+// 118.1 / 112.8, 48 159.0 / 157.3 / 161.9, 56 187.4 / 246.3 / 187.7, 64 212.1 / 254.5 /
+// 211.9.
 constexpr int kPipeTeam = 64, kPipeTeamWide = 128;
 constexpr int64_t kPipeSmallBytes = int64_t(200) << 20;   // at most: the wide team
 constexpr int64_t kPipeMidBytes = int64_t(480) << 20;     // at most: the narrow team

@@ -51,8 +51,8 @@ __device__ __noinline__ void pipe_decide(const PipeParams &pp, float *s_pref_all
 }
 
 // The streaming warps' rings, indexed by streaming warp: two stages each, as
-// in the streaming kernel (three measured slower here too: 64.5 against 63.9
-// us per round).
+// in the streaming kernel (three measured slower here too, on a kernel that then
+// took 63.9 us per round: 64.5).
 constexpr int kPipeStages = 2;
 __host__ __device__ constexpr int pipe_rings(int team) { return ring_bytes(kPipeStages, kWarpsPerCta - team / 32); }
 

@@ -34,7 +34,7 @@ int scan_max_ctas_per_sm() {
     return n;
 }
 
-// Opt both instantiations in to their dynamic shared memory on the current device.
+// Opt every instantiation in to its dynamic shared memory on the current device.
 cudaError_t scan_prepare_device() {
     for (const auto &row : kScanKernels)
         for (auto k : row) {
