@@ -35,9 +35,6 @@ __device__ __forceinline__ float clamp_ref() { return ceilf(clamp_floor() * kLog
 __device__ __forceinline__ float pow2f_int(float k) {
     return (k < -126.f) ? 0.f : __int_as_float((127 + static_cast<int>(k)) << 23);
 }
-__device__ __forceinline__ double pow2d_int(float k) {
-    return (k < -1022.f) ? 0.0 : __longlong_as_double(static_cast<long long>(1023 + static_cast<int>(k)) << 52);
-}
 
 // ---------------------------------------------------------------------------
 // Records exchanged through the workspace
